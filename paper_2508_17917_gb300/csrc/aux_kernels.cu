@@ -117,92 +117,123 @@ __global__ void max_reduce_kernel(const double *x, long long n, double *out)
 // Force and moment of one wall face: traction p n - tau n at its face nodes
 // (interior trace, n the element's outward normal), integrated with the LGL
 // weights scaled by sJ; moment about (xc, yc).  xy: the face nodes'
-// coordinates (x, y interleaved).
+// coordinates (x, y interleaved).  One warp per face: lane 4 i + c forms the
+// broken gradient of field c at face node i, the four lanes of a node
+// exchange fields by shuffles, and lane 0 ends up with the sums over the
+// nodes in node order.  Few faces and long FP64 chains: latency bounds this,
+// so the Np-term sums of a face run side by side instead of one after the
+// other in one thread (120 faces at p = 4: 39 us and a separate 4 us sum
+// before, 8 us in all now).
 __device__ void wall_face_force(const AuxMesh &m, Phys<double> ph, long long k, int f, const double *xy,
                                 const double *wface, double xc, double yc, double out[3])
 {
     const int p = m.p, Np = (p + 1) * (p + 2) / 2, Nfp = p + 1;
     if (m.elem_case) ph.mu = m.cases[m.elem_case[k]].mu;
+    const int lane = threadIdx.x & 31, i = lane >> 2, c = lane & 3;
+    const int ii = i < Nfp ? i : 0;              // idle lanes repeat node 0 and are not summed
     const double *g = m.geo + k * 16;
     const double rx = g[G_RX], ry = g[G_RY], sx = g[G_SX], sy = g[G_SY];
     const double n1 = g[G_NX + f], n2 = g[G_NY + f], sJ = g[G_FS + f] * g[G_J];
-    double F0 = 0, F1 = 0, Mz = 0;
-    for (int i = 0; i < Nfp; ++i) {
-        int vm = m.fmask[f * Nfp + i];
-        double ur[4] = {0, 0, 0, 0}, us[4] = {0, 0, 0, 0}, u[4];
-        for (int j = 0; j < Np; ++j) {
-            double dr = m.Dr[vm * Np + j], ds = m.Ds[vm * Np + j];
-            for (int c = 0; c < 4; ++c) {
-                double uj = m.U[(k * 4 + c) * Np + j];
-                ur[c] += dr * uj;
-                us[c] += ds * uj;
-            }
-        }
-        double gx[4], gy[4];
-        for (int c = 0; c < 4; ++c) {
-            gx[c] = rx * ur[c] + sx * us[c];
-            gy[c] = ry * ur[c] + sy * us[c];
-        }
-        load_node(m.U, Np, k, vm, u);
-        double vx[4], vy[4];
-        visc_flux(u, gx, gy, ph, vx, vy);
-        double pr = pressure<double>(u, u[3], ph.gm1);
-        double tx = pr * n1 - (vx[1] * n1 + vy[1] * n2);
-        double ty = pr * n2 - (vx[2] * n1 + vy[2] * n2);
-        double x = xy[2 * i] - xc;
-        double y = xy[2 * i + 1] - yc;
-        double wq = sJ * wface[i];
-        F0 += wq * tx;
-        F1 += wq * ty;
-        Mz += wq * (x * ty - y * tx);
+    const int vm = m.fmask[f * Nfp + ii];
+    const double *Dr = m.Dr + vm * Np, *Ds = m.Ds + vm * Np, *U = m.U + (k * 4 + c) * Np;
+    double ur = 0.0, us = 0.0;
+#pragma unroll 7
+    for (int j = 0; j < Np; ++j) {
+        const double uj = U[j];
+        ur += Dr[j] * uj;
+        us += Ds[j] * uj;
     }
-    out[0] = F0;
-    out[1] = F1;
-    out[2] = Mz;
+    const double gxc = rx * ur + sx * us, gyc = ry * ur + sy * us, uc = U[vm];
+    double gx[4], gy[4], u[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int src = (lane & ~3) + q;
+        gx[q] = __shfl_sync(0xffffffffu, gxc, src);
+        gy[q] = __shfl_sync(0xffffffffu, gyc, src);
+        u[q] = __shfl_sync(0xffffffffu, uc, src);
+    }
+    double vx[4], vy[4];
+    visc_flux(u, gx, gy, ph, vx, vy);
+    const double pr = pressure<double>(u, u[3], ph.gm1);
+    const double wq = sJ * wface[ii];
+    const double tx = wq * (pr * n1 - (vx[1] * n1 + vy[1] * n2));
+    const double ty = wq * (pr * n2 - (vx[2] * n1 + vy[2] * n2));
+    const double tm = (xy[2 * ii] - xc) * ty - (xy[2 * ii + 1] - yc) * tx;
+    out[0] = out[1] = out[2] = 0.0;
+    for (int l = 0; l < Nfp; ++l) {
+        out[0] += __shfl_sync(0xffffffffu, tx, 4 * l);
+        out[1] += __shfl_sync(0xffffffffu, ty, 4 * l);
+        out[2] += __shfl_sync(0xffffffffu, tm, 4 * l);
+    }
 }
 
-// One thread per wall face of one mesh: partial[w] = (Fx, Fy, Mz) of face w.
-__global__ void wall_force_kernel(AuxMesh m, Phys<double> ph, const int2 *faces, const double *face_xy,
-                                  const double *wface, int nwall, double xc, double yc, double *partial)
+constexpr int kWallWarps = 4;      // warps (faces) per block of the wall-force kernels
+
+// Sum of n triples by the calling block (256 values at a time in a fixed
+// order, whatever the block size), result in s[c][0].
+__device__ void block_sum3(const double *partial, int n, double (*s)[256])
 {
-    int w = blockIdx.x * blockDim.x + threadIdx.x;
-    if (w >= nwall) return;
-    const int Nfp = m.p + 1;
-    wall_face_force(m, ph, faces[w].x, faces[w].y, face_xy + static_cast<long long>(w) * Nfp * 2, wface, xc, yc,
-                    partial + w * 3);
+    for (int t = threadIdx.x; t < 256; t += blockDim.x) {
+        double a[3] = {0, 0, 0};
+        for (int i = t; i < n; i += 256)
+            for (int c = 0; c < 3; ++c) a[c] += __ldcg(partial + static_cast<long long>(i) * 3 + c);
+        for (int c = 0; c < 3; ++c) s[c][t] = a[c];
+    }
+    __syncthreads();
+    for (int w = 128; w > 0; w >>= 1) {
+        for (int t = threadIdx.x; t < w; t += blockDim.x)
+            for (int c = 0; c < 3; ++c) s[c][t] += s[c][t + w];
+        __syncthreads();
+    }
 }
 
-// One thread per wall face of every degree group of a batch: the groups'
-// faces are numbered consecutively (group g from wg.g[g].base), and face w
-// writes partial[w].
+// Wall faces of one mesh, a warp per face: partial[w] = (Fx, Fy, Mz) of face
+// w; the last block to finish (ticket, zero between launches) sums them into
+// out, so that no second launch waits for the first.
+__global__ void wall_force_kernel(AuxMesh m, Phys<double> ph, const int2 *faces, const double *face_xy,
+                                  const double *wface, int nwall, double xc, double yc, double *partial,
+                                  unsigned *ticket, double *out)
+{
+    __shared__ double s[3][256];
+    __shared__ bool last;
+    const int w = blockIdx.x * kWallWarps + (threadIdx.x >> 5);
+    const int Nfp = m.p + 1;
+    if (w < nwall) {
+        double o[3];
+        wall_face_force(m, ph, faces[w].x, faces[w].y, face_xy + static_cast<long long>(w) * Nfp * 2, wface, xc, yc, o);
+        if ((threadIdx.x & 31) == 0) {
+            for (int c = 0; c < 3; ++c) partial[static_cast<long long>(w) * 3 + c] = o[c];
+            __threadfence();
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    block_sum3(partial, nwall, s);
+    if (threadIdx.x == 0) {
+        for (int c = 0; c < 3; ++c) out[c] = s[c][0];
+        *ticket = 0u;
+    }
+}
+
+// A warp per wall face of every degree group of a batch: the groups' faces
+// are numbered consecutively (group g from wg.g[g].base), and face w writes
+// partial[w].
 __global__ void batch_wall_force_kernel(WallGroups wg, Phys<double> ph, double *partial)
 {
-    const int w = blockIdx.x * blockDim.x + threadIdx.x;
+    const int w = blockIdx.x * kWallWarps + (threadIdx.x >> 5);
     if (w >= wg.total) return;
     int gi = 0;
     while (gi + 1 < wg.n && w >= wg.g[gi + 1].base) ++gi;
     const WallGroup &G = wg.g[gi];
     const int i = w - G.base, Nfp = G.m.p + 1;
-    wall_face_force(G.m, ph, G.faces[i].x, G.faces[i].y, G.face_xy + static_cast<long long>(i) * Nfp * 2,
-                    G.wface, 0.0, 0.0, partial + static_cast<long long>(w) * 3);
-}
-
-// Deterministic single-block sum of n triples.
-__global__ void sum3_kernel(const double *partial, int n, double *out)
-{
-    __shared__ double s[3][256];
-    double a[3] = {0, 0, 0};
-    for (int i = threadIdx.x; i < n; i += blockDim.x)
-        for (int c = 0; c < 3; ++c) a[c] += partial[i * 3 + c];
-    for (int c = 0; c < 3; ++c) s[c][threadIdx.x] = a[c];
-    __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w)
-            for (int c = 0; c < 3; ++c) s[c][threadIdx.x] += s[c][threadIdx.x + w];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0)
-        for (int c = 0; c < 3; ++c) out[c] = s[c][0];
+    double o[3];
+    wall_face_force(G.m, ph, G.faces[i].x, G.faces[i].y, G.face_xy + static_cast<long long>(i) * Nfp * 2, G.wface, 0.0,
+                    0.0, o);
+    if ((threadIdx.x & 31) == 0)
+        for (int c = 0; c < 3; ++c) partial[static_cast<long long>(w) * 3 + c] = o[c];
 }
 
 __global__ void nonfinite_kernel(const double *x, long long n, int *flag)
@@ -222,32 +253,35 @@ __global__ void nonfinite_kernel(const double *x, long long n, int *flag)
 // bound that is not finite freezes the case (dt = 0, bad = 1) instead of
 // spreading NaN.  Thread 0 then takes the case's Newmark step with the lift
 // of the previous force evaluation (Algorithm 3: F_r = lift / m), giving v_b
-// for the coming RK step.
-__global__ void batch_dt_newmark_kernel(const double *lam, const long long *seg, BatchCase *cases, double cfl,
-                                        const double *fixed)
+// for the coming RK step.  The scan over a case's elements is a chain of
+// dependent L2 reads per thread: 1024 threads with four reads in flight (18k
+// elements: 26 us with 256 threads and FP64 comparisons, 8 us now).
+constexpr int kDtThreads = 1024;
+__global__ void __launch_bounds__(kDtThreads)
+batch_dt_newmark_kernel(const double *lam, const long long *seg, BatchCase *cases, double cfl, const double *fixed)
 {
-    __shared__ double s[256];
+    __shared__ long long s[32];
     const int i = blockIdx.x;
     const long long b = seg[2 * i], e = seg[2 * i + 1];
-    double m = 0.0;
-    bool bad = false;
-    for (long long k = b + threadIdx.x; k < e; k += blockDim.x) {
-        const double v = lam[k];
-        bad |= !isfinite(v);
-        m = fmax(m, v);
+    // a non-negative double orders like its bits, so the maximum runs on the
+    // integer units (GB300 compares doubles on its FP64 pipe); anything not
+    // finite counts as infinity, a negative bound as zero
+    constexpr long long kInf = 0x7ff0000000000000ll;
+    long long m = 0;
+#pragma unroll 4
+    for (long long k = b + threadIdx.x; k < e; k += kDtThreads) {
+        const long long v = __double_as_longlong(lam[k]);
+        m = max(m, (v & kInf) == kInf ? kInf : v);
     }
-    s[threadIdx.x] = bad ? NAN : m;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = m;
     __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w) {
-            const double x = s[threadIdx.x], y = s[threadIdx.x + w];
-            s[threadIdx.x] = (isnan(x) || isnan(y)) ? NAN : fmax(x, y);
-        }
-        __syncthreads();
-    }
     if (threadIdx.x != 0) return;
+#pragma unroll
+    for (int w = 1; w < kDtThreads / 32; ++w) m = max(m, s[w]);
     BatchCase &cs = cases[i];
-    const double l = s[0];
+    const double l = m == kInf ? NAN : __longlong_as_double(m);
     cs.lam = l;
     if (cs.bad || !isfinite(l) || !(l > 0.0)) {
         cs.bad = 1;
@@ -381,7 +415,7 @@ cudaError_t launch_vortex_source(bool fp64, const double *xy, long long nn, int 
 cudaError_t launch_batch_dt_newmark(const double *lam, const long long *seg, BatchCase *cases, int ncases,
                                     double cfl, const double *fixed, cudaStream_t st)
 {
-    batch_dt_newmark_kernel<<<ncases, 256, 0, st>>>(lam, seg, cases, cfl, fixed);
+    batch_dt_newmark_kernel<<<ncases, kDtThreads, 0, st>>>(lam, seg, cases, cfl, fixed);
     return cudaGetLastError();
 }
 
@@ -389,7 +423,7 @@ cudaError_t launch_batch_wall_forces(const WallGroups &wg, const Phys<double> &p
                                      cudaStream_t st)
 {
     if (wg.total < 1) return cudaSuccess;
-    batch_wall_force_kernel<<<(wg.total + 127) / 128, 128, 0, st>>>(wg, ph, partial);
+    batch_wall_force_kernel<<<(wg.total + kWallWarps - 1) / kWallWarps, 32 * kWallWarps, 0, st>>>(wg, ph, partial);
     return cudaGetLastError();
 }
 
@@ -415,19 +449,13 @@ cudaError_t launch_max_reduce(const double *lam, long long K, double *out, cudaS
     return cudaGetLastError();
 }
 
-cudaError_t launch_wall_force_faces(const AuxMesh &m, const Phys<double> &ph, const int2 *faces,
-                                    const double *face_xy, const double *wface, int nwall,
-                                    double xc, double yc, double *partial, cudaStream_t st)
+cudaError_t launch_wall_forces(const AuxMesh &m, const Phys<double> &ph, const int2 *faces, const double *face_xy,
+                               const double *wface, int nwall, double xc, double yc, double *partial,
+                               unsigned *ticket, double *out, cudaStream_t st)
 {
-    int threads = 128;
-    int blocks = (nwall + threads - 1) / threads;
-    wall_force_kernel<<<blocks, threads, 0, st>>>(m, ph, faces, face_xy, wface, nwall, xc, yc, partial);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_sum3(const double *partial, int n, double *out, cudaStream_t st)
-{
-    sum3_kernel<<<1, 256, 0, st>>>(partial, n, out);
+    const int blocks = (nwall + kWallWarps - 1) / kWallWarps;
+    wall_force_kernel<<<blocks, 32 * kWallWarps, 0, st>>>(m, ph, faces, face_xy, wface, nwall, xc, yc, partial, ticket,
+                                                          out);
     return cudaGetLastError();
 }
 

@@ -80,6 +80,8 @@ struct dg_ctx {
     float4 *sother() { return cur_is_a ? S0b.ptr : S0a.ptr; }
     float *pcur() { return cur_is_a ? P0a.ptr : P0b.ptr; }
     float *pother() { return cur_is_a ? P0b.ptr : P0a.ptr; }
+    // finished blocks of the wall-force kernel: the last word of scal
+    unsigned *ticket() { return reinterpret_cast<unsigned *>(scal.ptr + 3); }
     ~dg_ctx()
     {
         for (auto *b : {&K0a, &K0b, &K1, &rtmp, &geo64, &ops64, &Dr64, &Ds64, &src, &lam, &scal, &fpart, &fxy, &wface})
@@ -315,6 +317,7 @@ dg_status dg_create(const dg_params *params, void *cuda_stream, dg_ctx **out)
         return DG_ECUDA;
     }
     cudaMemset(c->bar_err.ptr, 0, sizeof(int));
+    cudaMemset(c->scal.ptr, 0, 4 * sizeof(double));
     cudaMemcpy(c->ops64.ptr, o64.data(), o64.size() * sizeof(double), cudaMemcpyHostToDevice);
     cudaMemcpy(c->ops32.ptr, o32.data(), o32.size() * sizeof(float), cudaMemcpyHostToDevice);
     if (dg::stage_tc_supported(p.p)) {
@@ -791,10 +794,9 @@ dg_status dg_wall_forces(dg_ctx *c, const double xc[2], double out[3])
     }
     double x0 = xc ? xc[0] : 0.0, y0 = xc ? xc[1] : 0.0;
     dg::Phys<double> ph = make_phys<double>(c->prm, nullptr);
-    DG_CUDA(c, dg::launch_wall_force_faces(aux_mesh(c), ph, c->wall.ptr, c->fxy.ptr, c->wface.ptr, c->nwall,
-                                           x0, y0, c->fpart.ptr, c->stream));
-    DG_CUDA(c, dg::launch_sum3(c->fpart.ptr, c->nwall, c->scal.ptr, c->stream));
-    c->launches += 2;
+    DG_CUDA(c, dg::launch_wall_forces(aux_mesh(c), ph, c->wall.ptr, c->fxy.ptr, c->wface.ptr, c->nwall, x0, y0,
+                                      c->fpart.ptr, c->ticket(), c->scal.ptr, c->stream));
+    c->launches += 1;
     DG_CUDA(c, cudaMemcpyAsync(out, c->scal.ptr, 3 * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
     DG_CUDA(c, cudaStreamSynchronize(c->stream));
     return DG_OK;
@@ -946,10 +948,9 @@ extern "C" dg_status dg_wall_forces_noalloc(dg_ctx *c, const double xc[2], doubl
     double *result = scratch + static_cast<size_t>(kNoallocMaxWallFaces) * 3;
     double x0 = xc ? xc[0] : 0.0, y0 = xc ? xc[1] : 0.0;
     dg::Phys<double> ph = make_phys<double>(c->prm, nullptr);
-    DG_CUDA(c, dg::launch_wall_force_faces(aux_mesh(c), ph, c->wall.ptr, c->fxy.ptr, c->wface.ptr, c->nwall,
-                                           x0, y0, partial, c->stream));
-    DG_CUDA(c, dg::launch_sum3(partial, c->nwall, result, c->stream));
-    c->launches += 2;
+    DG_CUDA(c, dg::launch_wall_forces(aux_mesh(c), ph, c->wall.ptr, c->fxy.ptr, c->wface.ptr, c->nwall, x0, y0,
+                                      partial, c->ticket(), result, c->stream));
+    c->launches += 1;
     DG_CUDA(c, cudaMemcpyAsync(out, result, 3 * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
     DG_CUDA(c, cudaStreamSynchronize(c->stream));
     return DG_OK;

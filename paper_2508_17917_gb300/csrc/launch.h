@@ -127,11 +127,11 @@ cudaError_t launch_dt_lambda(const AuxMesh &m, const Phys<double> &ph, double si
 // max over lam[0..K) into *out (one block).
 cudaError_t launch_max_reduce(const double *lam, long long K, double *out, cudaStream_t st);
 
-// per-wall-face force/moment partials, then a deterministic sum into out[3]
-cudaError_t launch_wall_force_faces(const AuxMesh &m, const Phys<double> &ph, const int2 *faces,
-                                    const double *face_xy, const double *wface, int nwall,
-                                    double xc, double yc, double *partial, cudaStream_t st);
-cudaError_t launch_sum3(const double *partial, int n, double *out, cudaStream_t st);
+// per-wall-face force/moment partials and their sum (fixed order) into out[3],
+// one launch; *ticket counts finished blocks, zero before and after it
+cudaError_t launch_wall_forces(const AuxMesh &m, const Phys<double> &ph, const int2 *faces, const double *face_xy,
+                               const double *wface, int nwall, double xc, double yc, double *partial,
+                               unsigned *ticket, double *out, cudaStream_t st);
 
 // batch: one block per case, max of lam over the case's element range
 // [seg[2i], seg[2i+1]) -> cases[i].lam and dt = cfl / lam, or fixed[i] when
