@@ -1,7 +1,8 @@
 // aux_kernels.cu -- time step, wall forces and finiteness kernels (FP64).
 #include <math.h>
 
-#include "dg_stage.cuh"
+#include "dg_dt.cuh"
+#include "f64math.cuh"
 #include "launch.h"
 #include "rigid.h"
 
@@ -14,7 +15,8 @@ __device__ __forceinline__ void load_node(const double *U, int Np, long long k, 
     for (int c = 0; c < 4; ++c) u[c] = U[(k * 4 + c) * Np + i];
 }
 
-// One thread per element: Lambda_K of Eq. rayleigh_bound,
+// The FP64 pass of the time-step bound (dg_dt.cuh): Lambda_K of Eq.
+// rayleigh_bound,
 //   Lambda_K = 3/2 C_inv,2(K) G_K + (d+1) C_inv,K (3 sigma_K + beta_K) + beta'_K,
 // with C_inv,2 = p^4 / rho_K^2 (rho_K the inradius 2|K| / perimeter); G_K the
 // largest diffusivity of the system, max(4/3, gamma/Pr) mu / rho, over the
@@ -22,96 +24,124 @@ __device__ __forceinline__ void load_node(const double *U, int Np, long long k, 
 // N G N^T, which does not depend on the normal); sigma_K the largest penalty
 // sigma_e of Eq. penalty_final over the faces of K and C_inv,K the largest
 // C_inv; beta_K = max over nodes of |b_ns|_2, (b_ns)_j = |v_j - v_w,j| + c
-// (Eq. cfl_general), beta'_K = 0.
-__global__ void dt_lambda_kernel(AuxMesh m, Phys<double> ph, double sig_fac, double *lam)
+// (Eq. cfl_general), beta'_K = 0 -- on the elements whose screened value is
+// within the margin of the largest.  A block looks through every gridDim-th
+// element, so that neighbours in the numbering (a ring of equal elements)
+// are spread over the blocks, and works on its candidates eight at a time, a
+// thread per face node and then per node.  The last block to finish writes
+// the maximum and clears the words for the next call.
+constexpr int kDtTile = 8;
+__global__ void __launch_bounds__(128)
+dt_confirm_kernel(AuxMesh m, Phys<double> ph, double sig_fac, const float *lamS, unsigned *words, double *out)
 {
-    long long k = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x;
-    if (k >= m.K) return;
-    if (m.elem_case) {            // batch: the element's case sets mu and v_b
-        const BatchCase &cs = m.cases[m.elem_case[k]];
-        ph.mu = cs.mu;
-        ph.vw2 = cs.vb;
+    __shared__ int list[128];
+    __shared__ int n, isbad;
+    __shared__ unsigned long long best;
+    __shared__ double sG[kDtTile * 21], sR[kDtTile * 21], sB[kDtTile * 28];
+    const int p = m.p, Np = (p + 1) * (p + 2) / 2, Nfp = p + 1, NF = 3 * Nfp, tid = threadIdx.x;
+    const float thr = __uint_as_float(words[0]) * kDtMargin;
+    const double pp = 0.5 * (p + 1.0) * (p + 2.0);
+    if (tid == 0) {
+        best = 0ull;
+        isbad = 0;
     }
-    const int p = m.p, Np = (p + 1) * (p + 2) / 2, Nfp = p + 1;
-    const double *g = m.geo + k * 16;
-    const int4 cn = m.conn[k];
-    double GK = 0, sigK = 0, ciK = 0, perim = 0;
-    const double pp = (p + 1.0) * (p + 2.0);
-    const double gdiff = fmax(4.0 / 3.0, ph.gPr);
-    for (int f = 0; f < 3; ++f) {
-        long long nb = (f == 0) ? cn.x : (f == 1 ? cn.y : cn.z);
-        int f2 = (cn.w >> (2 * f)) & 3;
-        int bt = (cn.w >> (8 + 2 * f)) & 3;
-        double n1 = g[G_NX + f], n2 = g[G_NY + f], fs = g[G_FS + f];
-        double gbar = 0, rmin = INFINITY;
-        for (int i = 0; i < Nfp; ++i) {
-            int vm = m.fmask[f * Nfp + i];
-            double u[4];
-            load_node(m.U, Np, k, vm, u);
-            double a = penalty_norm(u[0], u[1] / u[0], u[2] / u[0], u[3] / u[0], n1, n2, ph);
-            double b;
-            rmin = fmin(rmin, u[0]);
-            if (bt == BCT_INTERIOR) {
-                double w[4];
-                load_node(m.U, Np, nb, m.fmask[f2 * Nfp + (Nfp - 1 - i)], w);
-                b = penalty_norm(w[0], w[1] / w[0], w[2] / w[0], w[3] / w[0], n1, n2, ph);
-                rmin = fmin(rmin, w[0]);
-            } else if (bt == BCT_FARFIELD) {
-                const double *w = ph.Uinf;
-                b = penalty_norm(w[0], w[1] / w[0], w[2] / w[0], w[3] / w[0], n1, n2, ph);
-                rmin = fmin(rmin, w[0]);
-            } else {   // wall ghost: the interior density
-                double pw = pressure<double>(u, u[3], ph.gm1);
-                double eb = (pw / ph.gm1 + 0.5 * u[0] * (ph.vw1 * ph.vw1 + ph.vw2 * ph.vw2)) / u[0];
-                b = penalty_norm(u[0], ph.vw1, ph.vw2, eb, n1, n2, ph);
-            }
-            gbar = fmax(gbar, fmax(a, b));
-        }
-        double ci = pp * fs * 0.5;
-        double cmax = ci;
-        if (bt == BCT_INTERIOR) cmax = fmax(ci, pp * m.geo[nb * 16 + G_FS + f2] * 0.5);
-        double sig = sig_fac * gbar * cmax;
-        GK = fmax(GK, gdiff * ph.mu / rmin);
-        sigK = fmax(sigK, sig);
-        ciK = fmax(ciK, ci);
-        perim += 2.0 * fs * g[G_J];     // |e| = 2 sJ = 2 Fscale J
-    }
-    double area = 2.0 * g[G_J];
-    double rhoK = 2.0 * area / perim;
-    double cinv2 = double(p) * p * p * p / (rhoK * rhoK);
-    double beta = 0;
-    for (int i = 0; i < Np; ++i) {
-        double u[4];
-        load_node(m.U, Np, k, i, u);
-        double pr = pressure<double>(u, u[3], ph.gm1);
-        double c = sqrt(ph.gamma * pr / u[0]);
-        double b1 = fabs(u[1] / u[0] - ph.vw1) + c, b2 = fabs(u[2] / u[0] - ph.vw2) + c;
-        beta = fmax(beta, sqrt(b1 * b1 + b2 * b2));
-    }
-    lam[k] = 1.5 * cinv2 * GK + 3.0 * ciK * (3.0 * sigK + beta);
-}
-
-// Single-block maximum; non-finite entries propagate as NaN.
-__global__ void max_reduce_kernel(const double *x, long long n, double *out)
-{
-    __shared__ double s[1024];
-    double m = 0.0;
-    bool bad = false;
-    for (long long i = threadIdx.x; i < n; i += blockDim.x) {
-        double v = x[i];
-        if (!isfinite(v)) bad = true;
-        m = fmax(m, v);
-    }
-    s[threadIdx.x] = bad ? NAN : m;
-    __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w) {
-            double a = s[threadIdx.x], b = s[threadIdx.x + w];
-            s[threadIdx.x] = (isnan(a) || isnan(b)) ? NAN : fmax(a, b);
-        }
+    const long long G = gridDim.x;
+    for (long long c0 = 0; c0 * G < m.K; c0 += 128) {
         __syncthreads();
+        if (tid == 0) n = 0;
+        __syncthreads();
+        const long long kc = (c0 + tid) * G + blockIdx.x;
+        if (kc < m.K && lamS[kc] >= thr) list[atomicAdd(&n, 1)] = static_cast<int>(kc);
+        __syncthreads();
+        for (int t0 = 0; t0 < n; t0 += kDtTile) {
+            const int nc = min(kDtTile, n - t0);
+            for (int it = tid; it < nc * NF; it += 128) {
+                const int q = it / NF, s = it - q * NF, f = s / Nfp, i = s - f * Nfp;
+                const long long k = list[t0 + q];
+                const int4 cn = m.conn[k];
+                const int f2 = (cn.w >> (2 * f)) & 3, bt = (cn.w >> (8 + 2 * f)) & 3;
+                const double n1 = m.geo[k * 16 + G_NX + f], n2 = m.geo[k * 16 + G_NY + f];
+                double u[4], w[4];
+                load_node(m.U, Np, k, m.fmask[s], u);
+                const double ir = rcp64(u[0]);
+                const double a = penalty_norm64(ir, u[1] * ir, u[2] * ir, u[3] * ir, n1, n2, ph);
+                double b, rmin = u[0];
+                if (bt == BCT_WALL) {             // wall ghost: the interior density and pressure
+                    const double pw = pressure<double>(u, u[3], ph.gm1);
+                    const double eb = (pw / ph.gm1 + 0.5 * u[0] * (ph.vw1 * ph.vw1 + ph.vw2 * ph.vw2)) * ir;
+                    b = penalty_norm64(ir, ph.vw1, ph.vw2, eb, n1, n2, ph);
+                } else {
+                    if (bt == BCT_INTERIOR) {
+                        const long long nb = (f == 0) ? cn.x : (f == 1 ? cn.y : cn.z);
+                        load_node(m.U, Np, nb, m.fmask[f2 * Nfp + (Nfp - 1 - i)], w);
+                    } else {
+                        for (int c = 0; c < 4; ++c) w[c] = ph.Uinf[c];
+                    }
+                    const double iw = rcp64(w[0]);
+                    b = penalty_norm64(iw, w[1] * iw, w[2] * iw, w[3] * iw, n1, n2, ph);
+                    rmin = fmin(rmin, w[0]);
+                }
+                sG[it] = fmax(a, b);
+                sR[it] = rmin;
+            }
+            for (int it = tid; it < nc * Np; it += 128) {
+                const long long k = list[t0 + it / Np];
+                double u[4];
+                load_node(m.U, Np, k, it - (it / Np) * Np, u);
+                const double ir = rcp64(u[0]), v1 = u[1] * ir, v2 = u[2] * ir;
+                const double pr = ph.gm1 * (u[3] - 0.5 * (u[1] * v1 + u[2] * v2));
+                const double c = sqrt64(ph.gamma * pr * ir);
+                const double b1 = fabs(v1 - ph.vw1) + c, b2 = fabs(v2 - ph.vw2) + c;
+                sB[it] = sqrt64(b1 * b1 + b2 * b2);
+            }
+            __syncthreads();
+            if (tid < nc) {
+                const long long k = list[t0 + tid];
+                const double *g = m.geo + k * 16;
+                const int4 cn = m.conn[k];
+                const double gdiff = fmax(4.0 / 3.0, ph.gPr);
+                double GK = 0, sigK = 0, ciK = 0, perim = 0, beta = 0;
+                for (int f = 0; f < 3; ++f) {
+                    double gbar = 0, rmin = INFINITY;
+                    for (int i = 0; i < Nfp; ++i) {
+                        gbar = fmax(gbar, sG[tid * NF + f * Nfp + i]);
+                        rmin = fmin(rmin, sR[tid * NF + f * Nfp + i]);
+                    }
+                    const double fs = g[G_FS + f], ci = pp * fs;
+                    double cmax = ci;
+                    if (((cn.w >> (8 + 2 * f)) & 3) == BCT_INTERIOR) {
+                        const long long nb = (f == 0) ? cn.x : (f == 1 ? cn.y : cn.z);
+                        cmax = fmax(ci, pp * m.geo[nb * 16 + G_FS + ((cn.w >> (2 * f)) & 3)]);
+                    }
+                    GK = fmax(GK, gdiff * ph.mu / rmin);
+                    sigK = fmax(sigK, sig_fac * gbar * cmax);
+                    ciK = fmax(ciK, ci);
+                    perim += 2.0 * fs * g[G_J];       // |e| = 2 sJ = 2 Fscale J
+                }
+                for (int i = 0; i < Np; ++i) beta = fmax(beta, sB[tid * Np + i]);
+                const double rhoK = 4.0 * g[G_J] / perim;
+                const double cinv2 = double(p) * p * p * p / (rhoK * rhoK);
+                const double lam = 1.5 * cinv2 * GK + 3.0 * ciK * (3.0 * sigK + beta);
+                if (!isfinite(lam)) isbad = 1;
+                else if (lam > 0.0) atomicMax(&best, static_cast<unsigned long long>(__double_as_longlong(lam)));
+            }
+            __syncthreads();
+        }
     }
-    if (threadIdx.x == 0) *out = s[0];
+    __syncthreads();
+    unsigned long long *gbest = reinterpret_cast<unsigned long long *>(words + 2);
+    if (tid == 0) {
+        if (best) atomicMax(gbest, best);
+        if (isbad) atomicExch(words + 4, 1u);
+        __threadfence();
+        if (atomicAdd(words + 1, 1u) == gridDim.x - 1) {
+            __threadfence();
+            const unsigned long long b = atomicExch(gbest, 0ull);
+            *out = atomicExch(words + 4, 0u) ? NAN : __longlong_as_double(static_cast<long long>(b));
+            words[0] = 0u;
+            words[1] = 0u;
+        }
+    }
 }
 
 // Force and moment of one wall face: traction p n - tau n at its face nodes
@@ -434,18 +464,12 @@ cudaError_t launch_batch_forces_record(const double *partial, const int *wseg, B
     return cudaGetLastError();
 }
 
-cudaError_t launch_dt_lambda(const AuxMesh &m, const Phys<double> &ph, double sig_fac, double *lam,
-                             cudaStream_t st)
+cudaError_t launch_dt_confirm(const AuxMesh &m, const Phys<double> &ph, double sig_fac, const float *lam,
+                              unsigned *words, double *out, cudaStream_t st)
 {
-    int threads = 128;
-    long long blocks = (m.K + threads - 1) / threads;
-    dt_lambda_kernel<<<static_cast<unsigned>(blocks), threads, 0, st>>>(m, ph, sig_fac, lam);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_max_reduce(const double *lam, long long K, double *out, cudaStream_t st)
-{
-    max_reduce_kernel<<<1, 1024, 0, st>>>(lam, K, out);
+    const long long most = (m.K + 127) / 128;
+    const int blocks = static_cast<int>(most < 1216 ? most : 1216);      // 8 blocks on each of 152 SMs
+    dt_confirm_kernel<<<blocks, 128, 0, st>>>(m, ph, sig_fac, lam, words, out);
     return cudaGetLastError();
 }
 

@@ -42,7 +42,9 @@ struct dg_ctx {
     std::vector<int32_t> EToV;
     std::vector<double> geo64h;
     // device
-    dg::DevBuf<double> K0a, K0b, K1, rtmp, geo64, ops64, Dr64, Ds64, src, lam, scal, fpart, fxy, wface;
+    dg::DevBuf<double> K0a, K0b, K1, rtmp, geo64, ops64, Dr64, Ds64, src, scal, fpart, fxy, wface;
+    dg::DevBuf<float> lam;                        // time-step bound: screened Lambda_K
+    dg::DevBuf<unsigned> dtw;                     // ... and its words (zero between calls)
     dg::DevBuf<float> geo32, ops32, P0a, P0b;     // mixed path: pressures of the two K0 buffers
     dg::DevBuf<float4> S0a, S0b;                  // mixed path: FP32 copies of the two K0 buffers
     dg::DevBuf<int4> conn;
@@ -84,7 +86,7 @@ struct dg_ctx {
     unsigned *ticket() { return reinterpret_cast<unsigned *>(scal.ptr + 3); }
     ~dg_ctx()
     {
-        for (auto *b : {&K0a, &K0b, &K1, &rtmp, &geo64, &ops64, &Dr64, &Ds64, &src, &lam, &scal, &fpart, &fxy, &wface})
+        for (auto *b : {&K0a, &K0b, &K1, &rtmp, &geo64, &ops64, &Dr64, &Ds64, &src, &scal, &fpart, &fxy, &wface})
             b->release();
         geo32.release();
         ops32.release();
@@ -311,13 +313,14 @@ dg_status dg_create(const dg_params *params, void *cuda_stream, dg_ctx **out)
     if (c->ops64.alloc(o64.size()) != cudaSuccess || c->ops32.alloc(o32.size()) != cudaSuccess ||
         c->Dr64.alloc(Np * Np) != cudaSuccess || c->Ds64.alloc(Np * Np) != cudaSuccess ||
         c->fmask.alloc(NF) != cudaSuccess || c->flag.alloc(1) != cudaSuccess || c->bar_err.alloc(1) != cudaSuccess ||
-        c->scal.alloc(4) != cudaSuccess || c->wface.alloc(c->ops.Nfp) != cudaSuccess) {
+        c->scal.alloc(4) != cudaSuccess || c->dtw.alloc(8) != cudaSuccess || c->wface.alloc(c->ops.Nfp) != cudaSuccess) {
         cudaGetLastError();
         delete c;
         return DG_ECUDA;
     }
     cudaMemset(c->bar_err.ptr, 0, sizeof(int));
     cudaMemset(c->scal.ptr, 0, 4 * sizeof(double));
+    cudaMemset(c->dtw.ptr, 0, 8 * sizeof(unsigned));
     cudaMemcpy(c->ops64.ptr, o64.data(), o64.size() * sizeof(double), cudaMemcpyHostToDevice);
     cudaMemcpy(c->ops32.ptr, o32.data(), o32.size() * sizeof(float), cudaMemcpyHostToDevice);
     if (dg::stage_tc_supported(p.p)) {
@@ -772,8 +775,10 @@ dg_status dg_compute_dt(dg_ctx *c, double cfl, const double vw[2], double *dt)
     c->err.clear();
     if (!dt || c->K < 1 || !(cfl > 0.0)) return fail(c, DG_EINVAL, "need dt pointer, mesh and cfl > 0");
     dg::Phys<double> ph = make_phys<double>(c->prm, vw);
-    DG_CUDA(c, dg::launch_dt_lambda(aux_mesh(c), ph, sigma_factor(c->prm), c->lam.ptr, c->stream));
-    DG_CUDA(c, dg::launch_max_reduce(c->lam.ptr, c->K, c->scal.ptr, c->stream));
+    const double sf = sigma_factor(c->prm);
+    DG_CUDA(c, dg::launch_dt_screen(aux_mesh(c), make_phys<float>(c->prm, vw), c->prm.gamma - 1.0,
+                                    static_cast<float>(sf), c->lam.ptr, c->dtw.ptr, c->stream));
+    DG_CUDA(c, dg::launch_dt_confirm(aux_mesh(c), ph, sf, c->lam.ptr, c->dtw.ptr, c->scal.ptr, c->stream));
     c->launches += 2;
     double lam = 0.0;
     DG_CUDA(c, cudaMemcpyAsync(&lam, c->scal.ptr, sizeof(double), cudaMemcpyDeviceToHost, c->stream));

@@ -644,15 +644,6 @@ __device__ __forceinline__ void dt_lambda_mixed_tile(const float4 *S, const floa
     }
 }
 
-template <int P>
-__global__ void __launch_bounds__(Shape<P>::NT)
-dt_lambda_mixed_kernel(const float4 *S, const float *Pr, const float *geo, const int4 *conn, const int *fmask,
-                       const int4 *tiles, const BatchCase *cases, long long K, Phys<float> ph, float sig_fac,
-                       double *lam)
-{
-    dt_lambda_mixed_tile<P>(S, Pr, geo, conn, fmask, tiles, cases, K, ph, sig_fac, lam, blockIdx.x);
-}
-
 // The time-step bound of every degree group of a batch in one launch: block
 // b works on tile b - first_block of the group whose block range holds b.
 template <int... Ps>

@@ -55,15 +55,9 @@ cudaError_t launch_stage_mixed(int p, const LaunchShape &ls, const StageParams &
 cudaError_t stage_shape_mixed_batch(int p, long long ntiles, LaunchShape &out);
 cudaError_t launch_stage_mixed_batch(int p, const LaunchShape &ls, const StageParams &sp,
                                      const Phys<float> &ph, cudaStream_t st);
-// Lambda_K in FP32 from the FP32 state copy (mixed path); tiles == nullptr:
-// K elements in tiles of E, ph carries mu and v_w; otherwise the batch tile
-// table and per-case mu, v_b
 // Lambda_K of every degree group of a batch in one launch (one block per tile)
 cudaError_t launch_dt_lambda_mixed_multi(const DtGroups &dgs, const BatchCase *cases, const Phys<float> &ph,
                                          float sig_fac, cudaStream_t st);
-cudaError_t launch_dt_lambda_mixed(int p, const float4 *S, const float *Pr, const float *geo, const int4 *conn,
-                                   const int *fmask, const int4 *tiles, long long ntiles, const BatchCase *cases,
-                                   long long K, const Phys<float> &ph, float sig_fac, double *lam, cudaStream_t st);
 // the mixed IIP kernel with two nodes per thread: units = K elements (single
 // mesh) or the tile count of a tile table (batch); its tiles hold
 // stage_tile_elems2(p) elements
@@ -120,12 +114,14 @@ struct AuxMesh {
     int p;
 };
 
-// Lambda_K of Eq. rayleigh_bound per element into lam[K] (FP64);
-// sig_fac = C1 (1+theta)^2 (d+1) of Eq. penalty_final.
-cudaError_t launch_dt_lambda(const AuxMesh &m, const Phys<double> &ph, double sig_fac,
-                             double *lam, cudaStream_t st);
-// max over lam[0..K) into *out (one block).
-cudaError_t launch_max_reduce(const double *lam, long long K, double *out, cudaStream_t st);
+// max_K Lambda_K of Eq. rayleigh_bound in FP64: an FP32 screen of every
+// element into lam[K], then FP64 on the elements that can hold the maximum,
+// whose value goes to *out (NaN if one is not finite).  sig_fac = C1
+// (1+theta)^2 (d+1) of Eq. penalty_final; words: 8 words, zero between calls.
+cudaError_t launch_dt_screen(const AuxMesh &m, const Phys<float> &ph, double gm1d, float sig_fac, float *lam,
+                             unsigned *words, cudaStream_t st);
+cudaError_t launch_dt_confirm(const AuxMesh &m, const Phys<double> &ph, double sig_fac, const float *lam,
+                              unsigned *words, double *out, cudaStream_t st);
 
 // per-wall-face force/moment partials and their sum (fixed order) into out[3],
 // one launch; *ticket counts finished blocks, zero before and after it

@@ -1,5 +1,6 @@
 // stage_mixed.cu -- mixed-precision stage kernel instantiations (p = 1..6):
 // FP32 arithmetic, FP64 state in HBM, FP64 pressure recovery and registers.
+#include "dg_dt.cuh"
 #include "dg_stage_mixed.cuh"
 #include "dg_stage_mixed2.cuh"
 #include "launch.h"
@@ -225,18 +226,6 @@ cudaError_t launch_stage_mixed_batch(int p, const LaunchShape &ls, const StagePa
 #undef C_
 }
 
-template <int P>
-cudaError_t dt_mixed_p(const float4 *S, const float *Pr, const float *geo, const int4 *conn, const int *fmask,
-                       const int4 *tiles, long long ntiles, const BatchCase *cases, long long K,
-                       const Phys<float> &ph, float sig_fac, double *lam, cudaStream_t st)
-{
-    const long long nblk = tiles ? ntiles : (K + Shape<P>::E - 1) / Shape<P>::E;
-    if (nblk < 1) return cudaSuccess;
-    dt_lambda_mixed_kernel<P><<<static_cast<unsigned>(nblk), Shape<P>::NT, 0, st>>>(S, Pr, geo, conn, fmask, tiles,
-                                                                                   cases, K, ph, sig_fac, lam);
-    return cudaGetLastError();
-}
-
 cudaError_t launch_dt_lambda_mixed_multi(const DtGroups &dgs, const BatchCase *cases, const Phys<float> &ph,
                                          float sig_fac, cudaStream_t st)
 {
@@ -246,12 +235,21 @@ cudaError_t launch_dt_lambda_mixed_multi(const DtGroups &dgs, const BatchCase *c
     return cudaGetLastError();
 }
 
-cudaError_t launch_dt_lambda_mixed(int p, const float4 *S, const float *Pr, const float *geo, const int4 *conn,
-                                   const int *fmask, const int4 *tiles, long long ntiles, const BatchCase *cases,
-                                   long long K, const Phys<float> &ph, float sig_fac, double *lam, cudaStream_t st)
+template <int P>
+cudaError_t dt_screen_p(const AuxMesh &m, const Phys<float> &ph, double gm1d, float sig_fac, float *lam,
+                        unsigned *words, cudaStream_t st)
 {
-#define C_(P) dt_mixed_p<P>(S, Pr, geo, conn, fmask, tiles, ntiles, cases, K, ph, sig_fac, lam, st)
-    DG_SWITCH_P(p, C_)
+    const long long blocks = (m.K + Shape<P>::E - 1) / Shape<P>::E;
+    dt_screen_kernel<P><<<static_cast<unsigned>(blocks), Shape<P>::NT, 0, st>>>(m.U, m.geo, m.conn, m.fmask, m.K, ph,
+                                                                               gm1d, sig_fac, lam, words);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_dt_screen(const AuxMesh &m, const Phys<float> &ph, double gm1d, float sig_fac, float *lam,
+                             unsigned *words, cudaStream_t st)
+{
+#define C_(P) dt_screen_p<P>(m, ph, gm1d, sig_fac, lam, words, st)
+    DG_SWITCH_P(m.p, C_)
 #undef C_
 }
 
