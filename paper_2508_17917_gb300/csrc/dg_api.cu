@@ -42,6 +42,11 @@ struct dg_ctx {
     std::vector<int32_t> EToV;
     std::vector<double> geo64h;
     // device
+    // FP64 path: symmetric operator tables, every face once, phase arrays
+    dg::DevBuf<double> sym64, flux64, dh64, th64;
+    dg::DevBuf<int> symn;
+    dg::DevBuf<int4> faces;
+    int nfaces = 0;
     dg::DevBuf<double> K0a, K0b, K1, rtmp, geo64, ops64, Dr64, Ds64, src, scal, fpart, fxy, wface;
     dg::DevBuf<float> lam;                        // time-step bound: screened Lambda_K
     dg::DevBuf<unsigned> dtw;                     // ... and its words (zero between calls)
@@ -104,8 +109,13 @@ struct dg_ctx {
 
 namespace {
 
+// waits of about 100 ns (1.7 s in all) before a grid barrier between the
+// phases of an FP64 stage gives up; its blocks are resident together, so a
+// wait is as long as the slowest block's share of a phase
+constexpr unsigned kPhaseWaitLimit = 1u << 24;
+
 const char *const kWaitGaveUp =
-    "a bounded device wait gave up (a fused step's grid barrier or a stage kernel's copy wait: "
+    "a bounded device wait gave up (a grid barrier of a fused step or an FP64 stage, or a stage kernel's copy wait: "
     "the state is not valid; or the tcgen05 gradient kernel: its output is not valid)";
 
 dg_status fail(dg_ctx *c, dg_status st, const std::string &msg)
@@ -124,6 +134,23 @@ dg_status cuda_fail(dg_ctx *c, cudaError_t e, const char *where)
         cudaError_t e_ = (expr);                                  \
         if (e_ != cudaSuccess) return cuda_fail(ctx, e_, #expr);  \
     } while (0)
+
+// the words of the grid barriers, zero before their first launch
+dg_status need_barrier(dg_ctx *c)
+{
+    if (c->bar.ptr) return DG_OK;
+    DG_CUDA(c, c->bar.alloc(2));
+    DG_CUDA(c, cudaMemset(c->bar.ptr, 0, 2 * sizeof(unsigned)));
+    return DG_OK;
+}
+
+// clear the error flag and the barrier words a launch that gave up left behind
+dg_status wait_gave_up(dg_ctx *c)
+{
+    DG_CUDA(c, cudaMemset(c->bar_err.ptr, 0, sizeof(int)));
+    if (c->bar.ptr) DG_CUDA(c, cudaMemset(c->bar.ptr, 0, 2 * sizeof(unsigned)));
+    return fail(c, DG_ETIMEOUT, kWaitGaveUp);
+}
 
 template <typename real>
 dg::Phys<real> make_phys(const dg_params &p, const double vw[2])
@@ -215,7 +242,16 @@ dg_status run_stage(dg_ctx *c, int s, double t, double dt, const double vw[2], i
     if (c->prm.precision == DG_PRECISION_FP64) {
         sp.geo = c->geo64.ptr;
         sp.ops = c->ops64.ptr;
-        e = dg::launch_stage_fp64(c->prm.p, c->shape, sp, make_phys<double>(c->prm, vw), c->stream);
+        if (!c->shape.overint) {
+            // grid barriers between its phases, reported through the barrier flag
+            sp.bar = c->bar.ptr;
+            sp.bar_err = c->bar_err.ptr;
+            sp.bar_limit = kPhaseWaitLimit;
+            c->copy_used = true;
+        }
+        const dg::Stage64Args a64{c->sym64.ptr, c->symn.ptr, c->faces.ptr, c->nfaces, c->flux64.ptr, c->dh64.ptr,
+                                  c->th64.ptr};
+        e = dg::launch_stage_fp64(c->prm.p, c->shape, sp, a64, make_phys<double>(c->prm, vw), c->stream);
     } else {
         sp.geo = c->geo32.ptr;
         sp.ops = (c->shape.variant == 3) ? static_cast<const void *>(c->tcfrag.ptr) : c->ops32.ptr;
@@ -323,6 +359,21 @@ dg_status dg_create(const dg_params *params, void *cuda_stream, dg_ctx **out)
     cudaMemset(c->dtw.ptr, 0, 8 * sizeof(unsigned));
     cudaMemcpy(c->ops64.ptr, o64.data(), o64.size() * sizeof(double), cudaMemcpyHostToDevice);
     cudaMemcpy(c->ops32.ptr, o32.data(), o32.size() * sizeof(float), cudaMemcpyHostToDevice);
+    {
+        std::vector<double> tab;
+        std::vector<int> nodes;
+        if (!dg::build_sym64_tables(c->ops, tab, nodes)) {
+            delete c;
+            return DG_EINVAL;
+        }
+        if (c->sym64.alloc(tab.size()) != cudaSuccess || c->symn.alloc(nodes.size()) != cudaSuccess) {
+            cudaGetLastError();
+            delete c;
+            return DG_ECUDA;
+        }
+        cudaMemcpy(c->sym64.ptr, tab.data(), tab.size() * sizeof(double), cudaMemcpyHostToDevice);
+        cudaMemcpy(c->symn.ptr, nodes.data(), nodes.size() * sizeof(int), cudaMemcpyHostToDevice);
+    }
     if (dg::stage_tc_supported(p.p)) {
         std::vector<float> frag;
         dg::build_tc_fragments(Np, NF, c->ops.Dr.data(), c->ops.Ds.data(), c->ops.LIFT.data(), c->ops.Wr.data(),
@@ -378,9 +429,9 @@ dg_status dg_set_fused_steps(dg_ctx *c, int on)
     c->err.clear();
     if (on && (c->prm.precision != DG_PRECISION_MIXED || c->prm.theta != 0.0))
         return fail(c, DG_EUNSUPPORTED, "fused steps use the mixed-precision IIP kernels");
-    if (on && !c->bar.ptr) {
-        DG_CUDA(c, c->bar.alloc(2));
-        DG_CUDA(c, cudaMemset(c->bar.ptr, 0, 2 * sizeof(unsigned)));
+    if (on) {
+        dg_status st = need_barrier(c);
+        if (st != DG_OK) return st;
     }
     c->fused = on != 0;
     return DG_OK;
@@ -403,10 +454,7 @@ dg_status dg_barrier_status(dg_ctx *c)
     DG_CUDA(c, cudaStreamSynchronize(c->stream));
     c->bar_used = false;
     c->copy_used = false;
-    if (e) {
-        DG_CUDA(c, cudaMemset(c->bar_err.ptr, 0, sizeof(int)));
-        return fail(c, DG_ETIMEOUT, kWaitGaveUp);
-    }
+    if (e) return wait_gave_up(c);
     return DG_OK;
 }
 
@@ -456,6 +504,31 @@ dg_status dg_set_mesh(dg_ctx *c, int64_t Nv, const double *vx, const double *vy,
     DG_CUDA(c, c->lam.alloc(K));
     DG_CUDA(c, cudaMemcpy(c->geo64.ptr, geo.data(), geo.size() * sizeof(double), cudaMemcpyHostToDevice));
     DG_CUDA(c, cudaMemcpy(c->conn.ptr, conn.data(), K * sizeof(int4), cudaMemcpyHostToDevice));
+    if (c->prm.precision == DG_PRECISION_FP64) {
+        // every face once: interior faces in element order, then the boundary
+        std::vector<int4> fl, bl;
+        fl.reserve(static_cast<size_t>(K) * 3 / 2 + 3);
+        for (int64_t k = 0; k < K; ++k) {
+            const int4 cn = conn[k];
+            for (int f = 0; f < 3; ++f) {
+                const int nb = f == 0 ? cn.x : (f == 1 ? cn.y : cn.z);
+                const int f2 = (cn.w >> (2 * f)) & 3, bt = (cn.w >> (8 + 2 * f)) & 3;
+                const int4 fc = make_int4(static_cast<int>(k), nb, f | (f2 << 2) | (bt << 4), 0);
+                if (bt != dg::BCT_INTERIOR) bl.push_back(fc);
+                else if (k < nb) fl.push_back(fc);
+            }
+        }
+        fl.insert(fl.end(), bl.begin(), bl.end());
+        c->nfaces = static_cast<int>(fl.size());
+        DG_CUDA(c, c->faces.alloc(fl.size()));
+        DG_CUDA(c, cudaMemcpy(c->faces.ptr, fl.data(), fl.size() * sizeof(int4), cudaMemcpyHostToDevice));
+        const size_t nfn = static_cast<size_t>(K) * 3 * c->ops.Nfp;
+        DG_CUDA(c, c->flux64.alloc(2 * nd));
+        DG_CUDA(c, c->dh64.alloc(4 * nfn));
+        if (c->prm.theta != 0.0) DG_CUDA(c, c->th64.alloc(8 * nfn));
+        dg_status bs = need_barrier(c);
+        if (bs != DG_OK) return bs;
+    }
     if (c->prm.precision == DG_PRECISION_MIXED) {
         std::vector<float> g32(geo.begin(), geo.end());
         DG_CUDA(c, c->geo32.alloc(g32.size()));
@@ -565,10 +638,7 @@ dg_status dg_get_state(dg_ctx *c, double *U, int on_device)
     if (check) {
         c->bar_used = false;
         c->copy_used = false;
-        if (e) {
-            DG_CUDA(c, cudaMemset(c->bar_err.ptr, 0, sizeof(int)));
-            return fail(c, DG_ETIMEOUT, kWaitGaveUp);
-        }
+        if (e) return wait_gave_up(c);
     }
     return DG_OK;
 }

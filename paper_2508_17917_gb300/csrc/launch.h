@@ -47,8 +47,23 @@ inline cudaError_t launch_pdl(void (*kern)(Args...), const LaunchShape &ls, cuda
 // on the current device (persistent grid: SMs x resident CTAs, capped by tiles).
 cudaError_t stage_shape_fp64(int p, long long K, bool theta, LaunchShape &out, bool overint = false);
 cudaError_t stage_shape_mixed(int p, long long K, bool theta, LaunchShape &out);
-cudaError_t launch_stage_fp64(int p, const LaunchShape &ls, const StageParams &sp,
+// what the three-phase FP64 stage kernel reads and keeps besides StageParams:
+// the symmetric operator tables of build_sym64_tables, every face once as
+// (element, neighbour, face | its face << 2 | boundary type << 4, 0) with the
+// interior ones first, and its arrays (fluxes [K][Np][8], face terms
+// [K][3 Nfp][4], with theta terms [K][3 Nfp][8])
+struct Stage64Args {
+    const double *ops;
+    const int *nodes;
+    const int4 *faces;
+    int nfaces;
+    double *flux, *dh, *th;
+};
+cudaError_t launch_stage_fp64(int p, const LaunchShape &ls, const StageParams &sp, const Stage64Args &a,
                               const Phys<double> &ph, cudaStream_t st);
+// false if the operators are not symmetric under r <-> s
+struct RefOps;
+bool build_sym64_tables(const RefOps &o, std::vector<double> &tab, std::vector<int> &nodes);
 cudaError_t launch_stage_mixed(int p, const LaunchShape &ls, const StageParams &sp,
                                const Phys<float> &ph, cudaStream_t st);
 // batch variant of the mixed kernel (IIP): grid for `ntiles` tiles of a tile table

@@ -1,15 +1,22 @@
-// stage_fp64.cu -- FP64 instantiations of the fused stage kernel (p = 1..6).
-#include "dg_stage.cuh"
+// stage_fp64.cu -- the FP64 stage kernels (p = 1..6): the three-phase kernel
+// of dg_stage64.cuh with its operator tables and the over-integrated kernel
+// of dg_stage.cuh.
+#include <cmath>
+#include <vector>
+
+#include "dg_stage64.cuh"
 #include "launch.h"
+#include "refops.h"
 
 namespace dg {
 namespace {
 
-template <int P, typename real, bool TH, bool OI = false>
-cudaError_t shape_p(long long K, LaunchShape &ls)
+// over-integrated volume term
+template <int P>
+cudaError_t shape_oi_p(long long K, LaunchShape &ls)
 {
-    using L = Smem<P, real, TH, OI>;
-    auto kern = stage_kernel<P, real, TH, OI>;
+    using L = Smem<P, double>;
+    auto kern = stage_kernel<P, double>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          static_cast<int>(L::bytes));
     if (e != cudaSuccess) return e;
@@ -25,21 +32,138 @@ cudaError_t shape_p(long long K, LaunchShape &ls)
     ls.threads = Shape<P>::NT;
     ls.smem = L::bytes;
     ls.elems_per_tile = Shape<P>::E;
-    ls.theta = TH;
-    ls.overint = OI;
+    ls.theta = false;
+    ls.overint = true;
     return cudaSuccess;
 }
 
-template <int P, typename real>
-cudaError_t launch_p(const LaunchShape &ls, const StageParams &sp, const Phys<real> &ph, cudaStream_t st)
+// three phases in a cooperative launch: as many blocks as are resident at
+// once, capped by what the widest phase has for them
+template <int P, bool TH>
+cudaError_t shape64_p(long long K, LaunchShape &ls)
 {
-    if (ls.overint)
-        stage_kernel<P, real, false, true><<<ls.grid, ls.threads, ls.smem, st>>>(sp, ph);
-    else if (ls.theta)
-        stage_kernel<P, real, true><<<ls.grid, ls.threads, ls.smem, st>>>(sp, ph);
-    else
-        stage_kernel<P, real, false><<<ls.grid, ls.threads, ls.smem, st>>>(sp, ph);
-    return cudaGetLastError();
+    using S = Sym64<P>;
+    using L = Layout64<P, TH>;
+    auto kern = stage64_kernel<P, TH>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(L::bytes));
+    if (e != cudaSuccess) return e;
+    int per_sm = 0, dev = 0, sms = 0;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, S::NT, L::bytes);
+    if (e != cudaSuccess) return e;
+    if (per_sm < 1) return cudaErrorInvalidConfiguration;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const long long tiles = (K + S::EB - 1) / S::EB, groups = (3 * K + 4 * (32 / S::Nfp) - 1) / (4 * (32 / S::Nfp));
+    const long long most = tiles > groups ? tiles : groups, grid = static_cast<long long>(sms) * per_sm;
+    ls.grid = static_cast<int>(most < grid ? most : grid);
+    ls.threads = S::NT;
+    ls.smem = L::bytes;
+    ls.elems_per_tile = S::EB;
+    ls.theta = TH;
+    ls.overint = false;
+    return cudaSuccess;
+}
+
+template <int P>
+cudaError_t launch64_p(const LaunchShape &ls, const StageParams &sp, const Stage64 &x, const Phys<double> &ph,
+                       cudaStream_t st)
+{
+    if (ls.overint) {
+        stage_kernel<P, double><<<ls.grid, ls.threads, ls.smem, st>>>(sp, ph);
+        return cudaGetLastError();
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(ls.grid);
+    cfg.blockDim = dim3(ls.threads);
+    cfg.dynamicSmemBytes = ls.smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (ls.theta) return cudaLaunchKernelEx(&cfg, stage64_kernel<P, true>, sp, x, ph);
+    return cudaLaunchKernelEx(&cfg, stage64_kernel<P, false>, sp, x, ph);
+}
+
+template <int P>
+bool sym64_tables_p(const RefOps &o, std::vector<double> &tab, std::vector<int> &nodes)
+{
+    using S = Sym64<P>;
+    constexpr int Np = S::Np, NF = S::NF, NO = S::NO, NE = S::NE, TPE = S::TPE, NEF = S::NEF;
+    // mirrored nodes: (r, s) -> (s, r)
+    int mirror[Np];
+    for (int i = 0; i < Np; ++i) {
+        mirror[i] = -1;
+        for (int j = 0; j < Np; ++j)
+            if (std::fabs(o.r[i] - o.s[j]) < 1e-10 && std::fabs(o.s[i] - o.r[j]) < 1e-10) mirror[i] = j;
+        if (mirror[i] < 0) return false;
+    }
+    std::vector<int> pair, axis;
+    for (int i = 0; i < Np; ++i) {
+        if (mirror[i] == i) axis.push_back(i);
+        else if (i < mirror[i]) pair.push_back(i);
+    }
+    if (static_cast<int>(pair.size()) != NO || static_cast<int>(axis.size()) != NE - NO) return false;
+    // the reflection exchanges Dr and Ds (and Wr, Ws) and mirrors the face slots
+    double worst = 0.0;
+    for (int i = 0; i < Np; ++i) {
+        for (int j = 0; j < Np; ++j) {
+            worst = std::fmax(worst, std::fabs(o.Dr[i * Np + j] - o.Ds[mirror[i] * Np + mirror[j]]));
+            worst = std::fmax(worst, std::fabs(o.Wr[i * Np + j] - o.Ws[mirror[i] * Np + mirror[j]]));
+        }
+        for (int m = 0; m < NF; ++m)
+            worst = std::fmax(worst, std::fabs(o.LIFT[i * NF + m] - o.LIFT[mirror[i] * NF + NF - 1 - m]));
+    }
+    if (!(worst < 1e-9)) return false;
+    // Q = W LIFT for the theta terms
+    std::vector<double> Pm(Np * Np), Mm(Np * Np), Qp(Np * NF, 0.0), Qm(Np * NF, 0.0);
+    for (int i = 0; i < Np * Np; ++i) {
+        Pm[i] = 0.5 * (o.Dr[i] + o.Ds[i]);
+        Mm[i] = 0.5 * (o.Dr[i] - o.Ds[i]);
+    }
+    for (int i = 0; i < Np; ++i)
+        for (int m = 0; m < NF; ++m)
+            for (int j = 0; j < Np; ++j) {
+                Qp[i * NF + m] += 0.5 * (o.Wr[i * Np + j] + o.Ws[i * Np + j]) * o.LIFT[j * NF + m];
+                Qm[i * NF + m] += 0.5 * (o.Wr[i * Np + j] - o.Ws[i * Np + j]) * o.LIFT[j * NF + m];
+            }
+    // even (sign +1) and odd (-1) rows of a matrix over nodes, and over face slots
+    auto node_row = [&](const std::vector<double> &A, int i, int l, double sign) {
+        if (l >= NO) return sign > 0 ? A[i * Np + axis[l - NO]] : 0.0;
+        return 0.5 * (A[i * Np + pair[l]] + sign * A[i * Np + mirror[pair[l]]]);
+    };
+    auto face_row = [&](const std::vector<double> &A, int i, int m, double sign) {
+        if (m == NF - 1 - m) return sign > 0 ? A[i * NF + m] : 0.0;
+        return 0.5 * (A[i * NF + m] + sign * A[i * NF + NF - 1 - m]);
+    };
+    tab.assign(2 * S::NTAB, 0.0);
+    nodes.assign(2 * TPE, -1);
+    for (int t = 0; t < TPE; ++t) {
+        const bool pr = t < NO;
+        const int a = pr ? pair[t] : axis[2 * (t - NO)];
+        const int b = pr ? mirror[pair[t]] : (2 * (t - NO) + 1 < NE - NO ? axis[2 * (t - NO) + 1] : -1);
+        nodes[2 * t] = a;
+        nodes[2 * t + 1] = b;
+        auto put = [&](int at, double x, double y) {
+            tab[2 * (at + t)] = x;
+            tab[2 * (at + t) + 1] = y;
+        };
+        for (int l = 0; l < NE; ++l)
+            put(l * TPE, node_row(Pm, a, l, 1), pr ? node_row(Mm, a, l, 1) : (b < 0 ? 0.0 : node_row(Pm, b, l, 1)));
+        for (int l = 0; l < NO; ++l)
+            put(S::oB + l * TPE, pr ? node_row(Pm, a, l, -1) : (b < 0 ? 0.0 : node_row(Mm, b, l, -1)),
+                node_row(Mm, a, l, -1));
+        for (int m = 0; m < NEF; ++m) {
+            put(S::oL + m * TPE, -face_row(o.LIFT, a, m, 1),
+                pr ? -face_row(o.LIFT, a, m, -1) : (b < 0 ? 0.0 : -face_row(o.LIFT, b, m, 1)));
+            put(S::oQA + m * TPE, -face_row(Qp, a, m, 1),
+                pr ? -face_row(Qm, a, m, 1) : (b < 0 ? 0.0 : -face_row(Qp, b, m, 1)));
+            put(S::oQB + m * TPE, pr ? -face_row(Qp, a, m, -1) : (b < 0 ? 0.0 : -face_row(Qm, b, m, -1)),
+                -face_row(Qm, a, m, -1));
+        }
+    }
+    return true;
 }
 
 }  // namespace
@@ -57,18 +181,31 @@ cudaError_t launch_p(const LaunchShape &ls, const StageParams &sp, const Phys<re
 
 cudaError_t stage_shape_fp64(int p, long long K, bool theta, LaunchShape &out, bool overint)
 {
-#define C_(P) (overint ? shape_p<P, double, false, true>(K, out) \
-                       : (theta ? shape_p<P, double, true>(K, out) : shape_p<P, double, false>(K, out)))
+#define C_(P) (overint ? shape_oi_p<P>(K, out) : (theta ? shape64_p<P, true>(K, out) : shape64_p<P, false>(K, out)))
     DG_SWITCH_P(p, C_)
 #undef C_
 }
 
-cudaError_t launch_stage_fp64(int p, const LaunchShape &ls, const StageParams &sp,
+cudaError_t launch_stage_fp64(int p, const LaunchShape &ls, const StageParams &sp, const Stage64Args &a,
                               const Phys<double> &ph, cudaStream_t st)
 {
-#define C_(P) launch_p<P, double>(ls, sp, ph, st)
+    const Stage64 x{reinterpret_cast<const double2 *>(a.ops), a.nodes, a.faces, a.nfaces, a.flux, a.dh, a.th};
+#define C_(P) launch64_p<P>(ls, sp, x, ph, st)
     DG_SWITCH_P(p, C_)
 #undef C_
+}
+
+bool build_sym64_tables(const RefOps &o, std::vector<double> &tab, std::vector<int> &nodes)
+{
+    switch (o.p) {
+    case 1: return sym64_tables_p<1>(o, tab, nodes);
+    case 2: return sym64_tables_p<2>(o, tab, nodes);
+    case 3: return sym64_tables_p<3>(o, tab, nodes);
+    case 4: return sym64_tables_p<4>(o, tab, nodes);
+    case 5: return sym64_tables_p<5>(o, tab, nodes);
+    case 6: return sym64_tables_p<6>(o, tab, nodes);
+    default: return false;
+    }
 }
 
 }  // namespace dg
