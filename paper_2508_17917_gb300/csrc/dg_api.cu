@@ -909,34 +909,31 @@ dg_status dg_broken_gradient(dg_ctx *c, double *gx, double *gy, int on_device, i
         ox = c->gtmp.ptr;
         oy = c->gtmp.ptr + n;
     }
-    dg::GradTc05Args a{};
-    a.U = c->cur();
-    a.Dr = c->ops.Dr.data();
-    a.Ds = c->ops.Ds.data();
-    a.Dr_dev = c->Dr64.ptr;
-    a.Ds_dev = c->Ds64.ptr;
-    a.geo = c->geo64.ptr;
-    a.K = c->K;
-    a.gx = ox;
-    a.gy = oy;
-    a.wait_limit = 1u << 20;
-    if (impl == 1) {
+    if (impl == 0) {
+        DG_CUDA(c, dg::launch_grad64(c->prm.p, c->cur(), c->geo64.ptr, c->sym64.ptr, c->symn.ptr, c->K, ox, oy,
+                                     c->stream));
+    } else {
+        dg::GradTc05Args a{};
+        a.U = c->cur();
+        a.Dr = c->ops.Dr.data();
+        a.Ds = c->ops.Ds.data();
+        a.geo = c->geo64.ptr;
+        a.K = c->K;
+        a.gx = ox;
+        a.gy = oy;
+        a.wait_limit = 1u << 20;
         const size_t nf = dg::grad_tc05_bimg_floats(c->prm.p);
         if (c->gimg.n != nf) {
             DG_CUDA(c, c->gimg.alloc(nf));
             c->gimg_ready = false;
         }
-        if (!c->bar_err.ptr) {
-            DG_CUDA(c, c->bar_err.alloc(1));
-            DG_CUDA(c, cudaMemset(c->bar_err.ptr, 0, sizeof(int)));
-        }
         a.bimg = c->gimg.ptr;
         a.upload_ops = !c->gimg_ready;   // the operators are fixed by p: one upload per context
         a.err = c->bar_err.ptr;        // reported by dg_barrier_status, as for fused steps
         c->bar_used = true;
+        DG_CUDA(c, dg::launch_grad_tc05(c->prm.p, a, c->stream));
+        c->gimg_ready = true;
     }
-    DG_CUDA(c, dg::launch_broken_gradient(c->prm.p, impl, a, c->stream));
-    if (impl == 1) c->gimg_ready = true;
     c->launches += 1;
     if (!on_device) {
         DG_CUDA(c, cudaMemcpyAsync(gx, ox, n * sizeof(double), cudaMemcpyDeviceToHost, c->stream));

@@ -544,4 +544,53 @@ stage64_kernel(StageParams sp, Stage64 x, Phys<double> ph)
     }
 }
 
+// Broken gradient of every element (dg_broken_gradient, FP64), by the same
+// symmetric contraction: about 1,250 FP64 instructions per element at p = 4
+// against 2,040 with the plain rows, on a kernel bound by their number.
+template <int P>
+__global__ void __launch_bounds__(Sym64<P>::NT)
+grad64_kernel(const double *U, const double *geo, const double2 *ops, const int *nodes, long long K, double *gx, double *gy)
+{
+    using S = Sym64<P>;
+    constexpr int Np = S::Np, NE = S::NE, EB = S::EB, TPE = S::TPE;
+    __shared__ double2 tab[S::oL];
+    __shared__ __align__(16) double sX[EB * Np * 4];
+    const int tid = threadIdx.x;
+    for (int i = tid; i < S::oL; i += S::NT) tab[i] = ops[i];
+    const int e = tid / TPE, t = tid - (tid / TPE) * TPE;
+    const int nA = nodes[2 * t], nB = nodes[2 * t + 1], nb0 = nB < 0 ? nA : nB;
+    double *mine = sX + e * Np * 4;
+    const long long ntiles = (K + EB - 1) / EB;
+    for (long long tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+        const long long k = tile * EB + e;
+        const bool act = e < EB && k < K;
+        __syncthreads();
+        if (act) {
+            double a[4], b[4];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                a[c] = U[(k * 4 + c) * Np + nA];
+                b[c] = U[(k * 4 + c) * Np + nb0];
+            }
+            put_even_odd<P>(mine, mine + 4 * NE, 4, t, a, b);
+        }
+        __syncthreads();
+        if (!act) continue;
+        double Pu[2][4], Mu[2][4];
+        sym_gradient<P>(tab, mine, mine + 4 * NE, t, Pu, Mu);
+        const double *g = geo + k * 16;
+        const double ax = g[G_RX] + g[G_SX], ay = g[G_RY] + g[G_SY], bx = g[G_RX] - g[G_SX], by = g[G_RY] - g[G_SY];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            if (q == 1 && nB < 0) break;
+            const long long o = k * 4 * Np + (q ? nB : nA);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                gx[o + c * Np] = fma(ax, Pu[q][c], bx * Mu[q][c]);
+                gy[o + c * Np] = fma(ay, Pu[q][c], by * Mu[q][c]);
+            }
+        }
+    }
+}
+
 }  // namespace dg

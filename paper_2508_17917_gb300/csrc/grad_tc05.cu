@@ -290,31 +290,6 @@ grad_tc05_kernel(const __grid_constant__ CUtensorMap tmap, const float *bimg, co
                      : "memory");
 }
 
-// FP64 reference on the CUDA cores: one thread per (element, node)
-template <int P>
-__global__ void grad_fp64_kernel(const double *U, const double *Dr, const double *Ds, const double *geo, long long K,
-                                 double *gx, double *gy)
-{
-    constexpr int Np = (P + 1) * (P + 2) / 2;
-    const long long n = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x;
-    if (n >= K * Np) return;
-    const long long k = n / Np;
-    const int i = static_cast<int>(n - k * Np);
-    const double *g = geo + k * 16;
-    const double rx = g[G_RX], ry = g[G_RY], sx = g[G_SX], sy = g[G_SY];
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-        const double *u = U + (k * 4 + c) * Np;
-        double ur = 0.0, us = 0.0;
-        for (int j = 0; j < Np; ++j) {
-            ur += Dr[i * Np + j] * u[j];
-            us += Ds[i * Np + j] * u[j];
-        }
-        gx[(k * 4 + c) * Np + i] = rx * ur + sx * us;
-        gy[(k * 4 + c) * Np + i] = ry * ur + sy * us;
-    }
-}
-
 float tf32_round_host(float x)
 {
     unsigned u;
@@ -381,17 +356,6 @@ cudaError_t grad_tc05_p(const GradTc05Args &a, cudaStream_t st)
     return cudaGetLastError();
 }
 
-template <int P>
-cudaError_t grad_fp64_p(const GradTc05Args &a, cudaStream_t st)
-{
-    constexpr int Np = (P + 1) * (P + 2) / 2;
-    const long long n = a.K * Np;
-    if (n < 1) return cudaSuccess;
-    grad_fp64_kernel<P><<<static_cast<unsigned>((n + 127) / 128), 128, 0, st>>>(a.U, a.Dr_dev, a.Ds_dev, a.geo,
-                                                                                 a.K, a.gx, a.gy);
-    return cudaGetLastError();
-}
-
 }  // namespace
 
 size_t grad_tc05_bimg_floats(int p)
@@ -400,9 +364,9 @@ size_t grad_tc05_bimg_floats(int p)
     return static_cast<size_t>(2 * (NR / 8)) * (2 * NR) * 8;
 }
 
-cudaError_t launch_broken_gradient(int p, int impl, const GradTc05Args &a, cudaStream_t st)
+cudaError_t launch_grad_tc05(int p, const GradTc05Args &a, cudaStream_t st)
 {
-#define C_(P) (impl == 1 ? grad_tc05_p<P>(a, st) : grad_fp64_p<P>(a, st))
+#define C_(P) grad_tc05_p<P>(a, st)
     switch (p) {
     case 1: return C_(1);
     case 2: return C_(2);

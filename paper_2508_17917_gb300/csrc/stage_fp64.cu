@@ -1,6 +1,6 @@
 // stage_fp64.cu -- the FP64 stage kernels (p = 1..6): the three-phase kernel
-// of dg_stage64.cuh with its operator tables and the over-integrated kernel
-// of dg_stage.cuh.
+// of dg_stage64.cuh with its operator tables, the over-integrated kernel of
+// dg_stage.cuh, and the FP64 broken gradient.
 #include <cmath>
 #include <vector>
 
@@ -84,6 +84,22 @@ cudaError_t launch64_p(const LaunchShape &ls, const StageParams &sp, const Stage
     cfg.numAttrs = 1;
     if (ls.theta) return cudaLaunchKernelEx(&cfg, stage64_kernel<P, true>, sp, x, ph);
     return cudaLaunchKernelEx(&cfg, stage64_kernel<P, false>, sp, x, ph);
+}
+
+template <int P>
+cudaError_t grad64_p(const double *U, const double *geo, const double *ops, const int *nodes, long long K, double *gx,
+                     double *gy, cudaStream_t st)
+{
+    using S = Sym64<P>;
+    int per_sm = 0, dev = 0, sms = 0;
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, grad64_kernel<P>, S::NT, 0);
+    if (e != cudaSuccess) return e;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const long long tiles = (K + S::EB - 1) / S::EB, most = static_cast<long long>(sms) * (per_sm < 1 ? 1 : per_sm);
+    grad64_kernel<P><<<static_cast<unsigned>(tiles < most ? tiles : most), S::NT, 0, st>>>(
+        U, geo, reinterpret_cast<const double2 *>(ops), nodes, K, gx, gy);
+    return cudaGetLastError();
 }
 
 template <int P>
@@ -191,6 +207,14 @@ cudaError_t launch_stage_fp64(int p, const LaunchShape &ls, const StageParams &s
 {
     const Stage64 x{reinterpret_cast<const double2 *>(a.ops), a.nodes, a.faces, a.nfaces, a.flux, a.dh, a.th};
 #define C_(P) launch64_p<P>(ls, sp, x, ph, st)
+    DG_SWITCH_P(p, C_)
+#undef C_
+}
+
+cudaError_t launch_grad64(int p, const double *U, const double *geo, const double *ops, const int *nodes, long long K,
+                          double *gx, double *gy, cudaStream_t st)
+{
+#define C_(P) grad64_p<P>(U, geo, ops, nodes, K, gx, gy, st)
     DG_SWITCH_P(p, C_)
 #undef C_
 }
