@@ -431,9 +431,28 @@ dg_status loss_grad(dg_mlp *m, const float *X, const float *T, int B, float *gra
 
 // ---- chunked path: every block takes whole 32-row chunks of the batch
 
+// The two kernels of a chunked step follow one another with programmatic
+// stream serialization: the next one's blocks are placed and set up while
+// the last one drains, and wait (griddepcontrol.wait) before they read.
+template <typename... KArgs, typename... Args>
+cudaError_t launch_after(void (*kern)(KArgs...), int grid, int threads, size_t smem, cudaStream_t st, Args... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
+}
+
 int fused_blocks(const dg_mlp *m, int B) { return std::min((B + mlpf::R - 1) / mlpf::R, m->fgrid); }
 
-int reduce_blocks(const dg_mlp *m) { return static_cast<int>((m->nparams + mlpf::RP - 1) / mlpf::RP); }
+int reduce_blocks(const dg_mlp *m) { return (m->fnet.npart + mlpf::RP - 1) / mlpf::RP; }
 
 dg_status fused_forward(dg_mlp *m, const float *X, int B, float *Y)
 {
@@ -448,10 +467,9 @@ dg_status fused_forward(dg_mlp *m, const float *X, int B, float *Y)
 // step (or null): the replayed step's index, advanced by the kernel
 dg_status fused_chunks(dg_mlp *m, const float *X, const float *T, int B, int *step = nullptr)
 {
-    mlpf::mlp_chunk_kernel<true><<<fused_blocks(m, B), mlpf::NT, m->fnet.bytes, m->stream>>>(
-        m->fnet, m->p.ptr, m->wstaged.ptr, X, T, B, nullptr, m->fpart.ptr, m->flpart.ptr, step);
+    M_CUDA(m, launch_after(mlpf::mlp_chunk_kernel<true>, fused_blocks(m, B), mlpf::NT, m->fnet.bytes, m->stream, m->fnet,
+                           m->p.ptr, m->wstaged.ptr, X, T, B, nullptr, m->fpart.ptr, m->flpart.ptr, step));
     m->launches += 1;
-    M_CUDA(m, cudaGetLastError());
     return DG_OK;
 }
 
@@ -459,11 +477,10 @@ dg_status fused_loss_grad(dg_mlp *m, const float *X, const float *T, int B, floa
 {
     dg_status st = fused_chunks(m, X, T, B);
     if (st != DG_OK) return st;
-    mlpf::mlp_reduce_kernel<false><<<reduce_blocks(m), mlpf::RP * mlpf::RQ, 0, m->stream>>>(
-        m->fnet, fused_blocks(m, B), m->fpart.ptr, m->flpart.ptr, static_cast<long long>(B) * m->n_out, grad, loss,
-        nullptr, nullptr, nullptr, nullptr, nullptr, mlpf::Adam{});
+    M_CUDA(m, launch_after(mlpf::mlp_reduce_kernel<false>, reduce_blocks(m), mlpf::RP * mlpf::RQ, 0, m->stream, m->fnet,
+                           fused_blocks(m, B), m->fpart.ptr, m->flpart.ptr, static_cast<long long>(B) * m->n_out, grad,
+                           loss, nullptr, nullptr, nullptr, nullptr, nullptr, mlpf::Adam{}));
     m->launches += 1;
-    M_CUDA(m, cudaGetLastError());
     return DG_OK;
 }
 
@@ -476,11 +493,10 @@ dg_status fused_step(dg_mlp *m, const float *X, const float *T, int B, float *lo
     dg_status st = fused_chunks(m, X, T, B, bc ? cnt : nullptr);
     if (st != DG_OK) return st;
     const mlpf::Adam o{lr, 0.9f, 0.999f, 1e-8f, bc1, bc2, bc, cnt, hist};
-    mlpf::mlp_reduce_kernel<true><<<reduce_blocks(m), mlpf::RP * mlpf::RQ, 0, m->stream>>>(
-        m->fnet, fused_blocks(m, B), m->fpart.ptr, m->flpart.ptr, static_cast<long long>(B) * m->n_out, nullptr,
-        loss, m->p.ptr, m->m.ptr, m->v.ptr, m->wstaged.ptr, m->wq.ptr, o);
+    M_CUDA(m, launch_after(mlpf::mlp_reduce_kernel<true>, reduce_blocks(m), mlpf::RP * mlpf::RQ, 0, m->stream, m->fnet,
+                           fused_blocks(m, B), m->fpart.ptr, m->flpart.ptr, static_cast<long long>(B) * m->n_out, nullptr,
+                           loss, m->p.ptr, m->m.ptr, m->v.ptr, m->wstaged.ptr, m->wq.ptr, o));
     m->launches += 1;
-    M_CUDA(m, cudaGetLastError());
     return DG_OK;
 }
 
@@ -618,7 +634,7 @@ dg_status dg_mlp_create(int n_in, int width, int depth, int n_out, int max_batch
             chk(cudaFuncSetAttribute(mlpf::mlp_chunk_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
             chk(cudaFuncSetAttribute(mlpf::mlp_chunk_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
             m->fgrid = std::max(1, std::min(sms, (max_batch + mlpf::R - 1) / mlpf::R));
-            chk(m->fpart.alloc(static_cast<size_t>(m->fgrid) * static_cast<size_t>(m->nparams)));
+            chk(m->fpart.alloc(static_cast<size_t>(m->fgrid) * static_cast<size_t>(m->fnet.npart)));
             chk(m->flpart.alloc(static_cast<size_t>(m->fgrid)));
             chk(m->wstaged.alloc(static_cast<size_t>(m->fnet.nstaged)));
             if (e == cudaSuccess) chk(cudaMemset(m->wstaged.ptr, 0, sizeof(bf16) * m->fnet.nstaged));

@@ -14,9 +14,11 @@
 // of the layer inputs and of W, so nothing is transposed in memory.  The
 // rounding points are those of the layer-by-layer
 // kernels: bf16 inputs and activations, FP32 pre-activations, dz in FP32 and
-// rounded to bf16 for the next products.  The block's weight and bias
-// gradients over its chunks go to its own slice of a workspace, its loss sum
-// to one float.
+// rounded to bf16 for the next products.  The forward pass keeps GELU' of
+// every pre-activation (one error function serves both).  The block's weight
+// and bias gradients over its chunks go to its own slice of a workspace, a
+// weight tile in the order of the accumulators (a 512-byte run per warp
+// store), its loss sum to one float.
 //
 // mlp_reduce_kernel: adds the slices in block order (deterministic) and
 // either returns the gradient and the loss or applies Adam and refreshes the
@@ -52,11 +54,12 @@ struct Net {
     int din[MAXL], dout[MAXL];
     long long woff[MAXL], boff[MAXL], qoff[MAXL];
     long long nparams;
+    int po[MAXL], bo[MAXL], npart;          // slice of a block's gradient: W_l in fragment order, b_l; floats in all
     long long fo[MAXL];                     // element offset of the staged copy of W_l: [kpad(dout)][ldk(din)]
     long long nstaged;                      // elements in the staged copies
     int nbuf;                               // staging buffers (2: the next copy is prefetched)
     unsigned oH[MAXL];                      // bf16 [R][ldk(din[l])]: input of layer l
-    unsigned oZ[MAXL];                      // float [R][zld(dout[l])]: pre-activation of hidden layer l
+    unsigned oZ[MAXL];                      // float [R][zld(dout[l])]: GELU' of hidden layer l's pre-activation
     unsigned oW[2];                         // bf16: staged weight matrices
     unsigned oB;                            // float [nl][maxd]: biases
     unsigned oD16[2];                       // bf16 [R][ldk(maxd)]: dz rounded, two buffers
@@ -93,6 +96,7 @@ inline bool plan(Net &n, int nl, const int *din, const int *dout, const long lon
     };
     size_t wsz = 0;
     long long st = 0;
+    int part = 0;
     for (int l = 0; l < nl; ++l) {
         n.oH[l] = take(sizeof(bf16) * R * ldk(din[l]));
         if (l < nl - 1) n.oZ[l] = take(sizeof(float) * R * zld(dout[l]));
@@ -102,7 +106,14 @@ inline bool plan(Net &n, int nl, const int *din, const int *dout, const long lon
         wsz = w > wsz ? w : wsz;
         n.fo[l] = st;
         st += static_cast<long long>(w);
+        n.po[l] = part;
+        part += kpad(dout[l]) * npad(din[l]);
     }
+    for (int l = 0; l < nl; ++l) {
+        n.bo[l] = part;
+        part += (dout[l] + 3) & ~3;
+    }
+    n.npart = part;
     n.nstaged = st;
     n.oB = take(sizeof(float) * nl * maxd);
     n.oW[0] = take(sizeof(bf16) * wsz);
@@ -123,9 +134,12 @@ inline bool plan(Net &n, int nl, const int *din, const int *dout, const long lon
 
 __device__ __forceinline__ float gelu(float z) { return 0.5f * z * (1.0f + erff(z * 0.70710678118654752f)); }
 
-__device__ __forceinline__ float gelu_grad(float z)
+// GELU and its derivative from one error function
+__device__ __forceinline__ float gelu_both(float z, float &grad)
 {
-    return 0.5f * (1.0f + erff(z * 0.70710678118654752f)) + z * expf(-0.5f * z * z) * 0.39894228040143268f;
+    const float e = 1.0f + erff(z * 0.70710678118654752f);
+    grad = 0.5f * e + z * expf(-0.5f * z * z) * 0.39894228040143268f;
+    return 0.5f * z * e;
 }
 
 __device__ __forceinline__ unsigned smem_u32(const void *p)
@@ -133,7 +147,7 @@ __device__ __forceinline__ unsigned smem_u32(const void *p)
     return static_cast<unsigned>(__cvta_generic_to_shared(p));
 }
 
-// four / two 8x8 bf16 matrices from shared memory, lane i naming row i % 8 of
+// four 8x8 bf16 matrices from shared memory, lane i naming row i % 8 of
 // matrix i / 8; .trans hands out the transposed fragments
 __device__ __forceinline__ void ldsm4(unsigned r[4], const bf16 *p, bool trans)
 {
@@ -145,68 +159,54 @@ __device__ __forceinline__ void ldsm4(unsigned r[4], const bf16 *p, bool trans)
                      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(smem_u32(p)) : "memory");
 }
 
-__device__ __forceinline__ void ldsm2(unsigned r[2], const bf16 *p, bool trans)
-{
-    if (trans)
-        asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];\n"
-                     : "=r"(r[0]), "=r"(r[1]) : "r"(smem_u32(p)) : "memory");
-    else
-        asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0,%1}, [%2];\n"
-                     : "=r"(r[0]), "=r"(r[1]) : "r"(smem_u32(p)) : "memory");
-}
-
 // Block-wide C = A B over shared-memory bf16 operands, with FP32 sums.
 // AT = false: A stored [m][k] (row stride lda); AT = true: stored [k][m].
 // BT = false: B stored [n][k] (row stride ldb); BT = true: stored [k][n].
 // M = 16 Mt, N = 8 Nt, K = 16 Ks, every stored row 16-byte aligned and the
 // operands zero past their extents up to those multiples.  Each warp takes a
-// 16-row strip of up to NJ 8-column tiles at a time and hands the results
-// to epi(row, col, v(row, col), v(row, col + 1)) for even col.  Jobs of NJ
-// tiles keep every warp of the block busy on the smallest products.
+// 16-row strip of NJ = 2 8-column tiles at a time (the second may be past
+// the extent: its fragments repeat the first's) and hands the accumulators
+// to epi(mt, nt, acc): acc[0, 1] row 16 mt + g, columns 8 nt + 2 t, + 1;
+// acc[2, 3] row + 8; lane = 4 g + t.  Jobs of two tiles keep every warp of
+// the block busy on the smallest products, and their B fragments of a k-step
+// are one four-matrix load.
 template <bool AT, bool BT, typename Epi>
 __device__ __forceinline__ void bgemm(const bf16 *A, int lda, const bf16 *B, int ldb, int Mt, int Nt, int Ks, Epi epi)
 {
+    static_assert(NJ == 2, "one four-matrix load holds the B fragments of two column tiles");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int g = lane >> 2, t = lane & 3, rr = lane & 7, q = lane >> 3;
+    const int rr = lane & 7, q = lane >> 3;
     const int Nq = (Nt + NJ - 1) / NJ;
     for (int job = warp; job < Mt * Nq; job += NT / 32) {
         const int mt = job / Nq, nq = job - (job / Nq) * Nq;
+        const int n0 = NJ * nq, n1 = min(n0 + 1, Nt - 1), nb = (q & 2) ? n1 : n0;
         float acc[NJ][4];
 #pragma unroll
         for (int j = 0; j < NJ; ++j)
 #pragma unroll
             for (int r = 0; r < 4; ++r) acc[j][r] = 0.f;
+        // matrix q of the A fragment: rows 16 mt + 8 (q & 1), columns k + 8 (q >> 1);
+        // of the B fragments: k + 8 (q & 1), column tile nb
+        const bf16 *pa = AT ? A + (rr + 8 * (q >> 1)) * lda + 16 * mt + 8 * (q & 1)
+                            : A + (16 * mt + rr + 8 * (q & 1)) * lda + 8 * (q >> 1);
+        const bf16 *pb = BT ? B + (rr + 8 * (q & 1)) * ldb + 8 * nb : B + (8 * nb + rr) * ldb + 8 * (q & 1);
+        const int sa = AT ? 16 * lda : 16, sb = BT ? 16 * ldb : 16;
+#pragma unroll 4
         for (int ks = 0; ks < Ks; ++ks) {
-            const int k0 = 16 * ks, m0 = 16 * mt;
-            unsigned a[4];
-            // matrix q of the A fragment: rows m0 + 8 (q & 1), columns k0 + 8 (q >> 1)
-            if (AT) ldsm4(a, A + (k0 + rr + 8 * (q >> 1)) * lda + m0 + 8 * (q & 1), true);
-            else ldsm4(a, A + (m0 + rr + 8 * (q & 1)) * lda + k0 + 8 * (q >> 1), false);
+            unsigned a[4], b[4];
+            ldsm4(a, pa + ks * sa, AT);
+            ldsm4(b, pb + ks * sb, BT);
 #pragma unroll
-            for (int j = 0; j < NJ; ++j) {
-                const int nt = NJ * nq + j;
-                if (nt < Nt) {
-                    // matrix q & 1 of the B fragment: k0 + 8 (q & 1)
-                    unsigned b[2];
-                    if (BT) ldsm2(b, B + (k0 + rr + 8 * (q & 1)) * ldb + 8 * nt, true);
-                    else ldsm2(b, B + (8 * nt + rr) * ldb + k0 + 8 * (q & 1), false);
-                    asm volatile(
-                        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 "
-                        "{%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};\n"
-                        : "+f"(acc[j][0]), "+f"(acc[j][1]), "+f"(acc[j][2]), "+f"(acc[j][3])
-                        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
-                }
-            }
+            for (int j = 0; j < NJ; ++j)
+                asm volatile(
+                    "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 "
+                    "{%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};\n"
+                    : "+f"(acc[j][0]), "+f"(acc[j][1]), "+f"(acc[j][2]), "+f"(acc[j][3])
+                    : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[2 * j]), "r"(b[2 * j + 1]));
         }
-        // acc[j][0, 1]: row g, columns 2 t, 2 t + 1 of tile NJ nq + j; acc[j][2, 3]: row g + 8
 #pragma unroll
-        for (int j = 0; j < NJ; ++j) {
-            const int nt = NJ * nq + j;
-            if (nt < Nt) {
-                epi(16 * mt + g, 8 * nt + 2 * t, acc[j][0], acc[j][1]);
-                epi(16 * mt + g + 8, 8 * nt + 2 * t, acc[j][2], acc[j][3]);
-            }
-        }
+        for (int j = 0; j < NJ; ++j)
+            if (n0 + j < Nt) epi(mt, n0 + j, acc[j]);
     }
 }
 
@@ -236,23 +236,28 @@ __device__ __forceinline__ void zero_cols(bf16 *D, int ls, int c0, int c1)
 // gradient; the block's slice of part [gridDim.x][nparams] and lpart
 // [gridDim.x] receive its sums over its chunks.  step (graph replay, or
 // null): the step index, advanced here by one (it starts a call at -1), so
-// that the reduction kernel of the same step reads it.
+// that the reduction kernel of the same step reads it.  P and WS are written
+// by the kernel before this one, so they are not declared read-only.
 template <bool TRAIN>
-__global__ void __launch_bounds__(NT) mlp_chunk_kernel(Net net, const float *__restrict__ P, const bf16 *__restrict__ WS,
+__global__ void __launch_bounds__(NT) mlp_chunk_kernel(Net net, const float *P, const bf16 *WS,
                                                        const float *__restrict__ X, const float *__restrict__ T, int B,
                                                        float *__restrict__ Y, float *__restrict__ part,
                                                        float *__restrict__ lpart, int *step)
 {
     extern __shared__ __align__(16) unsigned char sm[];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (step && blockIdx.x == 0 && tid == 0) *step += 1;
     const int nl = net.nl, n_in = net.din[0], maxd = net.maxd, LDD = ldk(maxd), ZD = zld(maxd);
     float *D32 = reinterpret_cast<float *>(sm + net.oD32);
-    const long long NP = net.nparams;
+    const int gq = lane >> 2, tq = 2 * (lane & 3);      // row and column of the lane in an accumulator tile
+    float *slice = part + static_cast<long long>(blockIdx.x) * net.npart;
     const float sc = 2.0f / static_cast<float>(static_cast<long long>(B) * net.dout[nl - 1]);
     // the padding columns of the hidden activations are never written: clear once
     for (int l = 1; l < nl; ++l) zero_cols(reinterpret_cast<bf16 *>(sm + net.oH[l]), ldk(net.din[l]), net.din[l],
                                             kpad(net.din[l]));
+    // what the step before this one wrote is read and advanced from here on
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+    if (step && blockIdx.x == 0 && tid == 0) *step += 1;
     float *sB = reinterpret_cast<float *>(sm + net.oB);
     for (int l = 0; l < nl; ++l)
         for (int c = tid; c < net.dout[l]; c += NT) sB[l * maxd + c] = P[net.boff[l] + c];
@@ -318,25 +323,27 @@ __global__ void __launch_bounds__(NT) mlp_chunk_kernel(Net net, const float *__r
                 bf16 *Hn = reinterpret_cast<bf16 *>(sm + net.oH[l + 1]);
                 const int ln = ldk(dn), zs = zld(dn);
                 bgemm<false, false>(Hl, ldk(di), Ws, ldk(di), R / 16, npad(dn) / 8, kpad(di) / 16,
-                                    [&](int r, int c, float v0, float v1) {
-                                        if (c < dn) {
-                                            const float z = v0 + bias[c];
-                                            Z[r * zs + c] = z;
-                                            Hn[r * ln + c] = __float2bfloat16_rn(gelu(z));
-                                        }
-                                        if (c + 1 < dn) {
-                                            const float z = v1 + bias[c + 1];
-                                            Z[r * zs + c + 1] = z;
-                                            Hn[r * ln + c + 1] = __float2bfloat16_rn(gelu(z));
+                                    [&](int mt, int nt, const float *v) {
+                                        const int c = 8 * nt + tq;
+#pragma unroll
+                                        for (int e = 0; e < 4; ++e) {
+                                            const int r = 16 * mt + gq + 8 * (e >> 1), cc = c + (e & 1);
+                                            if (cc >= dn) continue;
+                                            const float z = v[e] + bias[cc];
+                                            float h;
+                                            if (TRAIN) h = gelu_both(z, Z[r * zs + cc]);
+                                            else h = gelu(z);
+                                            Hn[r * ln + cc] = __float2bfloat16_rn(h);
                                         }
                                     });
             } else {
                 bgemm<false, false>(Hl, ldk(di), Ws, ldk(di), R / 16, npad(dn) / 8, kpad(di) / 16,
-                                    [&](int r, int c0, float v0, float v1) {
-                                        for (int e = 0; e < 2; ++e) {
-                                            const int c = c0 + e;
-                                            if (c >= dn) break;
-                                            const float y = (e ? v1 : v0) + bias[c];
+                                    [&](int mt, int nt, const float *v) {
+#pragma unroll
+                                        for (int e = 0; e < 4; ++e) {
+                                            const int r = 16 * mt + gq + 8 * (e >> 1), c = 8 * nt + tq + (e & 1);
+                                            if (c >= dn) continue;
+                                            const float y = v[e] + bias[c];
                                             if (!TRAIN) {
                                                 if (r < nr) Y[static_cast<long long>(r0 + r) * dn + c] = y;
                                                 continue;
@@ -357,10 +364,13 @@ __global__ void __launch_bounds__(NT) mlp_chunk_kernel(Net net, const float *__r
             const int di = net.din[l], dn = net.dout[l];
             const bf16 *D16 = reinterpret_cast<const bf16 *>(sm + net.oD16[l & 1]);
             const bf16 *Hl = reinterpret_cast<const bf16 *>(sm + net.oH[l]);
-            float *pb = part + static_cast<long long>(blockIdx.x) * NP + net.boff[l];
+            float *pb = slice + net.bo[l];
             for (int c = tid; c < dn; c += NT) {
-                float s = 0.f;
-                for (int r = 0; r < R; ++r) s += D32[r * ZD + c];
+                float d[R], s = 0.f;
+#pragma unroll
+                for (int r = 0; r < R; ++r) d[r] = D32[r * ZD + c];      // the loads together, the sum in row order
+#pragma unroll
+                for (int r = 0; r < R; ++r) s += d[r];
                 pb[c] = first ? s : pb[c] + s;
             }
             const bf16 *Ws = nullptr;
@@ -371,30 +381,33 @@ __global__ void __launch_bounds__(NT) mlp_chunk_kernel(Net net, const float *__r
             __syncthreads();
             // dW_l += dz_l^T H_l over the chunk's rows: both operands stored
             // with the rows of the chunk as K
-            float *pw = part + static_cast<long long>(blockIdx.x) * NP + net.woff[l];
-            bgemm<true, true>(D16, LDD, Hl, ldk(di), kpad(dn) / 16, npad(di) / 8, R / 16,
-                              [&](int r, int c, float v0, float v1) {
-                                  if (r >= dn) return;
-                                  float *q = pw + static_cast<long long>(r) * di + c;
-                                  if (c < di) q[0] = first ? v0 : q[0] + v0;
-                                  if (c + 1 < di) q[1] = first ? v1 : q[1] + v1;
-                              });
+            // in the accumulators' own order, 16 bytes per lane: a tile is one
+            // 512-byte run (rows of W_l would be 8-byte pieces)
+            float4 *pw = reinterpret_cast<float4 *>(slice + net.po[l]) + lane;
+            const int Nt = npad(di) / 8;
+            bgemm<true, true>(D16, LDD, Hl, ldk(di), kpad(dn) / 16, Nt, R / 16, [&](int mt, int nt, const float *v) {
+                float4 *q = pw + (mt * Nt + nt) * 32;
+                float4 o = make_float4(v[0], v[1], v[2], v[3]);
+                if (!first) {
+                    const float4 u = *q;
+                    o = make_float4(u.x + o.x, u.y + o.y, u.z + o.z, u.w + o.w);
+                }
+                *q = o;
+            });
             if (l > 0) {
                 // dz_{l-1} = (dz_l W_l) * GELU'(z_{l-1}), W_l stored [k = out][n = in]
                 const float *Zp = reinterpret_cast<const float *>(sm + net.oZ[l - 1]);
                 bf16 *Dn = reinterpret_cast<bf16 *>(sm + net.oD16[(l - 1) & 1]);
                 const int zs = zld(di);
                 bgemm<false, true>(D16, LDD, Ws, ldk(di), R / 16, npad(di) / 8, kpad(dn) / 16,
-                                   [&](int r, int c, float v0, float v1) {
-                                       if (c < di) {
-                                           const float dz = v0 * gelu_grad(Zp[r * zs + c]);
+                                   [&](int mt, int nt, const float *v) {
+#pragma unroll
+                                       for (int e = 0; e < 4; ++e) {
+                                           const int r = 16 * mt + gq + 8 * (e >> 1), c = 8 * nt + tq + (e & 1);
+                                           if (c >= di) continue;
+                                           const float dz = v[e] * Zp[r * zs + c];
                                            D32[r * ZD + c] = dz;
                                            Dn[r * LDD + c] = __float2bfloat16_rn(dz);
-                                       }
-                                       if (c + 1 < di) {
-                                           const float dz = v1 * gelu_grad(Zp[r * zs + c + 1]);
-                                           D32[r * ZD + c + 1] = dz;
-                                           Dn[r * LDD + c + 1] = __float2bfloat16_rn(dz);
                                        }
                                    });
             }
@@ -424,16 +437,14 @@ struct Adam {
 };
 
 // weight i (a parameter index) rounded to bf16 into the staged copy WS
-// (W_l at [k][n] with padded rows) and, if wq is set, the row-major copy
-__device__ __forceinline__ void put_weight(const Net &net, long long i, float w, bf16 *WS, bf16 *wq)
+// (W_l at [k][n] with padded rows)
+__device__ __forceinline__ void put_weight(const Net &net, long long i, float w, bf16 *WS)
 {
     for (int l = 0; l < net.nl; ++l) {
         if (i < net.woff[l] || i >= net.boff[l]) continue;
-        const bf16 b = __float2bfloat16_rn(w);
         const long long j = i - net.woff[l];
         const int di = net.din[l], k = static_cast<int>(j / di), n = static_cast<int>(j - (j / di) * di);
-        WS[net.fo[l] + static_cast<long long>(k) * ldk(di) + n] = b;
-        if (wq) wq[net.qoff[l] + j] = b;
+        WS[net.fo[l] + static_cast<long long>(k) * ldk(di) + n] = __float2bfloat16_rn(w);
     }
 }
 
@@ -443,36 +454,61 @@ __global__ void mlp_stage_copies_kernel(Net net, const float *__restrict__ p, bf
 {
     for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < net.nparams;
          i += static_cast<long long>(gridDim.x) * blockDim.x)
-        put_weight(net, i, p[i], WS, nullptr);
+        put_weight(net, i, p[i], WS);
 }
 
-constexpr int RP = 64;          // parameters per block of the reduction
-constexpr int RQ = 4;           // partial sums per parameter (RP x RQ threads)
+constexpr int RP = 64;          // slice values per block of the reduction
+constexpr int RQ = 4;           // partial sums per value (RP x RQ threads)
+constexpr int LB = 128;         // loss sums read at a time
 
-// Sum of the G slices of every parameter's gradient (quarter q of the
-// slices by threads q, then the four quarters in order: a fixed order), and
-// of the G loss sums.  ADAM = false: grad and loss out.  ADAM = true: loss
-// out, Adam step on p with moments m, v, and the bf16 copies of every
-// weight.  Blocks of RP x RQ threads, RP parameters each.
+// Sum of the G slices of every parameter's gradient (quarter q of the slices
+// by threads q, then the four quarters in order: a fixed order), and of the G
+// loss sums in block order.  ADAM = false: grad and loss out.  ADAM = true:
+// loss out, Adam step on p with moments m, v, and the bf16 copies of every
+// weight.  Bound by the G slices, 22 MB from L2 at B = 4096: a thread per
+// value and quarter, so that enough reads are in flight.
 template <bool ADAM>
 __global__ void __launch_bounds__(RP * RQ)
-mlp_reduce_kernel(Net net, int G, const float *__restrict__ part, const float *__restrict__ lpart, long long nsum,
-                  float *__restrict__ grad, float *__restrict__ loss, float *p, float *m, float *v, bf16 *WS,
-                  bf16 *wq, Adam o)
+mlp_reduce_kernel(Net net, int G, const float *part, const float *lpart, long long nsum, float *grad, float *loss,
+                  float *p, float *m, float *v, bf16 *WS, bf16 *wq, Adam o)
 {
     __shared__ float red[RQ][RP];
-    const long long NP = net.nparams;
     const int j = threadIdx.x % RP, qr = threadIdx.x / RP;
-    const long long i = static_cast<long long>(blockIdx.x) * RP + j;
+    const int at = blockIdx.x * RP + j;
+    // the value's parameter: row r and column c of layer l's W, or bias r of
+    // layer l; none where the slice is padding
+    int l = 0, r = 0, c = 0;
+    bool any = false;
+    const bool weight = at < net.bo[0];
+    long long i = 0;
+    if (at < net.npart) {
+        if (weight) {
+            while (l + 1 < net.nl && at >= net.po[l + 1]) ++l;
+            const int w = at - net.po[l], lane = (w & 127) >> 2, tile = w >> 7, Nt = npad(net.din[l]) / 8;
+            const int mt = tile / Nt, nt = tile - (tile / Nt) * Nt;
+            r = 16 * mt + (lane >> 2) + 8 * ((w >> 1) & 1);
+            c = 8 * nt + 2 * (lane & 3) + (w & 1);
+            any = r < net.dout[l] && c < net.din[l];
+            i = net.woff[l] + static_cast<long long>(r) * net.din[l] + c;
+        } else {
+            while (l + 1 < net.nl && at >= net.bo[l + 1]) ++l;
+            r = at - net.bo[l];
+            any = r < net.dout[l];
+            i = net.boff[l] + r;
+        }
+    }
     const int qg = (G + RQ - 1) / RQ, c0 = qr * qg, c1 = min(G, c0 + qg);
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
     float gq = 0.f;
-    if (i < NP) {
-#pragma unroll 8
-        for (int c = c0; c < c1; ++c) gq += part[static_cast<long long>(c) * NP + i];
+    if (any) {
+        const float *src = part + at;
+#pragma unroll 16
+        for (int k = c0; k < c1; ++k) gq += __ldcg(src + static_cast<long long>(k) * net.npart);
     }
     red[qr][j] = gq;
     __syncthreads();
-    if (qr == 0 && i < NP) {
+    if (qr == 0 && any) {
         const float gi = (red[0][j] + red[1][j]) + (red[2][j] + red[3][j]);
         if (!ADAM) {
             grad[i] = gi;
@@ -483,20 +519,38 @@ mlp_reduce_kernel(Net net, int G, const float *__restrict__ part, const float *_
                 bc1 = o.bc[2 * k];
                 bc2 = o.bc[2 * k + 1];
             }
-            const float mi = o.b1 * m[i] + (1.0f - o.b1) * gi;
-            const float vi = o.b2 * v[i] + (1.0f - o.b2) * gi * gi;
+            // contracted one way, whatever the compiler would choose: a bit here
+            // is a bit in every later step
+            const float mi = fmaf(1.0f - o.b1, gi, __fmul_rn(o.b1, m[i]));
+            const float vi = fmaf(__fmul_rn(1.0f - o.b2, gi), gi, __fmul_rn(o.b2, v[i]));
             m[i] = mi;
             v[i] = vi;
             const float pi = p[i] - o.lr * (mi / bc1) / (sqrtf(vi / bc2) + o.eps);
             p[i] = pi;
-            put_weight(net, i, pi, WS, wq);
+            if (weight) {
+                // the bf16 copies: W_l at [row][column] with padded rows, and row-major
+                const bf16 b = __float2bfloat16_rn(pi);
+                WS[net.fo[l] + static_cast<long long>(r) * ldk(net.din[l]) + c] = b;
+                if (wq) wq[net.qoff[l] + i - net.woff[l]] = b;
+            }
         }
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        float s = 0.f;
-        for (int c = 0; c < G; ++c) s += lpart[c];
-        *loss = s / static_cast<float>(nsum);
-        if (ADAM && o.bc && o.hist) o.hist[*o.cnt] = s / static_cast<float>(nsum);
+    if (blockIdx.x == 0) {
+        // read by the block, added by one thread in block order (a chain of
+        // dependent reads by that thread took longer than the rest)
+        __shared__ float sl[LB];
+        float t = 0.f;
+        for (int k0 = 0; k0 < G; k0 += LB) {
+            __syncthreads();
+            if (threadIdx.x < LB && k0 + threadIdx.x < G) sl[threadIdx.x] = __ldcg(lpart + k0 + threadIdx.x);
+            __syncthreads();
+            if (threadIdx.x == 0)
+                for (int k = 0; k < min(LB, G - k0); ++k) t += sl[k];
+        }
+        if (threadIdx.x == 0) {
+            *loss = t / static_cast<float>(nsum);
+            if (ADAM && o.bc && o.hist) o.hist[*o.cnt] = t / static_cast<float>(nsum);
+        }
     }
 }
 
