@@ -47,6 +47,7 @@
 // and 6 (Np = 21, 28) the node rows span two 16-row tiles (MT = 2), so a lane
 // holds one node per tile, and the contractions take up to four k-steps.
 #pragma once
+#include "bulk.cuh"
 #include "dg_stage_mixed.cuh"
 #include "pair2.cuh"
 
@@ -85,6 +86,10 @@ struct ShapeTC {
     // lane): measured 3.5 % faster per step at p = 6 and 0.3 % at p = 5, 0.8 %
     // slower at p = 4 on 128^2 quads (neutral on 512^2), so from p = 5 on
     static constexpr bool TILE_BULK = MT > 1;
+    // connectivity (and the batch's tile table) copied one tile ahead: -2.4 %
+    // per step at p = 4 on 512^2 quads (489 -> 478 us a stage), -1 % on 128^2,
+    // -6 % on 16^2, -1 % at p = 5; +2 % at p = 6, whose registers are full
+    static constexpr bool AHEAD = P <= 5;
 };
 
 // operator table: the MMA fragments (ShapeTC<P>::NFRAG_ALL float4), then
@@ -103,8 +108,9 @@ struct TcLayout {
     static constexpr size_t hBar = hD + al(sizeof(float2) * Np * S::DS);   // mbarrier of the operator copy
     static constexpr size_t header = hBar + 16;
     // one region per warp
-    static constexpr size_t oConn = 0;                                      // int4 [WE]
-    static constexpr size_t oGeo = oConn + al(16 * WE);                     // float [WE][16]
+    static constexpr size_t oConn = 0;                                      // int4 [2][WE]: this tile's, the next one's
+    static constexpr size_t oTile = oConn + al(16 * 2 * WE);                // int4 [4]: batch tile table entries
+    static constexpr size_t oGeo = oTile + 64;                              // float [WE][16]
     static constexpr size_t oNGeo = oGeo + al(64 * WE);                     // float [3 WE][16]
     static constexpr size_t oU = oNGeo + al(64 * 3 * WE);                   // float4 [WE][US]
     static constexpr size_t oN = oU + al(16 * WE * S::US);                  // float4 [3 WE][UN]
@@ -119,41 +125,6 @@ struct TcLayout {
     static constexpr size_t warp = oBar + 16;
     static constexpr size_t bytes = header + S::NW * warp;
 };
-
-// Bulk copies (the tensor memory accelerator's 1-D form) into shared memory,
-// completing on an mbarrier: the warp's own tile and the operator table.
-__device__ __forceinline__ void mbar_init1(unsigned bar)
-{
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ void mbar_expect(unsigned bar, unsigned bytes)
-{
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-// 16-byte aligned addresses, a multiple of 16 bytes
-__device__ __forceinline__ void bulk_g2s(unsigned dst, const void *src, unsigned bytes, unsigned bar)
-{
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                 ::"r"(dst), "l"(src), "r"(bytes), "r"(bar)
-                 : "memory");
-}
-// bounded wait for phase `parity` of an mbarrier; false if it gave up
-__device__ __forceinline__ bool mbar_wait_bounded(unsigned bar, unsigned parity, unsigned limit)
-{
-    for (unsigned it = 0;; ++it) {
-        unsigned ok;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(ok)
-            : "r"(bar), "r"(parity)
-            : "memory");
-        if (ok) return true;
-        if (it >= limit) return false;
-        __nanosleep(100);
-    }
-}
 
 __device__ __forceinline__ void mma_tf32(float c[4], const float4 &a, float b0, float b1)
 {
