@@ -36,19 +36,28 @@ struct Group {
     long long lam_base = 0;          // first entry in the batch's Lambda_K array
     int wall_base = 0;               // first entry in the batch's wall partials
     int nwall = 0;
-    long long ntiles = 0, ntiles2 = 0, ntiles3 = 0;
+    long long ntiles = 0, ntiles3 = 0;
     dg::LaunchShape shape, shape2;   // one / two nodes per thread
     dg::LaunchShape shape3;          // tensor-core warp tiles (p <= 6)
     bool has_tc = false;
     int variant = 1;
-    float t_tc = 0.f;                // the tuner's time of the tensor-core shape (ms, 3 launches), 0 if not timed
+    float t_tc = 0.f;                // the tuner's time of the tensor-core shape (ms, a step), 0 if not timed
     dg::LaunchShape fshape;          // fused steps: cooperative launch of the chosen shape
     int fshape_variant = 0;
-    DevBuf<unsigned> bar;            // fused steps: barrier words of this group (+ tile counters)
+    DevBuf<unsigned> bar;            // barrier words of this group (+ fused steps: tile counters)
+    // two-node shape: symmetric operator rows, trace records and divergence between stages
+    DevBuf<float> sym32;
+    DevBuf<int> symn32;
+    DevBuf<float4> fd32, rv32;
+    dg::Stage2Args stage2(int s) const
+    {
+        return dg::stage2_args(sym32.ptr, symn32.ptr, fd32.ptr, rv32.ptr, elem_case.ptr,
+                               static_cast<size_t>(K) * 3 * ops.Nfp, s);
+    }
     DevBuf<double> K0a, K0b, K1, geo64, Dr64, Ds64, wface, fxy;
     DevBuf<float> geo32, ops32, P0a, P0b;
     DevBuf<float4> S0a, S0b;
-    DevBuf<int4> conn, tiles, tiles2, tiles3;
+    DevBuf<int4> conn, tiles, tiles3;
     DevBuf<float> tcfrag;            // operator table of the tensor-core shape
     DevBuf<int> fmask, elem_case;
     DevBuf<int2> walls;
@@ -336,14 +345,16 @@ dg_status enqueue_step(dg_batch *b, double cfl, double *hist, int rows)
             sp.bar_limit = b->bar_limit;
             if (b->fused) {
                 // the five stages in one cooperative launch (grid barriers between stages)
-                sp.tiles = (g.variant == 3) ? g.tiles3.ptr : (g.variant == 2) ? g.tiles2.ptr : g.tiles.ptr;
-                sp.ntiles = (g.variant == 3) ? g.ntiles3 : (g.variant == 2) ? g.ntiles2 : g.ntiles;
+                sp.tiles = (g.variant == 3) ? g.tiles3.ptr : g.tiles.ptr;
+                sp.ntiles = (g.variant == 3) ? g.ntiles3 : g.ntiles;
                 if (g.variant == 3) sp.ops = g.tcfrag.ptr;
                 if (g.fshape_variant != g.variant) {
                     if (g.variant == 3)
                         B_CUDA(b, dg::stage_shape_tc(g.p, sp.ntiles, true, true, g.fshape));
+                    else if (g.variant == 2)
+                        B_CUDA(b, dg::stage_shape_mixed2(g.p, g.K, true, true, g.fshape));
                     else
-                        B_CUDA(b, dg::stage_shape_mixed_fused(g.p, g.variant, true, sp.ntiles, g.fshape));
+                        B_CUDA(b, dg::stage_shape_mixed_fused(g.p, true, sp.ntiles, g.fshape));
                     g.fshape_variant = g.variant;
                 }
                 for (int i = 0; i < 5; ++i) {
@@ -354,6 +365,8 @@ dg_status enqueue_step(dg_batch *b, double cfl, double *hist, int rows)
                 B_CUDA(b, cudaMemsetAsync(g.bar.ptr, 0, 2 * sizeof(unsigned), b->stream));
                 if (g.variant == 3)
                     B_CUDA(b, dg::launch_stage_tc(g.p, true, true, g.fshape, sp, ph32, b->stream));
+                else if (g.variant == 2)
+                    B_CUDA(b, dg::launch_stage_mixed2(g.p, true, true, g.fshape, sp, g.stage2(0), ph32, b->stream));
                 else
                     B_CUDA(b, dg::launch_stage_mixed_fused(g.p, true, g.fshape, sp, ph32, b->stream));
             } else if (g.variant == 3) {
@@ -362,9 +375,8 @@ dg_status enqueue_step(dg_batch *b, double cfl, double *hist, int rows)
                 sp.ops = g.tcfrag.ptr;
                 B_CUDA(b, dg::launch_stage_tc(g.p, true, false, g.shape3, sp, ph32, b->stream));
             } else if (g.variant == 2) {
-                sp.tiles = g.tiles2.ptr;
-                sp.ntiles = g.ntiles2;
-                B_CUDA(b, dg::launch_stage_mixed2(g.p, true, g.shape2, sp, ph32, b->stream));
+                sp.bar = g.bar.ptr;
+                B_CUDA(b, dg::launch_stage_mixed2(g.p, true, false, g.shape2, sp, g.stage2(s), ph32, b->stream));
             } else {
                 sp.tiles = g.tiles.ptr;
                 sp.ntiles = g.ntiles;
@@ -378,66 +390,66 @@ dg_status enqueue_step(dg_batch *b, double cfl, double *hist, int rows)
 }
 
 // First run: per degree group, time every available stage-kernel shape on
-// the current states in residual-only launches (into a scratch array) and
-// keep the fastest.
+// the current states and keep the fastest for a step: a first stage untimed,
+// one timed, three inner ones.  Before a step the register and the other state
+// buffers hold nothing that is read again.
 dg_status tune_groups(dg_batch *b)
 {
     if (b->tuned) return DG_OK;
     const dg::Phys<float> ph32 = phys_of<float>(b->prm);
     // events destroyed on every return path
     struct Events {
-        cudaEvent_t e[2] = {nullptr, nullptr};
+        cudaEvent_t e[3] = {nullptr, nullptr, nullptr};
         ~Events()
         {
             for (auto &x : e)
                 if (x) cudaEventDestroy(x);
         }
     } ev;
-    B_CUDA(b, cudaEventCreate(&ev.e[0]));
-    B_CUDA(b, cudaEventCreate(&ev.e[1]));
-    cudaEvent_t e0 = ev.e[0], e1 = ev.e[1];
+    for (auto &e : ev.e) B_CUDA(b, cudaEventCreate(&e));
     for (auto &g : b->groups) {
         if (b->variant_req != 0) {
             // the tensor-core shape covers p <= 6; other groups would take the two-node shape
             g.variant = (b->variant_req == 3 && !g.has_tc) ? 2 : b->variant_req;
             continue;
         }
-        DevBuf<double> scratch;
-        B_CUDA(b, scratch.alloc(static_cast<size_t>(g.K) * 4 * g.ops.Np));
         float best = 0.f;
         for (int v = 1; v <= 3; ++v) {
             if (v == 3 && !g.has_tc) continue;
             dg::StageParams sp{};
             const bool a = b->cur_is_a;
             sp.K0in = a ? g.K0a.ptr : g.K0b.ptr;
+            sp.K0out = a ? g.K0b.ptr : g.K0a.ptr;
             sp.K1 = g.K1.ptr;
-            sp.Rout = scratch.ptr;
             sp.geo = g.geo32.ptr;
             sp.conn = g.conn.ptr;
             sp.ops = g.ops32.ptr;
             sp.fmask = g.fmask.ptr;
             sp.Sin = a ? g.S0a.ptr : g.S0b.ptr;
             sp.Pin = a ? g.P0a.ptr : g.P0b.ptr;
+            sp.Sout = a ? g.S0b.ptr : g.S0a.ptr;
+            sp.Pout = a ? g.P0b.ptr : g.P0a.ptr;
             sp.K = g.K;
+            sp.A = dg::kRkA[1];
+            sp.B = dg::kRkB[1];
             sp.gm1 = b->prm.gamma - 1.0;
             sp.sig_fac = sigma_factor(b->prm);
-            sp.mode = dg::STAGE_RHS_ONLY;
-            sp.first_stage = 1;
+            sp.mode = dg::STAGE_UPDATE;
             sp.cases = b->dcases.ptr;
             sp.bar_err = b->bar_err.ptr;
             sp.bar_limit = b->bar_limit;
-            float ms = 0.f;
             for (int rep = 0; rep < 5; ++rep) {
-                if (rep == 2) B_CUDA(b, cudaEventRecord(e0, b->stream));
+                if (rep == 1 || rep == 2) B_CUDA(b, cudaEventRecord(ev.e[rep - 1], b->stream));
+                const int s = rep == 0 ? 0 : rep - 1;
+                sp.first_stage = s == 0;
                 if (v == 3) {
                     sp.tiles = g.tiles3.ptr;
                     sp.ntiles = g.ntiles3;
                     sp.ops = g.tcfrag.ptr;
                     B_CUDA(b, dg::launch_stage_tc(g.p, true, false, g.shape3, sp, ph32, b->stream));
                 } else if (v == 2) {
-                    sp.tiles = g.tiles2.ptr;
-                    sp.ntiles = g.ntiles2;
-                    B_CUDA(b, dg::launch_stage_mixed2(g.p, true, g.shape2, sp, ph32, b->stream));
+                    sp.bar = g.bar.ptr;
+                    B_CUDA(b, dg::launch_stage_mixed2(g.p, true, false, g.shape2, sp, g.stage2(s), ph32, b->stream));
                 } else {
                     sp.tiles = g.tiles.ptr;
                     sp.ntiles = g.ntiles;
@@ -445,9 +457,12 @@ dg_status tune_groups(dg_batch *b)
                 }
                 b->launches += 1;
             }
-            B_CUDA(b, cudaEventRecord(e1, b->stream));
-            B_CUDA(b, cudaEventSynchronize(e1));
-            B_CUDA(b, cudaEventElapsedTime(&ms, e0, e1));
+            float first = 0.f, inner = 0.f;
+            B_CUDA(b, cudaEventRecord(ev.e[2], b->stream));
+            B_CUDA(b, cudaEventSynchronize(ev.e[2]));
+            B_CUDA(b, cudaEventElapsedTime(&first, ev.e[0], ev.e[1]));
+            B_CUDA(b, cudaEventElapsedTime(&inner, ev.e[1], ev.e[2]));
+            const float ms = first + 4.0f / 3.0f * inner;
             if (v == 3) g.t_tc = ms;
             if (v == 1 || ms < best) {
                 best = ms;
@@ -518,12 +533,12 @@ dg_status dg_batch_create(const dg_params *common, int ncases, const dg_case *ca
         g.p = degrees[gi];
         if (!dg::build_reference_operators(g.p, g.ops)) return bail(DG_EINVAL);
         const int Np = g.ops.Np, Nfp = g.ops.Nfp, NF = 3 * Nfp;
-        const int E = dg::stage_tile_elems(g.p), E2 = dg::stage_tile_elems2(g.p), E3 = dg::stage_tile_elems_tc();
+        const int E = dg::stage_tile_elems(g.p), E3 = dg::stage_tile_elems_tc();
         std::vector<double> geo;
         std::vector<int4> conn;
         std::vector<int2> walls;
         std::vector<double> wxy;
-        std::vector<int4> tiles, tiles2, tiles3;
+        std::vector<int4> tiles, tiles3;
         std::vector<int> ecase;
         g.lam_base = lam_total;
         g.wall_base = wall_total;
@@ -561,9 +576,6 @@ dg_status dg_batch_create(const dg_params *common, int ncases, const dg_case *ca
             for (long long k0 = 0; k0 < c.K; k0 += E)
                 tiles.push_back(make_int4(static_cast<int>(off + k0), static_cast<int>(std::min<long long>(E, c.K - k0)),
                                           i, 0));
-            for (long long k0 = 0; k0 < c.K; k0 += E2)
-                tiles2.push_back(make_int4(static_cast<int>(off + k0),
-                                           static_cast<int>(std::min<long long>(E2, c.K - k0)), i, 0));
             for (long long k0 = 0; k0 < c.K; k0 += E3)
                 tiles3.push_back(make_int4(static_cast<int>(off + k0),
                                            static_cast<int>(std::min<long long>(E3, c.K - k0)), i, 0));
@@ -581,7 +593,6 @@ dg_status dg_batch_create(const dg_params *common, int ncases, const dg_case *ca
         }
         g.nwall = static_cast<int>(walls.size());
         g.ntiles = static_cast<long long>(tiles.size());
-        g.ntiles2 = static_cast<long long>(tiles2.size());
         g.ntiles3 = static_cast<long long>(tiles3.size());
         g.has_tc = dg::stage_tc_supported(g.p);
         lam_total += g.K;
@@ -607,7 +618,16 @@ dg_status dg_batch_create(const dg_params *common, int ncases, const dg_case *ca
         chk(g.geo32.alloc(g32.size()));
         chk(g.conn.alloc(conn.size()));
         chk(g.tiles.alloc(tiles.size()));
-        chk(g.tiles2.alloc(tiles2.size()));
+        std::vector<double> tab;
+        std::vector<int> nodes, slots;
+        std::vector<float> tab32;
+        if (!dg::build_sym64_tables(g.ops, tab, nodes)) return bail(DG_EINVAL);
+        dg::build_sym32_tables(g.ops, tab, nodes, tab32, slots);
+        chk(g.sym32.alloc(tab32.size()));
+        chk(g.symn32.alloc(slots.size()));
+        chk(g.fd32.alloc(2 * static_cast<size_t>(g.K) * NF));
+        chk(g.rv32.alloc(static_cast<size_t>(g.K) * Np));
+        chk(g.bar.alloc(8));
         chk(g.tiles3.alloc(tiles3.size()));
         std::vector<float> frag;
         if (g.has_tc) {
@@ -630,7 +650,9 @@ dg_status dg_batch_create(const dg_params *common, int ncases, const dg_case *ca
         chk(cudaMemcpy(g.geo32.ptr, g32.data(), g32.size() * sizeof(float), cudaMemcpyHostToDevice));
         chk(cudaMemcpy(g.conn.ptr, conn.data(), conn.size() * sizeof(int4), cudaMemcpyHostToDevice));
         chk(cudaMemcpy(g.tiles.ptr, tiles.data(), tiles.size() * sizeof(int4), cudaMemcpyHostToDevice));
-        chk(cudaMemcpy(g.tiles2.ptr, tiles2.data(), tiles2.size() * sizeof(int4), cudaMemcpyHostToDevice));
+        chk(cudaMemcpy(g.sym32.ptr, tab32.data(), tab32.size() * sizeof(float), cudaMemcpyHostToDevice));
+        chk(cudaMemcpy(g.symn32.ptr, slots.data(), slots.size() * sizeof(int), cudaMemcpyHostToDevice));
+        chk(cudaMemset(g.bar.ptr, 0, 8 * sizeof(unsigned)));
         chk(cudaMemcpy(g.tiles3.ptr, tiles3.data(), tiles3.size() * sizeof(int4), cudaMemcpyHostToDevice));
         if (g.has_tc) chk(cudaMemcpy(g.tcfrag.ptr, frag.data(), frag.size() * sizeof(float), cudaMemcpyHostToDevice));
         chk(cudaMemcpy(g.elem_case.ptr, ecase.data(), ecase.size() * sizeof(int), cudaMemcpyHostToDevice));
@@ -651,7 +673,7 @@ dg_status dg_batch_create(const dg_params *common, int ncases, const dg_case *ca
         chk(cudaMemset(g.P0a.ptr, 0, npp * sizeof(float)));
         chk(cudaMemset(g.P0b.ptr, 0, npp * sizeof(float)));
         chk(dg::stage_shape_mixed_batch(g.p, g.ntiles, g.shape));
-        chk(dg::stage_shape_mixed2(g.p, g.ntiles2, true, g.shape2));
+        chk(dg::stage_shape_mixed2(g.p, g.K, true, false, g.shape2));
         if (g.has_tc) chk(dg::stage_shape_tc(g.p, g.ntiles3, true, false, g.shape3));
         if (e != cudaSuccess) return bail(DG_ECUDA);
     }
@@ -733,13 +755,6 @@ dg_status dg_batch_set_fused_steps(dg_batch *b, int on)
     if (!b) return DG_EINVAL;
     b->err.clear();
     if (on < 0 || on > 2) return bfail(b, DG_EINVAL, "fused steps: 0 (off), 1 (per degree group) or 2 (all groups)");
-    if (on) {
-        for (auto &g : b->groups) {
-            if (g.bar.ptr) continue;
-            B_CUDA(b, g.bar.alloc(8));
-            B_CUDA(b, cudaMemset(g.bar.ptr, 0, 8 * sizeof(unsigned)));
-        }
-    }
     b->fused = on != 0;
     b->fused_all = on == 2;
     b->all_nblk.clear();
@@ -897,8 +912,9 @@ dg_status dg_batch_run(dg_batch *b, double cfl, int nsteps, int use_graph, doubl
         B_CUDA(b, cudaMemcpy(&e, b->bar_err.ptr, sizeof(int), cudaMemcpyDeviceToHost));
         if (e) {
             B_CUDA(b, cudaMemset(b->bar_err.ptr, 0, sizeof(int)));
+            for (auto &g : b->groups) B_CUDA(b, cudaMemset(g.bar.ptr, 0, 8 * sizeof(unsigned)));
             return bfail(b, DG_ETIMEOUT,
-                         "a bounded device wait gave up (a fused step's grid barrier or a stage kernel's copy "
+                         "a bounded device wait gave up (a grid barrier, or a stage kernel's copy "
                          "wait); the states are not valid");
         }
     }

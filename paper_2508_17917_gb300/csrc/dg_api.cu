@@ -42,9 +42,11 @@ struct dg_ctx {
     std::vector<int32_t> EToV;
     std::vector<double> geo64h;
     // device
-    // FP64 path: symmetric operator tables, every face once, phase arrays
+    // FP64 and two-node kernels: symmetric operator tables, every face once, arrays between phases
     dg::DevBuf<double> sym64, flux64, dh64, th64;
-    dg::DevBuf<int> symn;
+    dg::DevBuf<float> sym32;
+    dg::DevBuf<float4> fd32, rv32;
+    dg::DevBuf<int> symn, symn32;
     dg::DevBuf<int4> faces;
     int nfaces = 0;
     dg::DevBuf<double> K0a, K0b, K1, rtmp, geo64, ops64, Dr64, Ds64, src, scal, fpart, fxy, wface;
@@ -89,8 +91,11 @@ struct dg_ctx {
     float *pother() { return cur_is_a ? P0b.ptr : P0a.ptr; }
     // finished blocks of the wall-force kernel: the last word of scal
     unsigned *ticket() { return reinterpret_cast<unsigned *>(scal.ptr + 3); }
+    cudaEvent_t tune_ev[9] = {};     // mixed: marks of the stage-shape timing
     ~dg_ctx()
     {
+        for (auto &e : tune_ev)
+            if (e) cudaEventDestroy(e);
         for (auto *b : {&K0a, &K0b, &K1, &rtmp, &geo64, &ops64, &Dr64, &Ds64, &src, &scal, &fpart, &fxy, &wface})
             b->release();
         geo32.release();
@@ -110,12 +115,12 @@ struct dg_ctx {
 namespace {
 
 // waits of about 100 ns (1.7 s in all) before a grid barrier between the
-// phases of an FP64 stage gives up; its blocks are resident together, so a
+// phases of a stage gives up; its blocks are resident together, so a
 // wait is as long as the slowest block's share of a phase
 constexpr unsigned kPhaseWaitLimit = 1u << 24;
 
 const char *const kWaitGaveUp =
-    "a bounded device wait gave up (a grid barrier of a fused step or an FP64 stage, or a stage kernel's copy wait: "
+    "a bounded device wait gave up (a grid barrier of a fused step or of a stage's phases, or a stage kernel's copy wait: "
     "the state is not valid; or the tcgen05 gradient kernel: its output is not valid)";
 
 dg_status fail(dg_ctx *c, dg_status st, const std::string &msg)
@@ -193,6 +198,28 @@ void manufactured_source(double x, double y, double kappa, double C2, const dg_p
 // C1 (1+theta)^2 (d+1) of Eq. penalty_final, d = 2
 double sigma_factor(const dg_params &p) { return p.C1 * (1.0 + p.theta) * (1.0 + p.theta) * 3.0; }
 
+// what the two-node kernel hands from stage to stage; a mesh that leaves no
+// memory for it runs with the other shapes
+cudaError_t two_node_arrays(dg_ctx *c)
+{
+    if (c->rv32.ptr) return cudaSuccess;
+    cudaError_t e = c->fd32.alloc(2 * static_cast<size_t>(c->K) * 3 * c->ops.Nfp);
+    if (e == cudaSuccess) e = c->rv32.alloc(static_cast<size_t>(c->K) * c->ops.Np);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        c->fd32.release();
+        c->rv32.release();
+    }
+    return e;
+}
+
+// s: stage of a step, -1 for a residual
+dg::Stage2Args stage2_args(const dg_ctx *c, int s)
+{
+    return dg::stage2_args(c->sym32.ptr, c->symn32.ptr, c->fd32.ptr, c->rv32.ptr, nullptr,
+                           static_cast<size_t>(c->K) * 3 * c->ops.Nfp, s);
+}
+
 dg_status run_stage(dg_ctx *c, int s, double t, double dt, const double vw[2], int mode,
                     const double *in, double *out, double *rout)
 {
@@ -263,7 +290,14 @@ dg_status run_stage(dg_ctx *c, int s, double t, double dt, const double vw[2], i
             e = dg::launch_stage_tc(c->prm.p, false, false, c->shape, sp, make_phys<float>(c->prm, vw), c->stream);
         }
         else if (c->shape.variant == 2)
-            e = dg::launch_stage_mixed2(c->prm.p, false, c->shape, sp, make_phys<float>(c->prm, vw), c->stream);
+            {
+                sp.bar = c->bar.ptr;
+                sp.bar_err = c->bar_err.ptr;
+                sp.bar_limit = kPhaseWaitLimit;
+                c->copy_used = true;
+                e = dg::launch_stage_mixed2(c->prm.p, false, false, c->shape, sp, stage2_args(c, s),
+                                            make_phys<float>(c->prm, vw), c->stream);
+            }
         else
             e = dg::launch_stage_mixed(c->prm.p, c->shape, sp, make_phys<float>(c->prm, vw), c->stream);
     }
@@ -329,6 +363,13 @@ dg_status dg_create(const dg_params *params, void *cuda_stream, dg_ctx **out)
         delete c;
         return DG_ECUDA;
     }
+    if (p.precision == DG_PRECISION_MIXED)
+        for (auto &e : c->tune_ev)
+            if (cudaEventCreate(&e) != cudaSuccess) {
+                cudaGetLastError();
+                delete c;
+                return DG_ECUDA;
+            }
     const int Np = c->ops.Np, NF = 3 * c->ops.Nfp;
     std::vector<double> o64;
     o64.insert(o64.end(), c->ops.Dr.begin(), c->ops.Dr.end());
@@ -373,6 +414,16 @@ dg_status dg_create(const dg_params *params, void *cuda_stream, dg_ctx **out)
         }
         cudaMemcpy(c->sym64.ptr, tab.data(), tab.size() * sizeof(double), cudaMemcpyHostToDevice);
         cudaMemcpy(c->symn.ptr, nodes.data(), nodes.size() * sizeof(int), cudaMemcpyHostToDevice);
+        std::vector<float> tab32;
+        std::vector<int> slots;
+        dg::build_sym32_tables(c->ops, tab, nodes, tab32, slots);
+        if (c->sym32.alloc(tab32.size()) != cudaSuccess || c->symn32.alloc(slots.size()) != cudaSuccess) {
+            cudaGetLastError();
+            delete c;
+            return DG_ECUDA;
+        }
+        cudaMemcpy(c->sym32.ptr, tab32.data(), tab32.size() * sizeof(float), cudaMemcpyHostToDevice);
+        cudaMemcpy(c->symn32.ptr, slots.data(), slots.size() * sizeof(int), cudaMemcpyHostToDevice);
     }
     if (dg::stage_tc_supported(p.p)) {
         std::vector<float> frag;
@@ -469,6 +520,10 @@ dg_status dg_set_stage_variant(dg_ctx *c, int variant)
         return fail(c, DG_EUNSUPPORTED, "the two-node kernel is an IIP kernel");
     if (variant == 3 && !dg::stage_tc_supported(c->prm.p))
         return fail(c, DG_EUNSUPPORTED, "the tensor-core kernel covers p <= 6");
+    if (variant == 2 && c->K > 0) {
+        const cudaError_t e = two_node_arrays(c);
+        if (e != cudaSuccess) return cuda_fail(c, e, "arrays of the two-node kernel");
+    }
     c->variant_req = variant;
     c->tuned = (variant != 0);
     if (c->K > 0 && c->prm.precision == DG_PRECISION_MIXED)
@@ -505,20 +560,8 @@ dg_status dg_set_mesh(dg_ctx *c, int64_t Nv, const double *vx, const double *vy,
     DG_CUDA(c, cudaMemcpy(c->geo64.ptr, geo.data(), geo.size() * sizeof(double), cudaMemcpyHostToDevice));
     DG_CUDA(c, cudaMemcpy(c->conn.ptr, conn.data(), K * sizeof(int4), cudaMemcpyHostToDevice));
     if (c->prm.precision == DG_PRECISION_FP64) {
-        // every face once: interior faces in element order, then the boundary
-        std::vector<int4> fl, bl;
-        fl.reserve(static_cast<size_t>(K) * 3 / 2 + 3);
-        for (int64_t k = 0; k < K; ++k) {
-            const int4 cn = conn[k];
-            for (int f = 0; f < 3; ++f) {
-                const int nb = f == 0 ? cn.x : (f == 1 ? cn.y : cn.z);
-                const int f2 = (cn.w >> (2 * f)) & 3, bt = (cn.w >> (8 + 2 * f)) & 3;
-                const int4 fc = make_int4(static_cast<int>(k), nb, f | (f2 << 2) | (bt << 4), 0);
-                if (bt != dg::BCT_INTERIOR) bl.push_back(fc);
-                else if (k < nb) fl.push_back(fc);
-            }
-        }
-        fl.insert(fl.end(), bl.begin(), bl.end());
+        std::vector<int4> fl;
+        dg::unique_faces(conn.data(), K, fl);
         c->nfaces = static_cast<int>(fl.size());
         DG_CUDA(c, c->faces.alloc(fl.size()));
         DG_CUDA(c, cudaMemcpy(c->faces.ptr, fl.data(), fl.size() * sizeof(int4), cudaMemcpyHostToDevice));
@@ -526,6 +569,8 @@ dg_status dg_set_mesh(dg_ctx *c, int64_t Nv, const double *vx, const double *vy,
         DG_CUDA(c, c->flux64.alloc(2 * nd));
         DG_CUDA(c, c->dh64.alloc(4 * nfn));
         if (c->prm.theta != 0.0) DG_CUDA(c, c->th64.alloc(8 * nfn));
+    }
+    {
         dg_status bs = need_barrier(c);
         if (bs != DG_OK) return bs;
     }
@@ -542,6 +587,12 @@ dg_status dg_set_mesh(dg_ctx *c, int64_t Nv, const double *vx, const double *vy,
         DG_CUDA(c, cudaMemsetAsync(c->S0b.ptr, 0, np * sizeof(float4), c->stream));
         DG_CUDA(c, cudaMemsetAsync(c->P0a.ptr, 0, npp * sizeof(float), c->stream));
         DG_CUDA(c, cudaMemsetAsync(c->P0b.ptr, 0, npp * sizeof(float), c->stream));
+        c->fd32.release();
+        c->rv32.release();
+        if (c->prm.theta == 0.0) {
+            const cudaError_t e = two_node_arrays(c);
+            if (e != cudaSuccess && c->variant_req == 2) return cuda_fail(c, e, "arrays of the two-node kernel");
+        }
     }
     c->nwall = static_cast<int>(walls.size());
     if (c->nwall > 0) {
@@ -569,7 +620,7 @@ dg_status dg_set_mesh(dg_ctx *c, int64_t Nv, const double *vx, const double *vy,
     c->has_tc = false;
     if (c->prm.precision == DG_PRECISION_MIXED) {
         if (!th) {
-            e = dg::stage_shape_mixed2(c->prm.p, K, false, c->shape2);
+            e = dg::stage_shape_mixed2(c->prm.p, K, false, false, c->shape2);
             if (e != cudaSuccess) return cuda_fail(c, e, "stage kernel configuration");
             if (c->variant_req == 2) c->shape = c->shape2;
         }
@@ -688,44 +739,47 @@ dg_status dg_set_source(dg_ctx *c, int kind, const double *params)
 
 // Mixed path, first use: time every available stage-kernel shape (one and
 // two nodes per thread, tensor-core warp tiles; the two-node shape is IIP
-// only) on the current state in residual-only mode and keep the fastest.
+// only) on the current state and keep the fastest for a step, whose first
+// stage costs the two-node shape a volume phase and a grid barrier more than
+// the other four.  A first stage untimed, one timed, three inner ones, register
+// traffic and all (dt = 0): before a step the register and the other state
+// buffers hold nothing that is read again.
 static dg_status tune_stage(dg_ctx *c, const double vw[2])
 {
     if (c->tuned || c->prm.precision != DG_PRECISION_MIXED || c->variant_req != 0) {
         c->tuned = true;
         return DG_OK;
     }
-    if (c->rtmp.n != ndof(c)) DG_CUDA(c, c->rtmp.alloc(ndof(c)));
-    // events destroyed on every return path
-    struct Events {
-        cudaEvent_t e[2] = {nullptr, nullptr};
-        ~Events()
-        {
-            for (auto &x : e)
-                if (x) cudaEventDestroy(x);
-        }
-    } ev;
-    DG_CUDA(c, cudaEventCreate(&ev.e[0]));
-    DG_CUDA(c, cudaEventCreate(&ev.e[1]));
-    cudaEvent_t e0 = ev.e[0], e1 = ev.e[1];
-    float best = 0.f;
-    dg::LaunchShape pick = c->shape1;
-    for (const dg::LaunchShape *cand : {&c->shape1, &c->shape2, &c->shape3}) {
-        if (cand == &c->shape3 && !c->has_tc) continue;
-        if (cand == &c->shape2 && c->prm.theta != 0.0) continue;
-        c->shape = *cand;
-        float ms = 0.f;
+    // timed on 2^21 nodes at most, four times the L2 cache
+    struct Part {
+        dg_ctx *c;
+        int64_t K;
+        ~Part() { c->K = K; }
+    } part{c, c->K};
+    c->K = std::min<int64_t>(c->K, (1 << 21) / c->ops.Np);
+    const dg::LaunchShape *const cand[3] = {&c->shape1, c->rv32.ptr ? &c->shape2 : nullptr, c->has_tc ? &c->shape3 : nullptr};
+    for (int v = 0; v < 3; ++v) {
+        if (!cand[v]) continue;
+        c->shape = *cand[v];
         for (int rep = 0; rep < 5; ++rep) {
-            if (rep == 2) DG_CUDA(c, cudaEventRecord(e0, c->stream));
-            dg_status st = run_stage(c, -1, 0.0, 0.0, vw, dg::STAGE_RHS_ONLY, c->cur(), nullptr, c->rtmp.ptr);
+            if (rep == 1 || rep == 2) DG_CUDA(c, cudaEventRecord(c->tune_ev[3 * v + rep - 1], c->stream));
+            dg_status st = run_stage(c, rep == 0 ? 0 : rep - 1, 0.0, 0.0, vw, dg::STAGE_UPDATE, c->cur(), c->other(), nullptr);
             if (st != DG_OK) return st;
         }
-        DG_CUDA(c, cudaEventRecord(e1, c->stream));
-        DG_CUDA(c, cudaEventSynchronize(e1));
-        DG_CUDA(c, cudaEventElapsedTime(&ms, e0, e1));
-        if (cand == &c->shape1 || ms < best) {
+        DG_CUDA(c, cudaEventRecord(c->tune_ev[3 * v + 2], c->stream));
+    }
+    DG_CUDA(c, cudaStreamSynchronize(c->stream));
+    float best = 0.f;
+    dg::LaunchShape pick = c->shape1;
+    for (int v = 0; v < 3; ++v) {
+        if (!cand[v]) continue;
+        float first = 0.f, inner = 0.f;
+        DG_CUDA(c, cudaEventElapsedTime(&first, c->tune_ev[3 * v], c->tune_ev[3 * v + 1]));
+        DG_CUDA(c, cudaEventElapsedTime(&inner, c->tune_ev[3 * v + 1], c->tune_ev[3 * v + 2]));
+        const float ms = first + 4.0f / 3.0f * inner;
+        if (v == 0 || ms < best) {
             best = ms;
-            pick = *cand;
+            pick = *cand[v];
         }
     }
     c->shape = pick;
@@ -757,9 +811,9 @@ dg_status dg_rhs(dg_ctx *c, double t, const double vw[2], double *dUdt, int on_d
 static dg_status run_fused_step(dg_ctx *c, double dt, const double vw[2])
 {
     if (c->fshape_variant != c->shape.variant) {
-        cudaError_t e = (c->shape.variant == 3)
-                            ? dg::stage_shape_tc(c->prm.p, c->K, false, true, c->fshape)
-                            : dg::stage_shape_mixed_fused(c->prm.p, c->shape.variant, false, c->K, c->fshape);
+        cudaError_t e = (c->shape.variant == 3)   ? dg::stage_shape_tc(c->prm.p, c->K, false, true, c->fshape)
+                        : (c->shape.variant == 2) ? dg::stage_shape_mixed2(c->prm.p, c->K, false, true, c->fshape)
+                                                  : dg::stage_shape_mixed_fused(c->prm.p, false, c->K, c->fshape);
         if (e != cudaSuccess) return cuda_fail(c, e, "fused stage kernel configuration");
         c->fshape_variant = c->shape.variant;
     }
@@ -794,6 +848,9 @@ static dg_status run_fused_step(dg_ctx *c, double dt, const double vw[2])
     DG_CUDA(c, cudaMemsetAsync(c->bar.ptr, 0, 2 * sizeof(unsigned), c->stream));
     if (c->fshape.variant == 3)
         DG_CUDA(c, dg::launch_stage_tc(c->prm.p, false, true, c->fshape, sp, make_phys<float>(c->prm, vw), c->stream));
+    else if (c->fshape.variant == 2)
+        DG_CUDA(c, dg::launch_stage_mixed2(c->prm.p, false, true, c->fshape, sp, stage2_args(c, 0),
+                                           make_phys<float>(c->prm, vw), c->stream));
     else
         DG_CUDA(c, dg::launch_stage_mixed_fused(c->prm.p, false, c->fshape, sp, make_phys<float>(c->prm, vw), c->stream));
     c->launches += 1;

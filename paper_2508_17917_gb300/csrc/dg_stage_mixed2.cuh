@@ -10,6 +10,10 @@
 // face nodes r and r + HF of one face, so every broadcast record feeds two
 // outputs (and both face nodes share the neighbour's records), at 128
 // threads per block with up to 128 registers per thread.
+// Of a single mesh's two-node kernels this is the one for p = 3 below 25,000
+// elements and p = 5 below 15,000, where the hand-off kernel's extra volume
+// phase and barrier in a step's first stage are not earned back or its tiles
+// leave a wave nearly empty (stage_shape_mixed2).
 #pragma once
 #include "dg_stage_mixed.cuh"
 
@@ -26,7 +30,7 @@ struct Shape2 {
     static constexpr int E = NT / W;
 };
 
-template <int P, bool BATCH, bool FUSE = false>
+template <int P, bool FUSE>
 __global__ void __launch_bounds__(128, 4)
 stage_mixed2_kernel(StageParams sp, Phys<float> ph)
 {
@@ -63,11 +67,11 @@ stage_mixed2_kernel(StageParams sp, Phys<float> ph)
     }
     const float *geo = static_cast<const float *>(sp.geo);
     const long long K = sp.K;
-    const long long ntiles = BATCH ? sp.ntiles : (K + E - 1) / E;
+    const long long ntiles = (K + E - 1) / E;
     const double gm1d = sp.gm1;
     const float cinv_fac = 0.5f * float(P + 1) * float(P + 2);
     const float sig_fac = static_cast<float>(sp.sig_fac);
-    float dtr = static_cast<float>(sp.dt);
+    const float dtr = static_cast<float>(sp.dt);
     const bool update = sp.mode == STAGE_UPDATE;
     bool need_k1 = update && !sp.first_stage;
     __syncthreads();
@@ -96,14 +100,8 @@ stage_mixed2_kernel(StageParams sp, Phys<float> ph)
     // group B (the FP64 registers K0, K1) of tile t is copied while tile t
     // runs P2 and P3.  The connectivity is double-buffered.
     auto tile_at = [&](long long t, long long &k0t, int &net) {
-        if constexpr (BATCH) {
-            const int4 td = sp.tiles[t];
-            k0t = td.x;
-            net = td.y;
-        } else {
-            k0t = t * E;
-            net = static_cast<int>((K - k0t) < E ? (K - k0t) : E);
-        }
+        k0t = t * E;
+        net = static_cast<int>((K - k0t) < E ? (K - k0t) : E);
     };
     auto issue_a = [&](long long k0t, int net, const int4 *cnt) {
         const char *gU = reinterpret_cast<const char *>(sp.Sin + k0t * Np);
@@ -149,12 +147,6 @@ stage_mixed2_kernel(StageParams sp, Phys<float> ph)
         long long k0;
         int ne;
         tile_at(tile, k0, ne);
-        if constexpr (BATCH) {
-            const BatchCase &cs = sp.cases[sp.tiles[tile].z];
-            ph.mu = cvt_d2f(cs.mu);           // integer conversions: no FP64-pipe work per tile
-            ph.vw2 = cvt_d2f(cs.vb);
-            dtr = cvt_d2f(cs.dt);
-        }
         const int4 *cnb = sConn + buf * E;
         int4 *cnx = sConn + (buf ^ 1) * E;
         const long long tn = tile + gridDim.x;

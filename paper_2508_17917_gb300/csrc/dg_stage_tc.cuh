@@ -108,9 +108,9 @@ struct TcLayout {
     static constexpr size_t hBar = hD + al(sizeof(float2) * Np * S::DS);   // mbarrier of the operator copy
     static constexpr size_t header = hBar + 16;
     // one region per warp
-    static constexpr size_t oConn = 0;                                      // int4 [2][WE]: this tile's, the next one's
-    static constexpr size_t oTile = oConn + al(16 * 2 * WE);                // int4 [4]: batch tile table entries
-    static constexpr size_t oGeo = oTile + 64;                              // float [WE][16]
+    static constexpr size_t oConn = 0;                                      // int4 [WE]; AHEAD: [2][WE], this tile's, the next one's
+    static constexpr size_t oTile = oConn + al(16 * (S::AHEAD ? 2 : 1) * WE);      // AHEAD: int4 [4], batch tile table entries
+    static constexpr size_t oGeo = oTile + (S::AHEAD ? 64 : 0);             // float [WE][16]
     static constexpr size_t oNGeo = oGeo + al(64 * WE);                     // float [3 WE][16]
     static constexpr size_t oU = oNGeo + al(64 * 3 * WE);                   // float4 [WE][US]
     static constexpr size_t oN = oU + al(16 * WE * S::US);                  // float4 [3 WE][UN]

@@ -21,6 +21,8 @@ struct LaunchShape {
     int threads = 0;
     size_t smem = 0;
     int elems_per_tile = 0;
+    bool handoff = false;    // two nodes per thread: the kernel that hands volume parts from stage to stage
+    int per_sm = 0;          // ... and its blocks per SM (4 or 5)
 };
 
 // Launch `kern` with programmatic stream serialization: its blocks may be
@@ -76,16 +78,40 @@ cudaError_t launch_stage_mixed_batch(int p, const LaunchShape &ls, const StagePa
 // Lambda_K of every degree group of a batch in one launch (one block per tile)
 cudaError_t launch_dt_lambda_mixed_multi(const DtGroups &dgs, const BatchCase *cases, const Phys<float> &ph,
                                          float sig_fac, cudaStream_t st);
-// the mixed IIP kernel with two nodes per thread: units = K elements (single
-// mesh) or the tile count of a tile table (batch); its tiles hold
-// stage_tile_elems2(p) elements
-cudaError_t stage_shape_mixed2(int p, long long units, bool batch, LaunchShape &out);
-cudaError_t launch_stage_mixed2(int p, bool batch, const LaunchShape &ls, const StageParams &sp,
-                                const Phys<float> &ph, cudaStream_t st);
-int stage_tile_elems2(int p);
-// five stages per cooperative launch (mixed IIP, shape `variant`): grid of
+// the mixed IIP kernel with two nodes per thread for K elements: one stage, or
+// the five of a step (fused).  Its tables are those of build_sym32_tables; it
+// hands a record per face node (pressure, viscous normal flux) [K][3 Nfp] and
+// the divergence [K][Np] from stage to stage.  A launch with `first` (and a
+// fused one) is cooperative.
+struct Stage2Args {
+    const float *ops;
+    const int *nodes;
+    const float4 *fin;         // trace records this stage reads (first: written to fout, then swapped)
+    float4 *fout;              // ... and the next one's
+    float4 *rv;
+    const int *elem_case;      // batch: case of every element
+    int first, next;           // a step's first stage (or a residual); not its last (residual: 1, 0)
+};
+// those of stage s of a step (-1: a residual; 0 also for a fused step) with the
+// two flux buffers of n records each at fd: the first stage fills the first
+// buffer, and the buffers change roles from stage to stage
+inline Stage2Args stage2_args(const float *ops, const int *nodes, float4 *fd, float4 *rv, const int *elem_case, size_t n, int s)
+{
+    const bool second = s <= 0 || (s & 1);
+    return {ops, nodes, second ? fd + n : fd, second ? fd : fd + n, rv, elem_case, s <= 0 ? 1 : 0, s >= 0 && s < 4 ? 1 : 0};
+}
+cudaError_t stage_shape_mixed2(int p, long long K, bool batch, bool fused, LaunchShape &out);
+cudaError_t launch_stage_mixed2(int p, bool batch, bool fused, const LaunchShape &ls, const StageParams &sp,
+                                const Stage2Args &a, const Phys<float> &ph, cudaStream_t st);
+// FP32 rows (each twice) from the FP64 tables, and per thread its two nodes
+// and up to two face slots of each
+void build_sym32_tables(const RefOps &o, const std::vector<double> &tab, const std::vector<int> &nodes,
+                        std::vector<float> &tab32, std::vector<int> &slots);
+// every face of K elements once, as Stage64Args has them
+void unique_faces(const int4 *conn, long long K, std::vector<int4> &faces);
+// five stages per cooperative launch (mixed IIP, one node per thread): grid of
 // co-resident blocks for `units` (K, or the tile count of a batch table)
-cudaError_t stage_shape_mixed_fused(int p, int variant, bool batch, long long units, LaunchShape &out);
+cudaError_t stage_shape_mixed_fused(int p, bool batch, long long units, LaunchShape &out);
 cudaError_t launch_stage_mixed_fused(int p, bool batch, const LaunchShape &ls, const StageParams &sp,
                                      const Phys<float> &ph, cudaStream_t st);
 // elements per tile of the mixed kernel for degree p

@@ -232,4 +232,61 @@ bool build_sym64_tables(const RefOps &o, std::vector<double> &tab, std::vector<i
     }
 }
 
+namespace {
+
+template <int P>
+void sym32_tables_p(const RefOps &o, const std::vector<double> &tab, const std::vector<int> &nodes,
+                    std::vector<float> &tab32, std::vector<int> &slots)
+{
+    using S = Sym64<P>;
+    tab32.resize(4 * S::oQA);
+    for (int i = 0; i < S::oQA; ++i) {
+        tab32[4 * i] = tab32[4 * i + 1] = static_cast<float>(tab[2 * i]);
+        tab32[4 * i + 2] = tab32[4 * i + 3] = static_cast<float>(tab[2 * i + 1]);
+    }
+    slots.assign(6 * S::TPE, -1);
+    for (int t = 0; t < S::TPE; ++t)
+        for (int q = 0; q < 2; ++q) {
+            const int n = nodes[2 * t + q];
+            slots[6 * t + q] = n;
+            int at = 6 * t + 2 + 2 * q;
+            for (int m = 0; m < S::NF; ++m)
+                if (n >= 0 && o.Fmask[m] == n) slots[at++] = m;      // a vertex belongs to two faces
+        }
+}
+
+}  // namespace
+
+void build_sym32_tables(const RefOps &o, const std::vector<double> &tab, const std::vector<int> &nodes,
+                        std::vector<float> &tab32, std::vector<int> &slots)
+{
+    switch (o.p) {
+    case 1: return sym32_tables_p<1>(o, tab, nodes, tab32, slots);
+    case 2: return sym32_tables_p<2>(o, tab, nodes, tab32, slots);
+    case 3: return sym32_tables_p<3>(o, tab, nodes, tab32, slots);
+    case 4: return sym32_tables_p<4>(o, tab, nodes, tab32, slots);
+    case 5: return sym32_tables_p<5>(o, tab, nodes, tab32, slots);
+    case 6: return sym32_tables_p<6>(o, tab, nodes, tab32, slots);
+    default: return;
+    }
+}
+
+void unique_faces(const int4 *conn, long long K, std::vector<int4> &faces)
+{
+    std::vector<int4> edge;
+    faces.clear();
+    faces.reserve(static_cast<size_t>(K) * 3 / 2 + 3);
+    for (long long k = 0; k < K; ++k) {
+        const int4 cn = conn[k];
+        for (int f = 0; f < 3; ++f) {
+            const int nb = f == 0 ? cn.x : (f == 1 ? cn.y : cn.z);
+            const int f2 = (cn.w >> (2 * f)) & 3, bt = (cn.w >> (8 + 2 * f)) & 3;
+            const int4 fc = make_int4(static_cast<int>(k), nb, f | (f2 << 2) | (bt << 4), 0);
+            if (bt != BCT_INTERIOR) edge.push_back(fc);
+            else if (k < nb) faces.push_back(fc);
+        }
+    }
+    faces.insert(faces.end(), edge.begin(), edge.end());
+}
+
 }  // namespace dg

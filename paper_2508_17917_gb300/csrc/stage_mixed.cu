@@ -2,6 +2,7 @@
 // FP32 arithmetic, FP64 state in HBM, FP64 pressure recovery and registers.
 #include "dg_dt.cuh"
 #include "dg_stage_mixed.cuh"
+#include "dg_stage_handoff.cuh"
 #include "dg_stage_mixed2.cuh"
 #include "launch.h"
 
@@ -76,15 +77,105 @@ cudaError_t launch_batch_p(const LaunchShape &ls, const StageParams &sp, const P
     return cudaGetLastError();
 }
 
-// two nodes per thread (IIP): shape for `ntiles` tiles (batch) or for K elements
-template <int P, bool BATCH>
-cudaError_t shape2_p(long long units, LaunchShape &ls)
+// Cooperative launch: the blocks are resident together
+template <typename... KArgs, typename... Args>
+cudaError_t launch_coop(void (*kern)(KArgs...), const LaunchShape &ls, cudaStream_t st, Args... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(ls.grid);
+    cfg.blockDim = dim3(ls.threads);
+    cfg.dynamicSmemBytes = ls.smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
+// two nodes per thread (IIP), hand-off kernel: as many blocks as are resident
+// at once (a step's first stage and fused steps have grid barriers), capped by
+// the tiles.  A wave of m blocks per SM takes about m units of time, so of five
+// (96 registers, a few spills) and four (128) the one with the smaller
+// m x waves is taken, four if they are equal.  Measured, us a stage with five
+// and with four, waves: p = 5, 60^2 quads 0.9 and 1.1: 20.5 and 24.9; 76^2 1.4
+// and 1.7: 32.5 and 28.4; 90^2 1.9 and 2.4: 34.4 and 38.7; 100^2 2.4 and 3.0:
+// 46.2 and 39.7; p = 3, 128^2 1.8 and 2.2: 29.8 and 32.3; 256^2 7.2 and 9.0: 98.6
+// and 95.2; p = 1, 256^2 2.7 and 3.4: 36.9 and 39.3.  At p = 6 five spill more
+// and are behind even in one wave against two (56^2: 25.9 and 24.5).
+template <int P, bool BATCH, bool FUSE, int M>
+cudaError_t handoff_grid_p(long long K, LaunchShape &ls)
+{
+    using S = Sym64<P>;
+    using L = Layout2<P>;
+    auto kern = stage_handoff_kernel<P, BATCH, FUSE, M>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(L::bytes));
+    if (e != cudaSuccess) return e;
+    int per_sm = 0, dev = 0, sms = 0;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, S::NT, L::bytes);
+    if (e != cudaSuccess) return e;
+    if (per_sm < 1) return cudaErrorInvalidConfiguration;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const long long per_block = L::EG * L::NG, tiles = (K + per_block - 1) / per_block;
+    const long long grid = static_cast<long long>(sms) * per_sm;
+    const long long cost = per_sm * ((tiles + grid - 1) / grid), have = ls.grid;
+    if (have > 0) {
+        // the shape in ls is the one with four
+        const long long g4 = static_cast<long long>(sms) * ls.per_sm;
+        if (cost >= ls.per_sm * ((tiles + g4 - 1) / g4)) return cudaSuccess;
+    }
+    ls.per_sm = per_sm;
+    ls.grid = static_cast<int>(tiles < grid ? tiles : grid);
+    ls.threads = S::NT;
+    ls.smem = L::bytes;
+    ls.elems_per_tile = L::EG;
+    ls.theta = false;
+    ls.variant = 2;
+    ls.handoff = true;
+    return cudaSuccess;
+}
+
+template <int P, bool BATCH, bool FUSE>
+cudaError_t handoff_shape_p(long long K, LaunchShape &ls)
+{
+    ls.grid = 0;
+    cudaError_t e = handoff_grid_p<P, BATCH, FUSE, 4>(K, ls);
+    if constexpr (!FUSE && P != 6)
+        if (e == cudaSuccess) e = handoff_grid_p<P, BATCH, FUSE, 5>(K, ls);
+    return e;
+}
+
+template <int P, bool BATCH, bool FUSE, int M>
+cudaError_t handoff_launch_p(const LaunchShape &ls, const StageParams &sp, const Stage2 &x, const Phys<float> &ph,
+                             cudaStream_t st)
+{
+    auto kern = stage_handoff_kernel<P, BATCH, FUSE, M>;
+    if (!FUSE && !x.first) {
+        if (!BATCH) return launch_pdl(kern, ls, st, sp, x, ph);
+        kern<<<ls.grid, ls.threads, ls.smem, st>>>(sp, x, ph);
+        return cudaGetLastError();
+    }
+    return launch_coop(kern, ls, st, sp, x, ph);
+}
+
+template <int P, bool BATCH, bool FUSE>
+cudaError_t launch2_p(const LaunchShape &ls, const StageParams &sp, const Stage2 &x, const Phys<float> &ph, cudaStream_t st)
+{
+    if constexpr (!FUSE && P != 6)
+        if (ls.per_sm == 5) return handoff_launch_p<P, BATCH, FUSE, 5>(ls, sp, x, ph, st);
+    return handoff_launch_p<P, BATCH, FUSE, 4>(ls, sp, x, ph, st);
+}
+
+// ... and the kernel whose stages stand alone (single mesh, p = 3 and 5)
+template <int P, bool FUSE>
+cudaError_t alone_shape_p(long long K, LaunchShape &ls)
 {
     using S2 = Shape2<P>;
     using L = MixedLayout<P, false, S2::E>;
-    auto kern = stage_mixed2_kernel<P, BATCH>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(L::bytes));
+    auto kern = stage_mixed2_kernel<P, FUSE>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(L::bytes));
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     if (e != cudaSuccess) return e;
@@ -93,50 +184,37 @@ cudaError_t shape2_p(long long units, LaunchShape &ls)
     if (e != cudaSuccess) return e;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (per_sm < 1) per_sm = 1;
-    const long long ntiles = BATCH ? units : (units + S2::E - 1) / S2::E;
-    long long grid = static_cast<long long>(sms) * per_sm;
+    if (per_sm < 1) {
+        if (FUSE) return cudaErrorInvalidConfiguration;
+        per_sm = 1;
+    }
+    const long long ntiles = (K + S2::E - 1) / S2::E, grid = static_cast<long long>(sms) * per_sm;
     ls.grid = static_cast<int>(ntiles < grid ? ntiles : grid);
     ls.threads = S2::NT;
     ls.smem = L::bytes;
     ls.elems_per_tile = S2::E;
     ls.theta = false;
     ls.variant = 2;
+    ls.handoff = false;
     return cudaSuccess;
 }
 
-template <int P, bool BATCH>
-cudaError_t launch2_p(const LaunchShape &ls, const StageParams &sp, const Phys<float> &ph, cudaStream_t st)
+template <int P>
+cudaError_t alone_launch_p(bool fused, const LaunchShape &ls, const StageParams &sp, const Phys<float> &ph, cudaStream_t st)
 {
-    if (BATCH) {
-        stage_mixed2_kernel<P, true><<<ls.grid, ls.threads, ls.smem, st>>>(sp, ph);
-        return cudaGetLastError();
-    }
-    return launch_pdl(stage_mixed2_kernel<P, false, false>, ls, st, sp, ph);
+    if (!fused) return launch_pdl(stage_mixed2_kernel<P, false>, ls, st, sp, ph);
+    return launch_coop(stage_mixed2_kernel<P, true>, ls, st, sp, ph);
 }
 
-// fused variant: five stages per cooperative launch; the grid is the number
-// of co-resident blocks of that instantiation (capped by the tile count)
-template <int P, int V, bool BATCH>
+// fused variant of the one-node shape: five stages per cooperative launch;
+// the grid is the number of co-resident blocks (capped by the tile count)
+template <int P, bool BATCH>
 cudaError_t fused_shape_p(long long units, LaunchShape &ls)
 {
-    const void *kern;
-    int nt;
-    size_t smem;
-    long long ntiles;
-    if (V == 2) {
-        kern = reinterpret_cast<const void *>(stage_mixed2_kernel<P, BATCH, true>);
-        nt = Shape2<P>::NT;
-        smem = MixedLayout<P, false, Shape2<P>::E>::bytes;
-        ntiles = BATCH ? units : (units + Shape2<P>::E - 1) / Shape2<P>::E;
-        ls.elems_per_tile = Shape2<P>::E;
-    } else {
-        kern = reinterpret_cast<const void *>(stage_mixed_kernel<P, false, BATCH, true>);
-        nt = Shape<P>::NT;
-        smem = MixedLayout<P, false>::bytes;
-        ntiles = BATCH ? units : (units + Shape<P>::E - 1) / Shape<P>::E;
-        ls.elems_per_tile = Shape<P>::E;
-    }
+    auto kern = stage_mixed_kernel<P, false, BATCH, true>;
+    const int nt = Shape<P>::NT;
+    const size_t smem = MixedLayout<P, false>::bytes;
+    const long long ntiles = BATCH ? units : (units + Shape<P>::E - 1) / Shape<P>::E;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
@@ -151,12 +229,13 @@ cudaError_t fused_shape_p(long long units, LaunchShape &ls)
     ls.grid = static_cast<int>(ntiles < grid ? ntiles : grid);
     ls.threads = nt;
     ls.smem = smem;
+    ls.elems_per_tile = Shape<P>::E;
     ls.theta = false;
-    ls.variant = V;
+    ls.variant = 1;
     return cudaSuccess;
 }
 
-template <int P, int V, bool BATCH>
+template <int P, bool BATCH>
 cudaError_t fused_launch_p(const LaunchShape &ls, const StageParams &sp, const Phys<float> &ph, cudaStream_t st)
 {
     cudaLaunchConfig_t cfg = {};
@@ -169,7 +248,6 @@ cudaError_t fused_launch_p(const LaunchShape &ls, const StageParams &sp, const P
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if (V == 2) return cudaLaunchKernelEx(&cfg, stage_mixed2_kernel<P, BATCH, true>, sp, ph);
     return cudaLaunchKernelEx(&cfg, stage_mixed_kernel<P, false, BATCH, true>, sp, ph);
 }
 
@@ -253,25 +331,39 @@ cudaError_t launch_dt_screen(const AuxMesh &m, const Phys<float> &ph, double gm1
 #undef C_
 }
 
-cudaError_t stage_shape_mixed2(int p, long long units, bool batch, LaunchShape &out)
+cudaError_t stage_shape_mixed2(int p, long long K, bool batch, bool fused, LaunchShape &out)
 {
-#define C_(P) (batch ? shape2_p<P, true>(units, out) : shape2_p<P, false>(units, out))
+    // Measured, us for two steps of a single mesh, fastest of the shapes of each
+    // side: p = 3, 76^2 quads 138 (stages alone) and 147 (hand-off), 110^2 231
+    // and 245, 119^2 295 and 247; p = 5, 50^2 140 and 172, 70^2 235 and 274, 86^2
+    // 329 and 341, 90^2 393 and 346.  Other degrees: hand-off ahead or neither
+    // the fastest shape.
+    if (!batch && p == 3 && K < 25000) return fused ? alone_shape_p<3, true>(K, out) : alone_shape_p<3, false>(K, out);
+    if (!batch && p == 5 && K < 15000) return fused ? alone_shape_p<5, true>(K, out) : alone_shape_p<5, false>(K, out);
+#define C_(P) (batch ? (fused ? handoff_shape_p<P, true, true>(K, out) : handoff_shape_p<P, true, false>(K, out)) \
+                     : (fused ? handoff_shape_p<P, false, true>(K, out) : handoff_shape_p<P, false, false>(K, out)))
     DG_SWITCH_P(p, C_)
 #undef C_
 }
 
-cudaError_t launch_stage_mixed2(int p, bool batch, const LaunchShape &ls, const StageParams &sp,
-                                const Phys<float> &ph, cudaStream_t st)
+cudaError_t launch_stage_mixed2(int p, bool batch, bool fused, const LaunchShape &ls, const StageParams &sp,
+                                const Stage2Args &a, const Phys<float> &ph, cudaStream_t st)
 {
-#define C_(P) (batch ? launch2_p<P, true>(ls, sp, ph, st) : launch2_p<P, false>(ls, sp, ph, st))
+    if (!ls.handoff) {
+        if (p == 3) return alone_launch_p<3>(fused, ls, sp, ph, st);
+        if (p == 5) return alone_launch_p<5>(fused, ls, sp, ph, st);
+        return cudaErrorInvalidValue;
+    }
+    const Stage2 x{reinterpret_cast<const float4 *>(a.ops), a.nodes, a.fin, a.fout, a.rv, a.elem_case, a.first, a.next};
+#define C_(P) (batch ? (fused ? launch2_p<P, true, true>(ls, sp, x, ph, st) : launch2_p<P, true, false>(ls, sp, x, ph, st)) \
+                     : (fused ? launch2_p<P, false, true>(ls, sp, x, ph, st) : launch2_p<P, false, false>(ls, sp, x, ph, st)))
     DG_SWITCH_P(p, C_)
 #undef C_
 }
 
-cudaError_t stage_shape_mixed_fused(int p, int variant, bool batch, long long units, LaunchShape &out)
+cudaError_t stage_shape_mixed_fused(int p, bool batch, long long units, LaunchShape &out)
 {
-#define C_(P) (variant == 2 ? (batch ? fused_shape_p<P, 2, true>(units, out) : fused_shape_p<P, 2, false>(units, out)) \
-                            : (batch ? fused_shape_p<P, 1, true>(units, out) : fused_shape_p<P, 1, false>(units, out)))
+#define C_(P) (batch ? fused_shape_p<P, true>(units, out) : fused_shape_p<P, false>(units, out))
     DG_SWITCH_P(p, C_)
 #undef C_
 }
@@ -279,25 +371,9 @@ cudaError_t stage_shape_mixed_fused(int p, int variant, bool batch, long long un
 cudaError_t launch_stage_mixed_fused(int p, bool batch, const LaunchShape &ls, const StageParams &sp,
                                      const Phys<float> &ph, cudaStream_t st)
 {
-#define C_(P) (ls.variant == 2 ? (batch ? fused_launch_p<P, 2, true>(ls, sp, ph, st)                 \
-                                        : fused_launch_p<P, 2, false>(ls, sp, ph, st))               \
-                               : (batch ? fused_launch_p<P, 1, true>(ls, sp, ph, st)                 \
-                                        : fused_launch_p<P, 1, false>(ls, sp, ph, st)))
+#define C_(P) (batch ? fused_launch_p<P, true>(ls, sp, ph, st) : fused_launch_p<P, false>(ls, sp, ph, st))
     DG_SWITCH_P(p, C_)
 #undef C_
-}
-
-int stage_tile_elems2(int p)
-{
-    switch (p) {
-    case 1: return Shape2<1>::E;
-    case 2: return Shape2<2>::E;
-    case 3: return Shape2<3>::E;
-    case 4: return Shape2<4>::E;
-    case 5: return Shape2<5>::E;
-    case 6: return Shape2<6>::E;
-    default: return 0;
-    }
 }
 
 int stage_tile_elems(int p)
