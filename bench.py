@@ -87,9 +87,10 @@ def algorithmic_bytes_per_step(K, geo_bytes):
 # the sources each mixed stage-kernel shape is compiled from
 KERNEL_FILES = {
     1: ("dg_stage.cuh", "dg_stage_mixed.cuh", "dg_device.cuh", "stage_mixed.cu"),
-    2: ("dg_stage.cuh", "dg_stage_mixed.cuh", "dg_stage_mixed2.cuh", "dg_device.cuh", "stage_mixed.cu"),
-    3: ("dg_stage.cuh", "dg_stage_mixed.cuh", "dg_stage_tc.cuh", "dg_stage_tc_body.inc", "pair2.cuh", "dg_device.cuh",
-        "stage_tc.cu"),
+    2: ("dg_stage.cuh", "dg_stage_mixed.cuh", "dg_stage_handoff.cuh", "dg_stage64.cuh", "bulk.cuh", "dg_device.cuh",
+        "stage_mixed.cu"),
+    3: ("dg_stage.cuh", "dg_stage_mixed.cuh", "dg_stage_tc.cuh", "dg_stage_tc_body.inc", "bulk.cuh", "pair2.cuh",
+        "dg_device.cuh", "stage_tc.cu"),
 }
 
 
@@ -109,9 +110,9 @@ def kernel_hash(variant=2):
     return h.hexdigest()[:16]
 
 
-KERNEL_OF_VARIANT = {1: "dg::stage_mixed_kernel<4, false>", 2: "dg::stage_mixed2_kernel<4, false>",
+KERNEL_OF_VARIANT = {1: "dg::stage_mixed_kernel<4, false>", 2: "dg::stage_handoff_kernel<4, false>",
                      3: "dg::stage_tc_kernel<4, false, false, false>"}
-SHAPE_OF_VARIANT = {1: "one node per thread", 2: "two nodes per thread",
+SHAPE_OF_VARIANT = {1: "one node per thread", 2: "two nodes per thread, volume parts handed from stage to stage",
                     3: "one warp per two elements, tensor-core contractions"}
 
 

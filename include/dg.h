@@ -103,19 +103,22 @@ dg_status dg_set_mesh(dg_ctx *ctx, int64_t Nv, const double *vx, const double *v
 
 /* Tile shape of the mixed-precision stage kernel (no counterpart in the
  * paper): 1 = one volume node and one face node per thread (256 threads),
- * 2 = two volume nodes and two face nodes of one face per thread (128
- * threads; IIP only), 3 = one warp per tile of 2 elements with the Dr / Ds /
+ * 2 = two volume nodes per thread (128 threads; IIP only), each stage but a
+ * step's first taking the divergence and the face records of its input state
+ * from the launch before (single meshes below 25,000 elements at p = 3 and
+ * 15,000 at p = 5: a kernel whose stages stand alone), 3 = one warp per tile of 2 elements with the Dr / Ds /
  * LIFT (and, for theta != 0, Wr / Ws) products on the tensor cores
  * (mma.sync TF32, three products of split operands, about 2^-21 relative;
- * p <= 6), 0 = time every available shape (residual-only launches on the
- * current state) at the first time step after a mesh upload and keep the
- * fastest (the default).  The FP64 path has one kernel and accepts 0 and 1.
+ * p <= 6), 0 = time every available shape (five stage launches each on the
+ * current state, at most 2^21 nodes of it, into buffers that hold nothing) at
+ * the first time step after a mesh upload and keep the fastest (the default).  The FP64 path has one kernel and accepts 0 and 1.
  * The shapes round their FP32 arithmetic differently (all within the mixed
  * path's tolerance), and the tuner's choice depends on timings, so two runs
  * of the same input can differ in the last FP32 bits under variant 0: a
  * fixed variant (1, 2 or 3) is the bit-reproducible mode.
  * Errors: DG_EINVAL (variant outside 0..3), DG_EUNSUPPORTED (2 or 3 on the
- * FP64 path, 2 with theta != 0). */
+ * FP64 path, 2 with theta != 0), DG_ECUDA (2: no memory for what it hands
+ * from stage to stage; the tuner then leaves it out). */
 dg_status dg_set_stage_variant(dg_ctx *ctx, int variant);
 
 /* The tile shape in use: 1, 2 or 3 (the single-node kernel until tuned). */
@@ -151,12 +154,14 @@ dg_status dg_set_fused_steps(dg_ctx *ctx, int on);
  * step's grid barrier, and the tensor-core stage kernel's waits for the bulk
  * copies of its operator table and of each warp's own element records
  * (default 2^24, about 1.7 s; 0 makes every wait give up unless its event
- * has already happened). */
+ * has already happened).  The barriers between the phases of an FP64 stage
+ * and of the two-node kernel's first stage keep the default limit: their
+ * blocks are resident together, so they always end. */
 dg_status dg_set_barrier_limit(dg_ctx *ctx, uint32_t waits);
 
 /* DG_ETIMEOUT if a bounded device wait since the last check gave up -- a
- * grid barrier of a fused step, a copy wait of the tensor-core stage kernel,
- * or a wait of the tcgen05 gradient kernel of dg_broken_gradient -- (then
+ * grid barrier of a fused step or between the phases of a stage, a copy wait
+ * of the tensor-core or two-node stage kernel, or a wait of the tcgen05 gradient kernel of dg_broken_gradient -- (then
  * clears the flag), DG_OK otherwise.  Synchronises when such kernels ran.
  * Errors: DG_EINVAL, DG_ECUDA. */
 dg_status dg_barrier_status(dg_ctx *ctx);
@@ -275,7 +280,8 @@ dg_status dg_wall_forces_noalloc(dg_ctx *ctx, const double xc[2], double out[3])
  * (rx Dr + sx Ds, ry Dr + sy Ds) U on every element, the gradient the
  * residual's viscous fluxes use): gx, gy [K][4][Np] FP64, host pointers if
  * on_device == 0, device pointers (borrowed for the call) otherwise.
- * impl 0: FP64 arithmetic on the CUDA cores.  impl 1: the element products
+ * impl 0: FP64 arithmetic on the CUDA cores (the operators' mirror symmetry
+ * halves its multiply-adds).  impl 1: the element products
  * batched 32 elements to a CTA as (128 x K)(K x 2 Np) products on the
  * fifth-generation tensor cores (tcgen05.mma kind::tf32, three products of
  * split operands, FP32 accumulation in tensor memory) with the FP64 state
