@@ -367,7 +367,7 @@ def run_ours(args):
     roof64 = {"bound": "alu", "achieved": fl64 * v64 / 1e9, "peak": FP64_PEAK_GFLOPS, "unit": "GFLOP/s",
               "frac": fl64 * v64 / 1e9 / FP64_PEAK_GFLOPS,
               "peak_kind": "nominal GB300 FP64 rate (DFMA probe: 1.18-1.20 TFLOP/s)",
-              "flops_per_dof_stage": fl64, "kernel": "dg::stage_kernel<4, double>"}
+              "flops_per_dof_stage": fl64, "kernel": "dg::stage64_kernel<4>"}
 
     # --- the same mixed path with the viscous vortex source (config 2's source
     #     term, S = -div F_v of the advected vortex, one source kernel per stage)

@@ -153,7 +153,7 @@ dt_confirm_kernel(AuxMesh m, Phys<double> ph, double sig_fac, const float *lamS,
 // nodes in node order.  Few faces and long FP64 chains: latency bounds this,
 // so the Np-term sums of a face run side by side instead of one after the
 // other in one thread (120 faces at p = 4: 39 us and a separate 4 us sum
-// before, 8 us in all now).
+// before, 13 us in all now).
 __device__ void wall_face_force(const AuxMesh &m, Phys<double> ph, long long k, int f, const double *xy,
                                 const double *wface, double xc, double yc, double out[3])
 {
@@ -285,7 +285,7 @@ __global__ void nonfinite_kernel(const double *x, long long n, int *flag)
 // of the previous force evaluation (Algorithm 3: F_r = lift / m), giving v_b
 // for the coming RK step.  The scan over a case's elements is a chain of
 // dependent L2 reads per thread: 1024 threads with four reads in flight (18k
-// elements: 26 us with 256 threads and FP64 comparisons, 8 us now).
+// elements: 26 us with 256 threads and FP64 comparisons, 6 us now).
 constexpr int kDtThreads = 1024;
 __global__ void __launch_bounds__(kDtThreads)
 batch_dt_newmark_kernel(const double *lam, const long long *seg, BatchCase *cases, double cfl, const double *fixed)

@@ -20,8 +20,8 @@
 // are ordinary launches.  The price is memory traffic, 52 bytes per DOF and stage
 // from DRAM instead of 45.  Measured, us a stage, the shape that was the fastest
 // before and this one: p = 5, 128^2 quads 71.1 and 62.6; p = 6, 128^2 88.3 and
-// 71.5, 200^2 203 and 164; p = 3, 256^2 112 (one node) and 95; p = 2, 400^2 164
-// and 139.  At p = 4 the tensor-core shape stays ahead (478 and 491 on 512^2).
+// 71.5, 200^2 203 and 164; p = 3, 256^2 112 (one node) and 96; p = 2, 400^2 164
+// and 139.  At p = 4 the tensor-core shape stays ahead (478 and 512 on 512^2).
 // The contractions use the mirror symmetry r <-> s of the operators as in
 // dg_stage64.cuh: a thread owns a pair of mirrored nodes or two nodes of the
 // axis, and half the multiply-adds remain; all lanes are busy at every
@@ -31,8 +31,8 @@
 // not, so fluxes and energy are taken relative to a state of the element, and
 // the inviscid fluxes of the two sides of a face node are formed alike.  RMS
 // error of a residual against 64 bits, rho, rho v1, rho v2, E, in 1e-5: vortex,
-// p = 4: 1.1, 3.1, 1.5, 2.1 (one-node shape 3.0, 7.1, 4.1, 4.6); perturbed free
-// stream around a cylinder, in 1e-7: 4.0, 2.3, 9.6, 6.9 (4.1, 3.0, 16.9, 6.2).
+// p = 4: 0.6, 1.9, 1.0, 2.1 (one-node shape 3.0, 7.1, 4.1, 4.6); perturbed free
+// stream around a cylinder, in 1e-7: 4.0, 2.4, 10.4, 7.0 (4.1, 3.0, 16.9, 6.2).
 #pragma once
 #include "bulk.cuh"
 #include "dg_stage64.cuh"
