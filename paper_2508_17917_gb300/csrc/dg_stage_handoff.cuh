@@ -83,7 +83,8 @@ struct Layout2 {
     static constexpr size_t bytes = header + NG * group;
 };
 
-// barrier of a group, and with the conjunction of a predicate
+// barrier of a group, and with the conjunction of a predicate.  Both order the
+// group's shared-memory accesses; a warp vote alone does not.
 template <int GW>
 __device__ __forceinline__ void group_sync(int g)
 {
@@ -94,7 +95,9 @@ template <int GW>
 __device__ __forceinline__ bool group_and(int g, bool v)
 {
     if constexpr (GW == 1) {
-        return __all_sync(0xffffffffu, v);
+        const bool all = __all_sync(0xffffffffu, v);
+        __syncwarp();
+        return all;
     } else {
         int r;
         asm volatile(
