@@ -4,6 +4,11 @@
 
 namespace dg {
 
+// Waits (about 100 ns each, 1.7 s in all) for copies still in flight after a
+// wait on them gave up: they land in the block's shared memory, so the block
+// stays until they have, whatever limit the caller set for its waits.
+constexpr unsigned kDrainWaits = 1u << 24;
+
 // Bulk copies (the tensor memory accelerator's 1-D form) into shared memory,
 // completing on an mbarrier: the warp's own tile and the operator table.
 __device__ __forceinline__ void mbar_init1(unsigned bar)

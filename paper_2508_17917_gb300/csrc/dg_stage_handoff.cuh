@@ -262,6 +262,7 @@ stage_handoff_kernel(StageParams sp, Stage2 x, Phys<float> ph)
     const double gm1d = sp.gm1;
     float dtr = static_cast<float>(sp.dt);
     unsigned parity = 0;
+    bool failed = false;       // a copy wait of the group gave up: no more tiles, every grid barrier is still met
     __syncthreads();
     pdl_wait_then_release();
 
@@ -375,7 +376,7 @@ stage_handoff_kernel(StageParams sp, Stage2 x, Phys<float> ph)
     // its V runs; the neighbours' traces are read where they are used.
     const bool need_k1 = update && !sp.first_stage;
     auto issue = [&](long long tile) {
-        if (gt >= 32 || tile >= ntiles) return;
+        if (gt >= 32 || tile >= ntiles || failed) return;
         const long long k0 = tile * EB;
         const unsigned ne = static_cast<unsigned>(K - k0 < EB ? K - k0 : EB);
         const unsigned reg = ne * unsigned(sizeof(double) * 4 * Np), nod = ne * unsigned(sizeof(float4) * Np);
@@ -393,7 +394,7 @@ stage_handoff_kernel(StageParams sp, Stage2 x, Phys<float> ph)
         if (gt == 6 && need_k1) bulk_g2s(sbase + unsigned(L::oK1), sp.K1 + k0 * 4 * Np, reg, bar);
     };
     issue(first_tile);
-    for (long long tile = first_tile; tile < ntiles; tile += step, parity ^= 1u) {
+    for (long long tile = first_tile; tile < ntiles && !failed; tile += step, parity ^= 1u) {
         const long long k0 = tile * EB, k = k0 + e;
         const int ne = static_cast<int>(K - k0 < EB ? K - k0 : EB);
         const bool act = e < ne;
@@ -479,10 +480,13 @@ stage_handoff_kernel(StageParams sp, Stage2 x, Phys<float> ph)
             }
         }
         if (!group_and<GW>(grp, ok)) {
-            // a copy wait gave up: the flag, the copies in flight, no more tiles
+            // a copy wait gave up: the flag, then the copies in flight.  They
+            // land in this block's memory, and a fused step goes on to its
+            // grid barriers: the phase of the mbarrier is not used again.
+            failed = true;
             if (gt == 0) {
                 if (sp.bar_err) atomicExch(sp.bar_err, 1);
-                mbar_wait_bounded(bar, parity, 1u << 24);      // they land in this block's memory, whatever the limit
+                mbar_wait_bounded(bar, parity, kDrainWaits);
             }
             break;
         }

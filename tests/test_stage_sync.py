@@ -43,3 +43,16 @@ def test_face_pass_and_update_are_separated_by_it():
     text = source("dg_stage_handoff.cuh")
     write, read = text.index("*slot = to_f4(dH)"), text.index("const float4 *fd = sFD + e * NF;")
     assert write < text.index("group_and<GW>(grp, ok)") < read
+
+
+def test_a_group_that_gave_up_copies_nothing_more():
+    """After a copy wait gave up, the group's mbarrier is a phase behind: in
+    the later stages of a fused step a wait on it would return at once and the
+    block could end with copies still landing in its shared memory.  So the
+    group starts no copy and takes no tile any more."""
+    text = source("dg_stage_handoff.cuh")
+    issue = braced(text, text.index("auto issue = [&](long long tile)"))
+    assert re.search(r"if \([^)]*\bfailed\) return;", issue)
+    assert "tile < ntiles && !failed; tile += step, parity ^= 1u" in text
+    gave_up = braced(text, text.index("if (!group_and<GW>(grp, ok))"))
+    assert re.search(r"\bfailed = true;.*kDrainWaits.*break;", gave_up, re.S)
