@@ -56,3 +56,13 @@ def test_a_group_that_gave_up_copies_nothing_more():
     assert "tile < ntiles && !failed; tile += step, parity ^= 1u" in text
     gave_up = braced(text, text.index("if (!group_and<GW>(grp, ok))"))
     assert re.search(r"\bfailed = true;.*kDrainWaits.*break;", gave_up, re.S)
+
+
+def test_copies_in_flight_are_waited_for_whatever_the_limit():
+    """The limit of dg_set_barrier_limit may be 0.  It bounds the waits of a
+    run, not those for copies that would land in a block that has ended."""
+    text = source("dg_stage_tc_body.inc")
+    drains = [braced(text, text.index("if (failed && tid == 0)")),
+              braced(text, text.index("auto copy_wait_failed"))]
+    for d, n in zip(drains, (1, 2)):
+        assert d.count("kDrainWaits") == n and "bar_limit" not in d
