@@ -22,7 +22,7 @@ struct LaunchShape {
     size_t smem = 0;
     int elems_per_tile = 0;
     bool handoff = false;    // two nodes per thread: the kernel that hands volume parts from stage to stage
-    int per_sm = 0;          // ... and its blocks per SM (4 or 5)
+    int minb = 0;            // ... and which of its builds (handoff_grid.h)
 };
 
 // Launch `kern` with programmatic stream serialization: its blocks may be

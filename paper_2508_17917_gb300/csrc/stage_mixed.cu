@@ -4,6 +4,7 @@
 #include "dg_stage_mixed.cuh"
 #include "dg_stage_handoff.cuh"
 #include "dg_stage_mixed2.cuh"
+#include "handoff_grid.h"
 #include "launch.h"
 
 namespace dg {
@@ -94,57 +95,42 @@ cudaError_t launch_coop(void (*kern)(KArgs...), const LaunchShape &ls, cudaStrea
     return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
-// two nodes per thread (IIP), hand-off kernel: as many blocks as are resident
-// at once (a step's first stage and fused steps have grid barriers), capped by
-// the tiles.  A wave of m blocks per SM takes about m units of time, so of five
-// (96 registers, a few spills) and four (128) the one with the smaller
-// m x waves is taken, four if they are equal.  Measured, us a stage with five
-// and with four, waves: p = 5, 60^2 quads 0.9 and 1.1: 20.5 and 24.9; 76^2 1.4
-// and 1.7: 32.5 and 28.4; 90^2 1.9 and 2.4: 34.4 and 38.7; 100^2 2.4 and 3.0:
-// 46.2 and 39.7; p = 3, 128^2 1.8 and 2.2: 29.8 and 32.3; 256^2 7.2 and 9.0: 98.6
-// and 95.2; p = 1, 256^2 2.7 and 3.4: 36.9 and 39.3.  At p = 6 five spill more
-// and are behind even in one wave against two (56^2: 25.9 and 24.5).
+// two nodes per thread (IIP), hand-off kernel: resident blocks per SM of the
+// build for at least M
 template <int P, bool BATCH, bool FUSE, int M>
-cudaError_t handoff_grid_p(long long K, LaunchShape &ls)
+cudaError_t handoff_occupancy_p(int &per_sm)
 {
-    using S = Sym64<P>;
     using L = Layout2<P>;
     auto kern = stage_handoff_kernel<P, BATCH, FUSE, M>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(L::bytes));
     if (e != cudaSuccess) return e;
-    int per_sm = 0, dev = 0, sms = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, S::NT, L::bytes);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, Sym64<P>::NT, L::bytes);
+    if (e == cudaSuccess && per_sm < 1) e = cudaErrorInvalidConfiguration;
+    return e;
+}
+
+template <int P, bool BATCH, bool FUSE>
+cudaError_t handoff_shape_p(long long K, LaunchShape &ls)
+{
+    using L = Layout2<P>;
+    int occ4 = 0, occ5 = 0, dev = 0, sms = 0;
+    cudaError_t e = handoff_occupancy_p<P, BATCH, FUSE, 4>(occ4);
+    if constexpr (!FUSE && P != 6)
+        if (e == cudaSuccess) e = handoff_occupancy_p<P, BATCH, FUSE, 5>(occ5);
     if (e != cudaSuccess) return e;
-    if (per_sm < 1) return cudaErrorInvalidConfiguration;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const long long per_block = L::EG * L::NG, tiles = (K + per_block - 1) / per_block;
-    const long long grid = static_cast<long long>(sms) * per_sm;
-    const long long cost = per_sm * ((tiles + grid - 1) / grid), have = ls.grid;
-    if (have > 0) {
-        // the shape in ls is the one with four
-        const long long g4 = static_cast<long long>(sms) * ls.per_sm;
-        if (cost >= ls.per_sm * ((tiles + g4 - 1) / g4)) return cudaSuccess;
-    }
-    ls.per_sm = per_sm;
-    ls.grid = static_cast<int>(tiles < grid ? tiles : grid);
-    ls.threads = S::NT;
+    const long long per_block = L::EG * L::NG;
+    const HandoffGrid h = handoff_grid(sms, occ4, occ5, (K + per_block - 1) / per_block);
+    ls.minb = h.minb;
+    ls.grid = h.grid;
+    ls.threads = Sym64<P>::NT;
     ls.smem = L::bytes;
     ls.elems_per_tile = L::EG;
     ls.theta = false;
     ls.variant = 2;
     ls.handoff = true;
     return cudaSuccess;
-}
-
-template <int P, bool BATCH, bool FUSE>
-cudaError_t handoff_shape_p(long long K, LaunchShape &ls)
-{
-    ls.grid = 0;
-    cudaError_t e = handoff_grid_p<P, BATCH, FUSE, 4>(K, ls);
-    if constexpr (!FUSE && P != 6)
-        if (e == cudaSuccess) e = handoff_grid_p<P, BATCH, FUSE, 5>(K, ls);
-    return e;
 }
 
 template <int P, bool BATCH, bool FUSE, int M>
@@ -164,7 +150,7 @@ template <int P, bool BATCH, bool FUSE>
 cudaError_t launch2_p(const LaunchShape &ls, const StageParams &sp, const Stage2 &x, const Phys<float> &ph, cudaStream_t st)
 {
     if constexpr (!FUSE && P != 6)
-        if (ls.per_sm == 5) return handoff_launch_p<P, BATCH, FUSE, 5>(ls, sp, x, ph, st);
+        if (ls.minb == 5) return handoff_launch_p<P, BATCH, FUSE, 5>(ls, sp, x, ph, st);
     return handoff_launch_p<P, BATCH, FUSE, 4>(ls, sp, x, ph, st);
 }
 
