@@ -198,7 +198,9 @@ dg_status dg_lsrk_steps(dg_ctx *ctx, double t, double dt, const double vw[2], in
  * C_inv,2 = p^4 / rho_K^2 with rho_K the inradius, G_K the largest Gbar_e over
  * the faces of K, sigma_K and C_inv,K the largest over its faces, beta_K the
  * largest |b_ns|_2 over its nodes (Eq. cfl_general), beta'_K = 0.
- * Synchronises the stream.  Errors: DG_EINVAL, DG_ENONFINITE, DG_ECUDA. */
+ * Synchronises the stream.  Errors: DG_EINVAL, DG_ENONFINITE (Lambda_K of an
+ * element that can hold the maximum has a term that is not finite: a state
+ * value, 1 / rho, a norm, the sound speed at a negative pressure), DG_ECUDA. */
 dg_status dg_compute_dt(dg_ctx *ctx, double cfl, const double vw[2], double *dt);
 
 /* Force and moment of the fluid on all wall faces (bc == 1): traction

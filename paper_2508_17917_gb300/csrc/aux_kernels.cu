@@ -30,7 +30,22 @@ __device__ __forceinline__ void load_node(const double *U, int Np, long long k, 
 // are spread over the blocks, and works on its candidates eight at a time, a
 // thread per face node and then per node.  The last block to finish writes
 // the maximum and clears the words for the next call.
+//
+// The maxima below drop a NaN, and the penalty norm turns one into zero, so
+// whatever is not finite on the way -- a node's state, its 1 / rho, a norm, a
+// wave speed (a negative pressure has none) -- marks the result instead.
 constexpr int kDtTile = 8;
+
+// by the exponent bits: no FP64 instruction
+__device__ __forceinline__ bool finite64(double x)
+{
+    return (static_cast<unsigned>(__double2hiint(x)) & 0x7ff00000u) != 0x7ff00000u;
+}
+__device__ __forceinline__ bool finite_state(const double u[4], double ir)
+{
+    return finite64(u[0]) && finite64(u[1]) && finite64(u[2]) && finite64(u[3]) && finite64(ir);
+}
+
 __global__ void __launch_bounds__(128)
 dt_confirm_kernel(AuxMesh m, Phys<double> ph, double sig_fac, const float *lamS, unsigned *words, double *out)
 {
@@ -64,6 +79,7 @@ dt_confirm_kernel(AuxMesh m, Phys<double> ph, double sig_fac, const float *lamS,
                 double u[4], w[4];
                 load_node(m.U, Np, k, m.fmask[s], u);
                 const double ir = rcp64(u[0]);
+                bool ok = finite_state(u, ir);
                 const double a = penalty_norm64(ir, u[1] * ir, u[2] * ir, u[3] * ir, n1, n2, ph);
                 double b, rmin = u[0];
                 if (bt == BCT_WALL) {             // wall ghost: the interior density and pressure
@@ -78,9 +94,11 @@ dt_confirm_kernel(AuxMesh m, Phys<double> ph, double sig_fac, const float *lamS,
                         for (int c = 0; c < 4; ++c) w[c] = ph.Uinf[c];
                     }
                     const double iw = rcp64(w[0]);
+                    ok = ok && finite_state(w, iw);
                     b = penalty_norm64(iw, w[1] * iw, w[2] * iw, w[3] * iw, n1, n2, ph);
                     rmin = fmin(rmin, w[0]);
                 }
+                if (!(ok && finite64(a) && finite64(b))) isbad = 1;
                 sG[it] = fmax(a, b);
                 sR[it] = rmin;
             }
@@ -92,7 +110,9 @@ dt_confirm_kernel(AuxMesh m, Phys<double> ph, double sig_fac, const float *lamS,
                 const double pr = ph.gm1 * (u[3] - 0.5 * (u[1] * v1 + u[2] * v2));
                 const double c = sqrt64(ph.gamma * pr * ir);
                 const double b1 = fabs(v1 - ph.vw1) + c, b2 = fabs(v2 - ph.vw2) + c;
-                sB[it] = sqrt64(b1 * b1 + b2 * b2);
+                const double b = sqrt64(b1 * b1 + b2 * b2);
+                sB[it] = b;
+                if (!finite64(b)) isbad = 1;
             }
             __syncthreads();
             if (tid < nc) {
