@@ -5,11 +5,28 @@
 // dt = cfl / max_K Lambda_K needs only the largest Lambda_K, and evaluating
 // every element in FP64 costs about 30 penalty norms per element on a pipe
 // at 1/60 of the FP32 rate.  The screen evaluates Lambda_K in FP32 from the
-// FP64 state; its relative error is below 1e-4 where the guards below hold
-// (the rounding of some tens of FP32 operations), and an element where a guard fails -- a non-finite or
-// extreme value, or a pressure that cancels -- is marked (infinity).  The
-// FP64 pass takes the marked elements and those within 2^-11 of the screen's
-// maximum, so the FP64 maximum over them is the maximum over all elements.
+// FP64 state.  With its values within e of the exact ones, relative, the
+// element with the largest Lambda_K is within (1 - e) / (1 + e) of the
+// screen's maximum; the FP64 pass takes all elements within kDtMargin =
+// 1 - 2^-11 of it, which holds for e <= 2^-12 = 2.4e-4.
+//
+// Lambda_K is formed of sums, products and maxima of positive terms, some
+// tens of roundings of u = 6e-8, except for
+//  - the penalty norm N = |B| of the trace: a41 = -(|v|^2 + vn^2/3) -
+//    gamma/Pr (e - |v|^2) cancels where gamma/Pr > 2.  Its inputs and terms
+//    carry at most 8 u Q, Q = gamma/Pr (e + |v|^2) + 4/3 |v|^2, and an error
+//    of one entry of B is at most that in |B|, so Q <= kDtSpread N bounds the
+//    relative error by 8 u kDtSpread = 4.8e-5; and at the double root of the
+//    eigenvalue's cubic the error of r enters with its square root, 1.5e-4 in
+//    N at most.  Measured over states that pass the guard: 1.3e-5 and
+//    7.0e-5; without the guard 9e-4 (gamma/Pr = 3, speeds of 9e3);
+//  - the sound speed: the pressure's rounding is some u of rho |v|^2 / 2, and
+//    p > 1e-3 rho |v|^2 bounds it by 7e-5 of p, 4e-5 of the speed; for the
+//    wall ghost, whose energy is formed from p, p > 1e-2 rho |v|^2 and
+//    Q <= 4 N give 3e-5 in its norm.
+// An element where a guard fails, or with a value that is not finite or
+// extreme, is marked (infinity) and goes to the FP64 pass, so the FP64
+// maximum over what the pass takes is the maximum over all elements.
 // A uniform state on a uniform mesh marks every element; the FP64 pass then
 // does what a pass over all elements would.
 // 40,800 elements at p = 4: 816 us (one thread per element in FP64, one
@@ -21,6 +38,13 @@
 namespace dg {
 
 constexpr float kDtMargin = 1.0f - 1.0f / 2048.0f;
+constexpr float kDtSpread = 100.0f;
+
+// the size of the terms of one trace's norm, Q / rho
+__device__ __forceinline__ float norm_terms(float ir, float vsq, float e, float gPr)
+{
+    return ir * fmaf(gPr, e + vsq, (4.0f / 3.0f) * vsq);
+}
 
 // words: [0] largest screened Lambda (FP32 bits), [1] finished blocks,
 // [2, 3] largest FP64 Lambda (bits), [4] a candidate was not finite; all zero
@@ -67,12 +91,27 @@ dt_screen_kernel(const double *U, const double *geo, const int4 *conn, const int
             rmin = fminf(rmin, ph.Uinf[0]);
         }
         const float pw = (bt == BCT_WALL) ? pressure<float>(u, Ed, gm1d) : 0.f;
-        const float nrm = trace_norms_max(u, 1.0f / u[0], pw, bt, w, n1, n2, ph);
+        const float ir = 1.0f / u[0];
+        const float nrm = trace_norms_max(u, ir, pw, bt, w, n1, n2, ph);
+        const float msq = u[1] * u[1] + u[2] * u[2];
+        float terms = norm_terms(ir, msq * ir * ir, u[3] * ir, ph.gPr);
+        bool wall_ok = true;
+        if (bt == BCT_WALL) {
+            const float wsq = ph.vw1 * ph.vw1 + ph.vw2 * ph.vw2;
+            const float tw = norm_terms(ir, wsq, fmaf(0.5f, wsq, pw / ph.gm1 * ir), ph.gPr);
+            wall_ok = pw > 1e-2f * (msq * ir) && ph.mu * tw <= 4.0f * nrm;
+        } else {
+            const float r = (bt == BCT_INTERIOR) ? w[0] : ph.Uinf[0], m1 = (bt == BCT_INTERIOR) ? w[1] : ph.Uinf[1];
+            const float m2 = (bt == BCT_INTERIOR) ? w[2] : ph.Uinf[2], E = (bt == BCT_INTERIOR) ? w[3] : ph.Uinf[3];
+            const float iw = 1.0f / r;
+            terms = fmaxf(terms, norm_terms(iw, (m1 * m1 + m2 * m2) * iw * iw, E * iw, ph.gPr));
+        }
         sNorm[fm + fe * NF] = nrm;
         sRmin[fm + fe * NF] = rmin;
         // comparisons written so that a NaN fails them
         const float all = (u[0] + u[1]) + (u[2] + u[3]) + ((bt == BCT_INTERIOR) ? (w[0] + w[1]) + (w[2] + w[3]) : 0.f);
-        const bool ok = rmin > 1e-12f && rmax < 1e12f && nrm < 1e15f && (nrm > 1e-15f || ph.mu == 0.f) && all - all == 0.f;
+        const bool ok = rmin > 1e-12f && rmax < 1e12f && nrm < 1e15f && (nrm > 1e-15f || ph.mu == 0.f) &&
+                        all - all == 0.f && ph.mu * terms <= kDtSpread * nrm && wall_ok;
         if (!ok) sMark[fe] = 1;
     }
     const int ve = tid / Np, vi = tid - (tid / Np) * Np;
@@ -91,7 +130,7 @@ dt_screen_kernel(const double *U, const double *geo, const int4 *conn, const int
         const float b1 = fabsf(v1 - ph.vw1) + c, b2 = fabsf(v2 - ph.vw2) + c;
         const float beta = sqrtf(b1 * b1 + b2 * b2);
         sBeta[ve * Np + vi] = beta;
-        const bool ok = beta > 1e-12f && beta < 1e12f && p > 1e-4f * (u[1] * v1 + u[2] * v2);
+        const bool ok = beta > 1e-12f && beta < 1e12f && p > 1e-3f * (u[1] * v1 + u[2] * v2);
         if (!ok) sMark[ve] = 1;
     }
     __syncthreads();
