@@ -150,19 +150,18 @@ int dg_overint_degree(int p);
  * Errors: DG_EUNSUPPORTED (FP64 or theta != 0), DG_ECUDA. */
 dg_status dg_set_fused_steps(dg_ctx *ctx, int on);
 
-/* Waits of about 100 ns before a bounded device wait gives up: a fused
- * step's grid barrier, and the tensor-core stage kernel's waits for the bulk
- * copies of its operator table and of each warp's own element records
- * (default 2^24, about 1.7 s; 0 makes every wait give up unless its event
- * has already happened).  The barriers between the phases of an FP64 stage
- * and of the two-node kernel's first stage keep the default limit: their
- * blocks are resident together, so they always end. */
+/* Waits of about 100 ns before a bounded device wait gives up: a grid barrier
+ * of a fused step, between the phases of an FP64 stage and in the two-node
+ * kernel's first stage, and the tensor-core and two-node stage kernels' waits
+ * for their bulk copies (default 2^24, about 1.7 s; 0 makes every wait give up
+ * unless its event has already happened). */
 dg_status dg_set_barrier_limit(dg_ctx *ctx, uint32_t waits);
 
 /* DG_ETIMEOUT if a bounded device wait since the last check gave up -- a
  * grid barrier of a fused step or between the phases of a stage, a copy wait
- * of the tensor-core or two-node stage kernel, or a wait of the tcgen05 gradient kernel of dg_broken_gradient -- (then
- * clears the flag), DG_OK otherwise.  Synchronises when such kernels ran.
+ * of the tensor-core or two-node stage kernel, or a wait of the tcgen05
+ * gradient kernel of dg_broken_gradient -- (then clears the flag), DG_OK
+ * otherwise.  Synchronises when such kernels ran.
  * Errors: DG_EINVAL, DG_ECUDA. */
 dg_status dg_barrier_status(dg_ctx *ctx);
 
@@ -180,8 +179,9 @@ dg_status dg_get_state(dg_ctx *ctx, double *U, int on_device);
 
 /* dU/dt = M^-1 R(t, U) of Eq. dg_on_K for the current state, with mesh
  * velocity vw (Sec. 2.1 term v_w (x) U), written to dUdt ([K][4][Np] FP64,
- * host or device).  Uses the context's precision.
- * Errors: DG_EINVAL, DG_ECUDA. */
+ * host or device).  Uses the context's precision.  Host output reports a
+ * bounded device wait that gave up (DG_ETIMEOUT: the residual is not valid).
+ * Errors: DG_EINVAL, DG_ETIMEOUT, DG_ECUDA. */
 dg_status dg_rhs(dg_ctx *ctx, double t, const double vw[2], double *dUdt, int on_device);
 
 /* One time step of Algorithm 1 (five stages, Carpenter-Kennedy 2N-storage

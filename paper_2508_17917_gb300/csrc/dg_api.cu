@@ -114,11 +114,6 @@ struct dg_ctx {
 
 namespace {
 
-// waits of about 100 ns (1.7 s in all) before a grid barrier between the
-// phases of a stage gives up; its blocks are resident together, so a
-// wait is as long as the slowest block's share of a phase
-constexpr unsigned kPhaseWaitLimit = 1u << 24;
-
 const char *const kWaitGaveUp =
     "a bounded device wait gave up (a grid barrier of a fused step or of a stage's phases, or a stage kernel's copy wait: "
     "the state is not valid; or the tcgen05 gradient kernel: its output is not valid)";
@@ -273,7 +268,7 @@ dg_status run_stage(dg_ctx *c, int s, double t, double dt, const double vw[2], i
             // grid barriers between its phases, reported through the barrier flag
             sp.bar = c->bar.ptr;
             sp.bar_err = c->bar_err.ptr;
-            sp.bar_limit = kPhaseWaitLimit;
+            sp.bar_limit = c->bar_limit;
             c->copy_used = true;
         }
         const dg::Stage64Args a64{c->sym64.ptr, c->symn.ptr, c->faces.ptr, c->nfaces, c->flux64.ptr, c->dh64.ptr,
@@ -289,15 +284,14 @@ dg_status run_stage(dg_ctx *c, int s, double t, double dt, const double vw[2], i
             c->copy_used = true;
             e = dg::launch_stage_tc(c->prm.p, false, false, c->shape, sp, make_phys<float>(c->prm, vw), c->stream);
         }
-        else if (c->shape.variant == 2)
-            {
-                sp.bar = c->bar.ptr;
-                sp.bar_err = c->bar_err.ptr;
-                sp.bar_limit = kPhaseWaitLimit;
-                c->copy_used = true;
-                e = dg::launch_stage_mixed2(c->prm.p, false, false, c->shape, sp, stage2_args(c, s),
-                                            make_phys<float>(c->prm, vw), c->stream);
-            }
+        else if (c->shape.variant == 2) {
+            sp.bar = c->bar.ptr;
+            sp.bar_err = c->bar_err.ptr;
+            sp.bar_limit = c->bar_limit;
+            c->copy_used = true;
+            e = dg::launch_stage_mixed2(c->prm.p, false, false, c->shape, sp, stage2_args(c, s),
+                                        make_phys<float>(c->prm, vw), c->stream);
+        }
         else
             e = dg::launch_stage_mixed(c->prm.p, c->shape, sp, make_phys<float>(c->prm, vw), c->stream);
     }
@@ -800,8 +794,17 @@ dg_status dg_rhs(dg_ctx *c, double t, const double vw[2], double *dUdt, int on_d
     dg_status st = run_stage(c, -1, t, 0.0, vw, dg::STAGE_RHS_ONLY, c->cur(), nullptr, out);
     if (st != DG_OK) return st;
     if (!on_device) {
+        // the error flag of the bounded device waits comes back with the residual
+        const bool check = c->bar_used || c->copy_used;
+        int e = 0;
+        if (check) DG_CUDA(c, cudaMemcpyAsync(&e, c->bar_err.ptr, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
         DG_CUDA(c, cudaMemcpyAsync(dUdt, out, ndof(c) * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
         DG_CUDA(c, cudaStreamSynchronize(c->stream));
+        if (check) {
+            c->bar_used = false;
+            c->copy_used = false;
+            if (e) return wait_gave_up(c);
+        }
     }
     return DG_OK;
 }
