@@ -44,6 +44,7 @@ struct dg_ctx {
     // device
     // FP64 and two-node kernels: symmetric operator tables, every face once, arrays between phases
     dg::DevBuf<double> sym64, flux64, dh64, th64;
+    bool no_coop = false;     // the stream refused the FP64 kernel's grid as a cooperative launch
     dg::DevBuf<float> sym32;
     dg::DevBuf<float4> fd32, rv32;
     dg::DevBuf<int> symn, symn32;
@@ -92,6 +93,13 @@ struct dg_ctx {
     // finished blocks of the wall-force kernel: the last word of scal
     unsigned *ticket() { return reinterpret_cast<unsigned *>(scal.ptr + 3); }
     cudaEvent_t tune_ev[9] = {};     // mixed: marks of the stage-shape timing
+    void drop_phases()
+    {
+        flux64.release();
+        dh64.release();
+        th64.release();
+        faces.release();
+    }
     ~dg_ctx()
     {
         for (auto &e : tune_ev)
@@ -193,6 +201,58 @@ void manufactured_source(double x, double y, double kappa, double C2, const dg_p
 // C1 (1+theta)^2 (d+1) of Eq. penalty_final, d = 2
 double sigma_factor(const dg_params &p) { return p.C1 * (1.0 + p.theta) * (1.0 + p.theta) * 3.0; }
 
+// What the three-phase FP64 kernel keeps between its phases, for a mesh with
+// connectivity `conn` (host; null: read back).  Over-integration does not run
+// it; without memory for it, or where the stream refused its grid, the mesh
+// runs with the kernel that needs none.
+dg_status phase_arrays(dg_ctx *c, const int4 *conn)
+{
+    if (c->overint || c->no_coop) {
+        c->drop_phases();
+        return DG_OK;
+    }
+    if (c->flux64.ptr) return DG_OK;
+    std::vector<int4> back, fl;
+    if (!conn) {
+        back.resize(c->K);
+        DG_CUDA(c, cudaMemcpy(back.data(), c->conn.ptr, c->K * sizeof(int4), cudaMemcpyDeviceToHost));
+        conn = back.data();
+    }
+    dg::unique_faces(conn, c->K, fl);
+    c->nfaces = static_cast<int>(fl.size());
+    const size_t nd = static_cast<size_t>(c->K) * 4 * c->ops.Np, nfn = static_cast<size_t>(c->K) * 3 * c->ops.Nfp;
+    cudaError_t e = c->faces.alloc(fl.size());
+    if (e == cudaSuccess) e = c->dh64.alloc(4 * nfn);
+    if (e == cudaSuccess && c->prm.theta != 0.0) e = c->th64.alloc(8 * nfn);
+    if (e == cudaSuccess) e = c->flux64.alloc(2 * nd);
+    if (e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        c->drop_phases();
+        return DG_OK;
+    }
+    DG_CUDA(c, e);
+    DG_CUDA(c, cudaMemcpy(c->faces.ptr, fl.data(), fl.size() * sizeof(int4), cudaMemcpyHostToDevice));
+    return DG_OK;
+}
+
+cudaError_t shape_fp64(dg_ctx *c)
+{
+    return dg::stage_shape_fp64(c->prm.p, c->K, c->prm.theta != 0.0, c->shape, c->overint, c->flux64.ptr != nullptr);
+}
+
+// An array that a call needs.  Where there is no memory for it, the arrays that
+// only make a kernel faster go first.
+template <typename T>
+cudaError_t alloc_needed(dg_ctx *c, dg::DevBuf<T> &b, size_t n)
+{
+    cudaError_t e = b.alloc(n);
+    if (e != cudaErrorMemoryAllocation || !c->flux64.ptr) return e;
+    cudaGetLastError();
+    c->drop_phases();                  // cudaFree waits for the kernels that use them
+    e = shape_fp64(c);
+    return e == cudaSuccess ? b.alloc(n) : e;
+}
+
 // what the two-node kernel hands from stage to stage; a mesh that leaves no
 // memory for it runs with the other shapes
 cudaError_t two_node_arrays(dg_ctx *c)
@@ -264,7 +324,7 @@ dg_status run_stage(dg_ctx *c, int s, double t, double dt, const double vw[2], i
     if (c->prm.precision == DG_PRECISION_FP64) {
         sp.geo = c->geo64.ptr;
         sp.ops = c->ops64.ptr;
-        if (!c->shape.overint) {
+        if (c->shape.phases) {
             // grid barriers between its phases, reported through the barrier flag
             sp.bar = c->bar.ptr;
             sp.bar_err = c->bar_err.ptr;
@@ -273,7 +333,15 @@ dg_status run_stage(dg_ctx *c, int s, double t, double dt, const double vw[2], i
         }
         const dg::Stage64Args a64{c->sym64.ptr, c->symn.ptr, c->faces.ptr, c->nfaces, c->flux64.ptr, c->dh64.ptr,
                                   c->th64.ptr};
-        e = dg::launch_stage_fp64(c->prm.p, c->shape, sp, a64, make_phys<double>(c->prm, vw), c->stream);
+        const dg::Phys<double> ph = make_phys<double>(c->prm, vw);
+        e = dg::launch_stage_fp64(c->prm.p, c->shape, sp, a64, ph, c->stream);
+        if (e == cudaErrorCooperativeLaunchTooLarge) {
+            // the grid is sized for the whole device, and the stream has a part of it
+            cudaGetLastError();
+            c->no_coop = true;
+            e = dg::stage_shape_fp64(c->prm.p, c->K, c->prm.theta != 0.0, c->shape, c->overint, false);
+            if (e == cudaSuccess) e = dg::launch_stage_fp64(c->prm.p, c->shape, sp, a64, ph, c->stream);
+        }
     } else {
         sp.geo = c->geo32.ptr;
         sp.ops = (c->shape.variant == 3) ? static_cast<const void *>(c->tcfrag.ptr) : c->ops32.ptr;
@@ -460,7 +528,9 @@ dg_status dg_set_overintegration(dg_ctx *c, int on)
         return fail(c, DG_EUNSUPPORTED, "over-integration is implemented in the FP64 IIP kernel");
     c->overint = on != 0;
     if (c->K > 0 && c->prm.precision == DG_PRECISION_FP64) {
-        cudaError_t e = dg::stage_shape_fp64(c->prm.p, c->K, false, c->shape, c->overint);
+        dg_status st = phase_arrays(c, nullptr);
+        if (st != DG_OK) return st;
+        cudaError_t e = shape_fp64(c);
         if (e != cudaSuccess) return cuda_fail(c, e, "stage kernel configuration");
     }
     return DG_OK;
@@ -543,6 +613,7 @@ dg_status dg_set_mesh(dg_ctx *c, int64_t Nv, const double *vx, const double *vy,
     std::vector<int2> &walls = ma.walls;
     std::vector<double> &wxy = ma.wxy;
     // --- device buffers
+    c->drop_phases();
     c->K = K;
     const size_t nd = static_cast<size_t>(K) * 4 * Np;
     DG_CUDA(c, c->K0a.alloc(nd));
@@ -553,17 +624,6 @@ dg_status dg_set_mesh(dg_ctx *c, int64_t Nv, const double *vx, const double *vy,
     DG_CUDA(c, c->lam.alloc(K));
     DG_CUDA(c, cudaMemcpy(c->geo64.ptr, geo.data(), geo.size() * sizeof(double), cudaMemcpyHostToDevice));
     DG_CUDA(c, cudaMemcpy(c->conn.ptr, conn.data(), K * sizeof(int4), cudaMemcpyHostToDevice));
-    if (c->prm.precision == DG_PRECISION_FP64) {
-        std::vector<int4> fl;
-        dg::unique_faces(conn.data(), K, fl);
-        c->nfaces = static_cast<int>(fl.size());
-        DG_CUDA(c, c->faces.alloc(fl.size()));
-        DG_CUDA(c, cudaMemcpy(c->faces.ptr, fl.data(), fl.size() * sizeof(int4), cudaMemcpyHostToDevice));
-        const size_t nfn = static_cast<size_t>(K) * 3 * c->ops.Nfp;
-        DG_CUDA(c, c->flux64.alloc(2 * nd));
-        DG_CUDA(c, c->dh64.alloc(4 * nfn));
-        if (c->prm.theta != 0.0) DG_CUDA(c, c->th64.alloc(8 * nfn));
-    }
     {
         dg_status bs = need_barrier(c);
         if (bs != DG_OK) return bs;
@@ -605,8 +665,11 @@ dg_status dg_set_mesh(dg_ctx *c, int64_t Nv, const double *vx, const double *vy,
     c->geo64h.swap(geo);
     c->source_kind = DG_SOURCE_NONE;
     const bool th = c->prm.theta != 0.0;
-    cudaError_t e = (c->prm.precision == DG_PRECISION_FP64) ? dg::stage_shape_fp64(c->prm.p, K, th, c->shape, c->overint)
-                                                             : dg::stage_shape_mixed(c->prm.p, K, th, c->shape);
+    if (c->prm.precision == DG_PRECISION_FP64) {
+        dg_status ps = phase_arrays(c, conn.data());
+        if (ps != DG_OK) return ps;
+    }
+    cudaError_t e = (c->prm.precision == DG_PRECISION_FP64) ? shape_fp64(c) : dg::stage_shape_mixed(c->prm.p, K, th, c->shape);
     if (e != cudaSuccess) return cuda_fail(c, e, "stage kernel configuration");
     c->shape1 = c->shape;
     c->tuned = false;
@@ -710,11 +773,11 @@ dg_status dg_set_source(dg_ctx *c, int kind, const double *params)
         c->vortex = dg::VortexSource{params[0], params[1], params[2], params[3], params[4], params[5],
                                      c->prm.mu, c->prm.Pr, 1.0 / params[3], params[0] / (2.0 * pi),
                                      params[0] * params[0] / (2.0 * pi * pi), 1.0 / c->prm.Pr};
-        DG_CUDA(c, c->src_xy.alloc(2 * x.size()));
+        DG_CUDA(c, alloc_needed(c, c->src_xy, 2 * x.size()));
         DG_CUDA(c, cudaMemcpy(c->src_xy.ptr, x.data(), x.size() * sizeof(double), cudaMemcpyHostToDevice));
         DG_CUDA(c, cudaMemcpy(c->src_xy.ptr + x.size(), y.data(), y.size() * sizeof(double),
                               cudaMemcpyHostToDevice));
-        DG_CUDA(c, c->src.alloc(5 * ndof(c)));         // one array per stage time of a step
+        DG_CUDA(c, alloc_needed(c, c->src, 5 * ndof(c)));         // one array per stage time of a step
         c->source_kind = kind;
         return DG_OK;
     }
@@ -725,7 +788,7 @@ dg_status dg_set_source(dg_ctx *c, int kind, const double *params)
             manufactured_source(x[k * Np + i], y[k * Np + i], params[0], params[1], c->prm, s4);
             for (int q = 0; q < 4; ++q) S[(k * 4 + q) * Np + i] = s4[q];
         }
-    DG_CUDA(c, c->src.alloc(S.size()));
+    DG_CUDA(c, alloc_needed(c, c->src, S.size()));
     DG_CUDA(c, cudaMemcpy(c->src.ptr, S.data(), S.size() * sizeof(double), cudaMemcpyHostToDevice));
     c->source_kind = kind;
     return DG_OK;
@@ -788,7 +851,7 @@ dg_status dg_rhs(dg_ctx *c, double t, const double vw[2], double *dUdt, int on_d
     if (!dUdt || c->K < 1) return fail(c, DG_EINVAL, "null output or no mesh");
     double *out = dUdt;
     if (!on_device) {
-        if (c->rtmp.n != ndof(c)) DG_CUDA(c, c->rtmp.alloc(ndof(c)));
+        if (c->rtmp.n != ndof(c)) DG_CUDA(c, alloc_needed(c, c->rtmp, ndof(c)));
         out = c->rtmp.ptr;
     }
     dg_status st = run_stage(c, -1, t, 0.0, vw, dg::STAGE_RHS_ONLY, c->cur(), nullptr, out);
@@ -965,7 +1028,7 @@ dg_status dg_broken_gradient(dg_ctx *c, double *gx, double *gy, int on_device, i
     const size_t n = ndof(c);
     double *ox = gx, *oy = gy;
     if (!on_device) {
-        if (c->gtmp.n != 2 * n) DG_CUDA(c, c->gtmp.alloc(2 * n));
+        if (c->gtmp.n != 2 * n) DG_CUDA(c, alloc_needed(c, c->gtmp, 2 * n));
         ox = c->gtmp.ptr;
         oy = c->gtmp.ptr + n;
     }
@@ -984,7 +1047,7 @@ dg_status dg_broken_gradient(dg_ctx *c, double *gx, double *gy, int on_device, i
         a.wait_limit = 1u << 20;
         const size_t nf = dg::grad_tc05_bimg_floats(c->prm.p);
         if (c->gimg.n != nf) {
-            DG_CUDA(c, c->gimg.alloc(nf));
+            DG_CUDA(c, alloc_needed(c, c->gimg, nf));
             c->gimg_ready = false;
         }
         a.bimg = c->gimg.ptr;

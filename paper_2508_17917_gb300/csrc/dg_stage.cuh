@@ -1,14 +1,26 @@
 // dg_stage.cuh -- what every stage kernel shares (parameters, tile shapes,
-// geometry records), and the FP64 stage kernel with the over-integrated
-// volume term.
+// geometry records), and the FP64 stage kernel that needs no memory of its
+// own: the one with the over-integrated volume term, and the one that a mesh
+// takes whose arrays between the phases of dg_stage64.cuh find no memory, or
+// whose stream cannot hold that kernel's grid at once.
 //
 // One launch evaluates, for every element, the nodal residual of Eq. dg_on_K
-//     dU/dt = M^-1 sum_q w_q grad l(x_q) . F_q - LIFT (Fscale H)
-// with F = F_c - v_w (x) U - G(U) grad_h U (Sec. 2.1) at the points of a
-// cubature rule, H the Roe + interior-penalty face flux with the penalty of
-// Eq. penalty_final (theta = 0), and then applies one stage of Algorithm 1:
-// K1 <- A K1 + dt R;  K0_out <- K0_in + B K1.  (Without over-integration the
-// FP64 path runs dg_stage64.cuh in the strong form.)
+// in strong form
+//     dU/dt = -(rx Dr + sx Ds) F_x - (ry Dr + sy Ds) F_y + LIFT (Fscale (F.n - H))
+// with F = F_c - v_w (x) U - G(U) grad_h U (Sec. 2.1), H the Roe + interior-
+// penalty face flux with the penalty of Eq. penalty_final, and then applies
+// one stage of Algorithm 1:  K1 <- A K1 + dt R;  K0_out <- K0_in + B K1.
+// For theta != 0 (SIP, NIPG) the terms -S_x H_theta,x - S_y H_theta,y of
+// Eq. dg_on_K add
+//     Wr (rx Lx + ry Ly) + Ws (sx Lx + sy Ly),  L_l = LIFT (Fscale theta w t_l),
+// with Wr = M^-1 Dr^T M, Ws = M^-1 Ds^T M, t_l the theta vector of each face
+// node (theta_vec) and w = 1/2 on interior faces (the average), 1 on boundary
+// faces; G is taken at U+ on interior and far-field faces, at U^b on walls.
+// (The strong form equals the paper's weak form exactly for collocated
+// fluxes on affine elements: the weak volume term integrated by parts gives
+// the strong divergence plus the lifted interior trace F.n.)
+// Over-integrated (theta = 0): M^-1 sum_q w_q grad l(x_q) . F_q - LIFT (Fscale H)
+// with the flux at the points of a cubature rule.
 //
 // Work decomposition: a CTA of NT threads owns a tile of E elements at a
 // time (persistent loop over tiles).  Thread t is volume node (t / Np, t % Np)
@@ -118,50 +130,58 @@ struct OIShape {
     static constexpr int Nq = N * N;
 };
 
-template <int P, typename real>
+template <int P, typename real, bool TH = false, bool OI = false>
 struct Smem {
     using S = Shape<P>;
     static constexpr int Np = S::Np, NF = S::NF, E = S::E;
-    static constexpr int Nq = OIShape<P>::Nq;
+    static constexpr int Nq = OI ? OIShape<P>::Nq : 0;
     // sizes in elements of `real`
-    static constexpr int ops = 2 * Np * Np + Np * NF;
+    static constexpr int ops = 2 * Np * Np + Np * NF + (TH ? 2 * Np * Np : 0);
     static constexpr int oiops = 5 * Nq * Np;           // Vq, Vqr, Vqs [Nq][Np]; Sr, Ss [Np][Nq]
     static constexpr int fq = 2 * E * 4 * Nq;           // contravariant fluxes at the cubature points
     static constexpr int u = E * 4 * Np;
     static constexpr int gx = E * 4 * Np;
     static constexpr int gy = E * 4 * Np;
+    static constexpr int fr = OI ? 0 : E * 4 * Np;
+    static constexpr int fs = OI ? 0 : E * 4 * Np;
     static constexpr int pr = E * Np;
     static constexpr int nb = E * 3 * 4 * Np;
     static constexpr int norm = E * NF;
     static constexpr int dh = E * NF * 4;
     static constexpr int geo = E * 16;
     static constexpr int ngeo = E * 3 * 8;
-    static constexpr int total_real = ops + u + gx + gy + pr + nb + norm + dh + geo + ngeo + oiops + fq;
+    static constexpr int th = TH ? E * NF * 8 : 0;
+    static constexpr int total_real = ops + u + gx + gy + fr + fs + pr + nb + norm + dh + geo + ngeo + th + oiops + fq;
     static constexpr size_t bytes = total_real * sizeof(real) + NF * sizeof(int) + 16;
 };
 
-template <int P, typename real>
+template <int P, typename real, bool TH, bool OI = false>
 __global__ void __launch_bounds__(Shape<P>::NT)
 stage_kernel(StageParams sp, Phys<real> ph)
 {
     using S = Shape<P>;
     constexpr int Np = S::Np, Nfp = S::Nfp, NF = S::NF, E = S::E, NT = S::NT;
-    using L = Smem<P, real>;
+    using L = Smem<P, real, TH, OI>;
     constexpr int Nq = L::Nq;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     real *sDr = reinterpret_cast<real *>(smem_raw);
     real *sDs = sDr + Np * Np;
     real *sLIFT = sDs + Np * Np;
+    real *sWr = sLIFT + Np * NF;               // theta variant only
+    real *sWs = sWr + Np * Np;
     real *sU = sDr + L::ops;
     real *sGx = sU + L::u;
     real *sGy = sGx + L::gx;
-    real *sP = sGy + L::gy;
+    real *sFr = sGy + L::gy;
+    real *sFs = sFr + L::fr;
+    real *sP = sFs + L::fs;
     real *sN = sP + L::pr;
     real *sNorm = sN + L::nb;
     real *sDH = sNorm + L::norm;
     real *sGeo = sDH + L::dh;
     real *sNGeo = sGeo + L::geo;
-    real *sVq = sNGeo + L::ngeo;               // Vq | Vqr | Vqs | Sr | Ss
+    real *sTH = sNGeo + L::ngeo;               // theta variant: Fscale theta w (t_x, t_y)
+    real *sVq = sTH + L::th;                   // over-integration: Vq | Vqr | Vqs | Sr | Ss
     real *sVqr = sVq + Nq * Np;
     real *sVqs = sVqr + Nq * Np;
     real *sSr = sVqs + Nq * Np;
@@ -174,9 +194,11 @@ stage_kernel(StageParams sp, Phys<real> ph)
         const real *ops = static_cast<const real *>(sp.ops);
         for (int i = tid; i < L::ops; i += NT) sDr[i] = ops[i];
         for (int i = tid; i < NF; i += NT) sFm[i] = sp.fmask[i];
-        // the operator buffer holds Dr | Ds | LIFT | Wr | Ws | Vq | Vqr | Vqs | Sr | Ss
-        const real *oi = ops + 4 * Np * Np + Np * NF;
-        for (int i = tid; i < L::oiops; i += NT) sVq[i] = oi[i];
+        if constexpr (OI) {
+            // the operator buffer holds Dr | Ds | LIFT | Wr | Ws | Vq | Vqr | Vqs | Sr | Ss
+            const real *oi = ops + 4 * Np * Np + Np * NF;
+            for (int i = tid; i < L::oiops; i += NT) sVq[i] = oi[i];
+        }
     }
     const real *geo = static_cast<const real *>(sp.geo);
     const long long K = sp.K;
@@ -184,6 +206,7 @@ stage_kernel(StageParams sp, Phys<real> ph)
     const double gm1d = sp.gm1;
     const real p1 = real(P + 1), p2 = real(P + 2);
     const real sig_fac = static_cast<real>(sp.sig_fac);
+    const real theta = static_cast<real>(sp.theta);
 
     for (long long tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
         const long long k0 = tile * E;
@@ -245,40 +268,53 @@ stage_kernel(StageParams sp, Phys<real> ph)
             double Ed = sp.K0in[((k0 + ve) * 4 + 3) * Np + vi];
             real p = pressure<real>(u, Ed, gm1d);
             sP[ve * Np + vi] = p;
+            if constexpr (!OI) {
+                real cx[4], cy[4], vx[4], vy[4];
+                adv_flux(u, p, ph, cx, cy);
+                visc_flux(u, gxv, gyv, ph, vx, vy);
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    real Fx = cx[c] - vx[c], Fy = cy[c] - vy[c];
+                    sFr[(ve * 4 + c) * Np + vi] = rx * Fx + ry * Fy;
+                    sFs[(ve * 4 + c) * Np + vi] = sx * Fx + sy * Fy;
+                }
+            }
         }
-        // flux at the cubature points from the state and broken gradient
-        // interpolated there (the polynomial U_h itself, not nodal values)
-        if (vol) {
-            const real *u_e = sU + ve * 4 * Np;
-            const real *g = sGeo + ve * 16;
-            const real rx = g[G_RX], ry = g[G_RY], sx = g[G_SX], sy = g[G_SY];
-            for (int q = vi; q < Nq; q += Np) {
-                real u[4] = {0, 0, 0, 0}, ur[4] = {0, 0, 0, 0}, us[4] = {0, 0, 0, 0};
-                for (int j = 0; j < Np; ++j) {
-                    const real a = sVq[q * Np + j], b = sVqr[q * Np + j], d = sVqs[q * Np + j];
+        if constexpr (OI) {
+            // flux at the cubature points from the state and broken gradient
+            // interpolated there (the polynomial U_h itself, not nodal values)
+            if (vol) {
+                const real *u_e = sU + ve * 4 * Np;
+                const real *g = sGeo + ve * 16;
+                const real rx = g[G_RX], ry = g[G_RY], sx = g[G_SX], sy = g[G_SY];
+                for (int q = vi; q < Nq; q += Np) {
+                    real u[4] = {0, 0, 0, 0}, ur[4] = {0, 0, 0, 0}, us[4] = {0, 0, 0, 0};
+                    for (int j = 0; j < Np; ++j) {
+                        const real a = sVq[q * Np + j], b = sVqr[q * Np + j], d = sVqs[q * Np + j];
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) {
+                            const real uj = u_e[c * Np + j];
+                            u[c] += a * uj;
+                            ur[c] += b * uj;
+                            us[c] += d * uj;
+                        }
+                    }
+                    real gxq[4], gyq[4];
 #pragma unroll
                     for (int c = 0; c < 4; ++c) {
-                        const real uj = u_e[c * Np + j];
-                        u[c] += a * uj;
-                        ur[c] += b * uj;
-                        us[c] += d * uj;
+                        gxq[c] = rx * ur[c] + sx * us[c];
+                        gyq[c] = ry * ur[c] + sy * us[c];
                     }
-                }
-                real gxq[4], gyq[4];
+                    const real pq = pressure<real>(u, to_f64<real>(u[3]), gm1d);
+                    real cx[4], cy[4], vx[4], vy[4];
+                    adv_flux(u, pq, ph, cx, cy);
+                    visc_flux(u, gxq, gyq, ph, vx, vy);
 #pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    gxq[c] = rx * ur[c] + sx * us[c];
-                    gyq[c] = ry * ur[c] + sy * us[c];
-                }
-                const real pq = pressure<real>(u, to_f64<real>(u[3]), gm1d);
-                real cx[4], cy[4], vx[4], vy[4];
-                adv_flux(u, pq, ph, cx, cy);
-                visc_flux(u, gxq, gyq, ph, vx, vy);
-#pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    const real Fx = cx[c] - vx[c], Fy = cy[c] - vy[c];
-                    sFq[((ve * 4 + c) * Nq + q) * 2] = rx * Fx + ry * Fy;
-                    sFq[((ve * 4 + c) * Nq + q) * 2 + 1] = sx * Fx + sy * Fy;
+                    for (int c = 0; c < 4; ++c) {
+                        const real Fx = cx[c] - vx[c], Fy = cy[c] - vy[c];
+                        sFq[((ve * 4 + c) * Nq + q) * 2] = rx * Fx + ry * Fy;
+                        sFq[((ve * 4 + c) * Nq + q) * 2 + 1] = sx * Fx + sy * Fy;
+                    }
                 }
             }
         }
@@ -323,13 +359,25 @@ stage_kernel(StageParams sp, Phys<real> ph)
 
         // ---- P3: divergence (volume) and face flux (face nodes)
         real R[4] = {0, 0, 0, 0};
-        if (vol) {
-            // weak volume term: sum_q Sr_iq Fr_q + Ss_iq Fs_q (Sr = M^-1 Vqr^T W)
-            const real *fq = sFq + ve * 4 * Nq * 2;
-            for (int q = 0; q < Nq; ++q) {
-                const real a = sSr[vi * Nq + q], b = sSs[vi * Nq + q];
+        if (vol && !OI) {
+            const real *fr = sFr + ve * 4 * Np;
+            const real *fs = sFs + ve * 4 * Np;
 #pragma unroll
-                for (int c = 0; c < 4; ++c) R[c] += a * fq[(c * Nq + q) * 2] + b * fq[(c * Nq + q) * 2 + 1];
+            for (int j = 0; j < Np; ++j) {
+                real dr = sDr[vi * Np + j], ds = sDs[vi * Np + j];
+#pragma unroll
+                for (int c = 0; c < 4; ++c) R[c] -= dr * fr[c * Np + j] + ds * fs[c * Np + j];
+            }
+        }
+        if constexpr (OI) {
+            // weak volume term: sum_q Sr_iq Fr_q + Ss_iq Fs_q (Sr = M^-1 Vqr^T W)
+            if (vol) {
+                const real *fq = sFq + ve * 4 * Nq * 2;
+                for (int q = 0; q < Nq; ++q) {
+                    const real a = sSr[vi * Nq + q], b = sSs[vi * Nq + q];
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) R[c] += a * fq[(c * Nq + q) * 2] + b * fq[(c * Nq + q) * 2 + 1];
+                }
             }
         }
         if (face) {
@@ -359,6 +407,12 @@ stage_kernel(StageParams sp, Phys<real> ph)
             flux_n(up, pp, n1, n2, ph, Fnp);
             visc_flux(up, gxp, gyp, ph, vxp, vyp);
             real dH[4];
+            // theta term inputs: jump U+ - U-, the state G is taken at, weight
+            real jmp[4], gs[4], wth = real(1);
+            {
+                const real ir = real(1) / up[0];
+                gs[0] = up[0]; gs[1] = up[1] * ir; gs[2] = up[2] * ir; gs[3] = up[3] * ir;
+            }
             if (btype == BCT_INTERIOR) {
                 const real *w = sN + (fe * 3 + ff) * 4 * Np;
                 const real *ng = sNGeo + (fe * 3 + ff) * 8;
@@ -386,6 +440,9 @@ stage_kernel(StageParams sp, Phys<real> ph)
                 flux_n(um, pm, n1, n2, ph, Fnm);
                 visc_flux(um, gxm, gym, ph, vxm, vym);
                 roe_dissipation(up, pp, um, pm, n1, n2, ph, D);
+                wth = real(0.5);
+#pragma unroll
+                for (int c = 0; c < 4; ++c) jmp[c] = up[c] - um[c];
 #pragma unroll
                 for (int c = 0; c < 4; ++c) {
                     real vnp = vxp[c] * n1 + vyp[c] * n2, vnm = vxm[c] * n1 + vym[c] * n2;
@@ -399,8 +456,10 @@ stage_kernel(StageParams sp, Phys<real> ph)
                 roe_dissipation(up, pp, ub, ph.pinf, n1, n2, ph, D);
                 // H = Roe - G(U+) grad U+ . n + sigma (U+ - Ub); F+.n - H:
 #pragma unroll
-                for (int c = 0; c < 4; ++c)
+                for (int c = 0; c < 4; ++c) {
                     dH[c] = real(0.5) * (Fnp[c] - Fnb[c]) - real(0.5) * D[c] - sigma * (up[c] - ub[c]);
+                    jmp[c] = up[c] - ub[c];
+                }
             } else {
                 // wall: U^b from Q^b = (rho+, v_w, p+); H = n.(F_c - v_w U)(U^b)
                 //       - G(U^b) grad U+ . n + sigma (U+ - U^b)
@@ -418,13 +477,27 @@ stage_kernel(StageParams sp, Phys<real> ph)
                 for (int c = 0; c < 4; ++c) {
                     real vnp = vxp[c] * n1 + vyp[c] * n2;
                     dH[c] = (Fnp[c] - vnp) - (Fnb[c] - vnb[c] + sigma * (up[c] - ub[c]));
+                    jmp[c] = up[c] - ub[c];
                 }
+                gs[0] = rb; gs[1] = ph.vw1; gs[2] = ph.vw2; gs[3] = ub[3] / rb;
             }
-            // weak form: the face term is -H itself, without the F+.n of the strong form
+            if constexpr (OI) {
+                // weak form: the face term is -H itself, without the F+.n of the strong form
 #pragma unroll
-            for (int c = 0; c < 4; ++c) dH[c] -= Fnp[c] - (vxp[c] * n1 + vyp[c] * n2);
+                for (int c = 0; c < 4; ++c) dH[c] -= Fnp[c] - (vxp[c] * n1 + vyp[c] * n2);
+            }
 #pragma unroll
             for (int c = 0; c < 4; ++c) sDH[(fe * NF + fm) * 4 + c] = fsc * dH[c];
+            if constexpr (TH) {
+                real tx[4], ty[4];
+                theta_vec(gs[0], gs[1], gs[2], gs[3], jmp, n1, n2, ph, tx, ty);
+                const real sc = theta * wth * fsc;
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    sTH[(fe * NF + fm) * 8 + c] = sc * tx[c];
+                    sTH[(fe * NF + fm) * 8 + 4 + c] = sc * ty[c];
+                }
+            }
         }
         __syncthreads();
 
@@ -436,6 +509,39 @@ stage_kernel(StageParams sp, Phys<real> ph)
                 real l = sLIFT[vi * NF + m];
 #pragma unroll
                 for (int c = 0; c < 4; ++c) R[c] += l * dh[m * 4 + c];
+            }
+        }
+        if constexpr (TH) {
+            // lift the theta vectors, map to (r, s) and park them in the flux slots
+            if (vol) {
+                const real *th = sTH + ve * NF * 8;
+                real Lx[4] = {0, 0, 0, 0}, Ly[4] = {0, 0, 0, 0};
+#pragma unroll
+                for (int m = 0; m < NF; ++m) {
+                    const real l = sLIFT[vi * NF + m];
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        Lx[c] += l * th[m * 8 + c];
+                        Ly[c] += l * th[m * 8 + 4 + c];
+                    }
+                }
+                const real *g = sGeo + ve * 16;
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    sFr[(ve * 4 + c) * Np + vi] = g[G_RX] * Lx[c] + g[G_RY] * Ly[c];
+                    sFs[(ve * 4 + c) * Np + vi] = g[G_SX] * Lx[c] + g[G_SY] * Ly[c];
+                }
+            }
+            __syncthreads();
+            if (vol) {
+                const real *ar = sFr + ve * 4 * Np;
+                const real *as = sFs + ve * 4 * Np;
+#pragma unroll
+                for (int j = 0; j < Np; ++j) {
+                    const real wr = sWr[vi * Np + j], ws = sWs[vi * Np + j];
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) R[c] += wr * ar[c * Np + j] + ws * as[c * Np + j];
+                }
             }
         }
         if (vol) {

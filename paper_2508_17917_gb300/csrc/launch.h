@@ -21,6 +21,7 @@ struct LaunchShape {
     int threads = 0;
     size_t smem = 0;
     int elems_per_tile = 0;
+    bool phases = false;     // FP64: the three-phase kernel (arrays between its phases, cooperative launch)
     bool handoff = false;    // two nodes per thread: the kernel that hands volume parts from stage to stage
     int minb = 0;            // ... and which of its builds (handoff_grid.h)
 };
@@ -47,7 +48,9 @@ inline cudaError_t launch_pdl(void (*kern)(Args...), const LaunchShape &ls, cuda
 
 // Launch configuration of the fused stage kernel for degree p and K elements
 // on the current device (persistent grid: SMs x resident CTAs, capped by tiles).
-cudaError_t stage_shape_fp64(int p, long long K, bool theta, LaunchShape &out, bool overint = false);
+// FP64: over-integrated, in three phases, or the kernel that needs neither
+// memory of its own nor a cooperative launch
+cudaError_t stage_shape_fp64(int p, long long K, bool theta, LaunchShape &out, bool overint, bool phases);
 cudaError_t stage_shape_mixed(int p, long long K, bool theta, LaunchShape &out);
 // what the three-phase FP64 stage kernel reads and keeps besides StageParams:
 // the symmetric operator tables of build_sym64_tables, every face once as

@@ -1,6 +1,6 @@
 // stage_fp64.cu -- the FP64 stage kernels (p = 1..6): the three-phase kernel
-// of dg_stage64.cuh with its operator tables, the over-integrated kernel of
-// dg_stage.cuh, and the FP64 broken gradient.
+// of dg_stage64.cuh with its operator tables, the kernels of dg_stage.cuh, and
+// the FP64 broken gradient.
 #include <cmath>
 #include <vector>
 
@@ -11,12 +11,12 @@
 namespace dg {
 namespace {
 
-// over-integrated volume term
-template <int P>
-cudaError_t shape_oi_p(long long K, LaunchShape &ls)
+// the kernel that needs no memory of its own
+template <int P, bool TH, bool OI>
+cudaError_t shape_alone_p(long long K, LaunchShape &ls)
 {
-    using L = Smem<P, double>;
-    auto kern = stage_kernel<P, double>;
+    using L = Smem<P, double, TH, OI>;
+    auto kern = stage_kernel<P, double, TH, OI>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          static_cast<int>(L::bytes));
     if (e != cudaSuccess) return e;
@@ -32,8 +32,9 @@ cudaError_t shape_oi_p(long long K, LaunchShape &ls)
     ls.threads = Shape<P>::NT;
     ls.smem = L::bytes;
     ls.elems_per_tile = Shape<P>::E;
-    ls.theta = false;
-    ls.overint = true;
+    ls.theta = TH;
+    ls.overint = OI;
+    ls.phases = false;
     return cudaSuccess;
 }
 
@@ -61,6 +62,7 @@ cudaError_t shape64_p(long long K, LaunchShape &ls)
     ls.elems_per_tile = S::EB;
     ls.theta = TH;
     ls.overint = false;
+    ls.phases = true;
     return cudaSuccess;
 }
 
@@ -68,8 +70,13 @@ template <int P>
 cudaError_t launch64_p(const LaunchShape &ls, const StageParams &sp, const Stage64 &x, const Phys<double> &ph,
                        cudaStream_t st)
 {
-    if (ls.overint) {
-        stage_kernel<P, double><<<ls.grid, ls.threads, ls.smem, st>>>(sp, ph);
+    if (!ls.phases) {
+        if (ls.overint)
+            stage_kernel<P, double, false, true><<<ls.grid, ls.threads, ls.smem, st>>>(sp, ph);
+        else if (ls.theta)
+            stage_kernel<P, double, true><<<ls.grid, ls.threads, ls.smem, st>>>(sp, ph);
+        else
+            stage_kernel<P, double, false><<<ls.grid, ls.threads, ls.smem, st>>>(sp, ph);
         return cudaGetLastError();
     }
     cudaLaunchConfig_t cfg = {};
@@ -195,9 +202,11 @@ bool sym64_tables_p(const RefOps &o, std::vector<double> &tab, std::vector<int> 
     default: return cudaErrorInvalidValue;        \
     }
 
-cudaError_t stage_shape_fp64(int p, long long K, bool theta, LaunchShape &out, bool overint)
+cudaError_t stage_shape_fp64(int p, long long K, bool theta, LaunchShape &out, bool overint, bool phases)
 {
-#define C_(P) (overint ? shape_oi_p<P>(K, out) : (theta ? shape64_p<P, true>(K, out) : shape64_p<P, false>(K, out)))
+#define C_(P) (overint  ? shape_alone_p<P, false, true>(K, out)                                                  \
+               : phases ? (theta ? shape64_p<P, true>(K, out) : shape64_p<P, false>(K, out))                     \
+                        : (theta ? shape_alone_p<P, true, false>(K, out) : shape_alone_p<P, false, false>(K, out)))
     DG_SWITCH_P(p, C_)
 #undef C_
 }
