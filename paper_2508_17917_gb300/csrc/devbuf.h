@@ -33,9 +33,11 @@ struct DevBuf {
     cudaError_t alloc(size_t count)
     {
         release();
-        n = count;
         if (count == 0) return cudaSuccess;
-        return cudaMalloc(reinterpret_cast<void **>(&ptr), count * sizeof(T));
+        const cudaError_t e = cudaMalloc(reinterpret_cast<void **>(&ptr), count * sizeof(T));
+        if (e == cudaSuccess) n = count;
+        else ptr = nullptr;
+        return e;
     }
     void release()
     {
