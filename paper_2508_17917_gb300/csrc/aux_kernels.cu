@@ -112,7 +112,7 @@ dt_confirm_kernel(AuxMesh m, Phys<double> ph, double sig_fac, const float *lamS,
                 const double b1 = fabs(v1 - ph.vw1) + c, b2 = fabs(v2 - ph.vw2) + c;
                 const double b = sqrt64(b1 * b1 + b2 * b2);
                 sB[it] = b;
-                if (!finite64(b)) isbad = 1;
+                if (!(finite_state(u, ir) && finite64(b))) isbad = 1;
             }
             __syncthreads();
             if (tid < nc) {
