@@ -105,20 +105,22 @@ dg_status dg_set_mesh(dg_ctx *ctx, int64_t Nv, const double *vx, const double *v
  * paper): 1 = one volume node and one face node per thread (256 threads),
  * 2 = two volume nodes per thread (128 threads; IIP only), each stage but a
  * step's first taking the divergence and the face records of its input state
- * from the launch before (single meshes below 25,000 elements at p = 3 and
- * 15,000 at p = 5: a kernel whose stages stand alone), 3 = one warp per tile of 2 elements with the Dr / Ds /
- * LIFT (and, for theta != 0, Wr / Ws) products on the tensor cores
- * (mma.sync TF32, three products of split operands, about 2^-21 relative;
- * p <= 6), 0 = time every available shape (five stage launches each on the
- * current state, at most 2^21 nodes of it, into buffers that hold nothing) at
- * the first time step after a mesh upload and keep the fastest (the default).  The FP64 path has one kernel and accepts 0 and 1.
+ * from the launch before (a kernel whose stages stand alone where those
+ * records find no memory, on a stream that cannot hold the first stage's
+ * grid at once, and below 25,000 elements at p = 3 and 15,000 at p = 5),
+ * 3 = one warp per tile of 2 elements with the Dr / Ds / LIFT (and, for
+ * theta != 0, Wr / Ws) products on the tensor cores (mma.sync TF32, three
+ * products of split operands, about 2^-21 relative; p <= 6), 0 = time every
+ * available shape (five stage launches each on the current state, at most
+ * 2^21 nodes of it, into buffers that hold nothing) at the first time step
+ * after a mesh upload and keep the fastest (the default).  The FP64 path has
+ * one shape and accepts 0 and 1.
  * The shapes round their FP32 arithmetic differently (all within the mixed
  * path's tolerance), and the tuner's choice depends on timings, so two runs
  * of the same input can differ in the last FP32 bits under variant 0: a
  * fixed variant (1, 2 or 3) is the bit-reproducible mode.
  * Errors: DG_EINVAL (variant outside 0..3), DG_EUNSUPPORTED (2 or 3 on the
- * FP64 path, 2 with theta != 0), DG_ECUDA (2: no memory for what it hands
- * from stage to stage; the tuner then leaves it out). */
+ * FP64 path, 2 with theta != 0), DG_ECUDA. */
 dg_status dg_set_stage_variant(dg_ctx *ctx, int variant);
 
 /* The tile shape in use: 1, 2 or 3 (the single-node kernel until tuned). */

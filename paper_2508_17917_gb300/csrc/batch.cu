@@ -49,6 +49,11 @@ struct Group {
     DevBuf<float> sym32;
     DevBuf<int> symn32;
     DevBuf<float4> fd32, rv32;
+    void drop_handoff()
+    {
+        fd32.release();
+        rv32.release();
+    }
     dg::Stage2Args stage2(int s) const
     {
         return dg::stage2_args(sym32.ptr, symn32.ptr, fd32.ptr, rv32.ptr, elem_case.ptr,
@@ -352,7 +357,7 @@ dg_status enqueue_step(dg_batch *b, double cfl, double *hist, int rows)
                     if (g.variant == 3)
                         B_CUDA(b, dg::stage_shape_tc(g.p, sp.ntiles, true, true, g.fshape));
                     else if (g.variant == 2)
-                        B_CUDA(b, dg::stage_shape_mixed2(g.p, g.K, true, true, g.fshape));
+                        B_CUDA(b, dg::stage_shape_mixed2(g.p, g.K, true, true, true, g.fshape));
                     else
                         B_CUDA(b, dg::stage_shape_mixed_fused(g.p, true, sp.ntiles, g.fshape));
                     g.fshape_variant = g.variant;
@@ -389,6 +394,19 @@ dg_status enqueue_step(dg_batch *b, double cfl, double *hist, int rows)
     return enqueue_forces(b, hist, rows);
 }
 
+// What the two-node shape of a group hands from stage to stage; no memory for
+// it leaves them empty, and the group runs with the other shapes.
+cudaError_t two_node_arrays(Group &g)
+{
+    if (g.rv32.ptr) return cudaSuccess;
+    cudaError_t e = g.fd32.alloc(2 * static_cast<size_t>(g.K) * 3 * g.ops.Nfp);
+    if (e == cudaSuccess) e = g.rv32.alloc(static_cast<size_t>(g.K) * g.ops.Np);
+    if (e != cudaErrorMemoryAllocation) return e;
+    cudaGetLastError();
+    g.drop_handoff();
+    return cudaSuccess;
+}
+
 // First run: per degree group, time every available stage-kernel shape on
 // the current states and keep the fastest for a step: a first stage untimed,
 // one timed, three inner ones.  Before a step the register and the other state
@@ -409,13 +427,19 @@ dg_status tune_groups(dg_batch *b)
     for (auto &e : ev.e) B_CUDA(b, cudaEventCreate(&e));
     for (auto &g : b->groups) {
         if (b->variant_req != 0) {
-            // the tensor-core shape covers p <= 6; other groups would take the two-node shape
+            // the tensor-core shape covers p <= 6; other groups would take the
+            // two-node shape, and without memory for that the one-node shape
             g.variant = (b->variant_req == 3 && !g.has_tc) ? 2 : b->variant_req;
+            if (g.variant == 2) B_CUDA(b, two_node_arrays(g));
+            if (g.variant == 2 && !g.rv32.ptr) g.variant = 1;
+            if (g.variant != 2) g.drop_handoff();
             continue;
         }
+        B_CUDA(b, two_node_arrays(g));
         float best = 0.f;
         for (int v = 1; v <= 3; ++v) {
             if (v == 3 && !g.has_tc) continue;
+            if (v == 2 && !g.rv32.ptr) continue;
             dg::StageParams sp{};
             const bool a = b->cur_is_a;
             sp.K0in = a ? g.K0a.ptr : g.K0b.ptr;
@@ -469,6 +493,7 @@ dg_status tune_groups(dg_batch *b)
                 g.variant = v;
             }
         }
+        if (g.variant != 2) g.drop_handoff();
     }
     b->tuned = true;
     return DG_OK;
@@ -625,8 +650,6 @@ dg_status dg_batch_create(const dg_params *common, int ncases, const dg_case *ca
         dg::build_sym32_tables(g.ops, tab, nodes, tab32, slots);
         chk(g.sym32.alloc(tab32.size()));
         chk(g.symn32.alloc(slots.size()));
-        chk(g.fd32.alloc(2 * static_cast<size_t>(g.K) * NF));
-        chk(g.rv32.alloc(static_cast<size_t>(g.K) * Np));
         chk(g.bar.alloc(8));
         chk(g.tiles3.alloc(tiles3.size()));
         std::vector<float> frag;
@@ -673,7 +696,7 @@ dg_status dg_batch_create(const dg_params *common, int ncases, const dg_case *ca
         chk(cudaMemset(g.P0a.ptr, 0, npp * sizeof(float)));
         chk(cudaMemset(g.P0b.ptr, 0, npp * sizeof(float)));
         chk(dg::stage_shape_mixed_batch(g.p, g.ntiles, g.shape));
-        chk(dg::stage_shape_mixed2(g.p, g.K, true, false, g.shape2));
+        chk(dg::stage_shape_mixed2(g.p, g.K, true, false, true, g.shape2));
         if (g.has_tc) chk(dg::stage_shape_tc(g.p, g.ntiles3, true, false, g.shape3));
         if (e != cudaSuccess) return bail(DG_ECUDA);
     }

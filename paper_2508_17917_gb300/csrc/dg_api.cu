@@ -44,7 +44,7 @@ struct dg_ctx {
     // device
     // FP64 and two-node kernels: symmetric operator tables, every face once, arrays between phases
     dg::DevBuf<double> sym64, flux64, dh64, th64;
-    bool no_coop = false;     // the stream refused the FP64 kernel's grid as a cooperative launch
+    bool no_coop = false;     // the stream refused a grid of theirs as a cooperative launch
     dg::DevBuf<float> sym32;
     dg::DevBuf<float4> fd32, rv32;
     dg::DevBuf<int> symn, symn32;
@@ -99,6 +99,11 @@ struct dg_ctx {
         dh64.release();
         th64.release();
         faces.release();
+    }
+    void drop_handoff()
+    {
+        fd32.release();
+        rv32.release();
     }
     ~dg_ctx()
     {
@@ -246,33 +251,45 @@ template <typename T>
 cudaError_t alloc_needed(dg_ctx *c, dg::DevBuf<T> &b, size_t n)
 {
     cudaError_t e = b.alloc(n);
-    if (e != cudaErrorMemoryAllocation || !c->flux64.ptr) return e;
+    if (e != cudaErrorMemoryAllocation || !(c->flux64.ptr || c->fd32.ptr)) return e;
     cudaGetLastError();
-    c->drop_phases();                  // cudaFree waits for the kernels that use them
-    e = shape_fp64(c);
+    if (c->flux64.ptr) {
+        c->drop_phases();                  // cudaFree waits for the kernels that use them
+        e = shape_fp64(c);
+    } else {
+        c->drop_handoff();
+        e = dg::stage_shape_mixed2(c->prm.p, c->K, false, false, false, c->shape2);
+        if (c->shape.variant == 2) c->shape = c->shape2;
+        c->fshape_variant = 0;
+    }
     return e == cudaSuccess ? b.alloc(n) : e;
 }
 
-// what the two-node kernel hands from stage to stage; a mesh that leaves no
-// memory for it runs with the other shapes
-cudaError_t two_node_arrays(dg_ctx *c)
+// The two-node shape of the mesh (IIP) and what its kernel hands from stage to
+// stage; without memory for that, or where the stream refused its grid, the
+// kernel whose stages stand alone.
+dg_status two_node_shape(dg_ctx *c)
 {
-    if (c->rv32.ptr) return cudaSuccess;
+    if (c->shape2.handoff && c->rv32.ptr) return DG_OK;
+    DG_CUDA(c, dg::stage_shape_mixed2(c->prm.p, c->K, false, false, !c->no_coop, c->shape2));
+    c->fshape_variant = 0;
+    if (!c->shape2.handoff) return DG_OK;
     cudaError_t e = c->fd32.alloc(2 * static_cast<size_t>(c->K) * 3 * c->ops.Nfp);
     if (e == cudaSuccess) e = c->rv32.alloc(static_cast<size_t>(c->K) * c->ops.Np);
-    if (e != cudaSuccess) {
-        cudaGetLastError();
-        c->fd32.release();
-        c->rv32.release();
+    if (e != cudaErrorMemoryAllocation) {
+        DG_CUDA(c, e);
+        return DG_OK;
     }
-    return e;
+    cudaGetLastError();
+    c->drop_handoff();
+    DG_CUDA(c, dg::stage_shape_mixed2(c->prm.p, c->K, false, false, false, c->shape2));
+    return DG_OK;
 }
 
 // s: stage of a step, -1 for a residual
 dg::Stage2Args stage2_args(const dg_ctx *c, int s)
 {
-    return dg::stage2_args(c->sym32.ptr, c->symn32.ptr, c->fd32.ptr, c->rv32.ptr, nullptr,
-                           static_cast<size_t>(c->K) * 3 * c->ops.Nfp, s);
+    return dg::stage2_args(c->sym32.ptr, c->symn32.ptr, c->fd32.ptr, c->rv32.ptr, nullptr, c->fd32.n / 2, s);
 }
 
 dg_status run_stage(dg_ctx *c, int s, double t, double dt, const double vw[2], int mode,
@@ -353,12 +370,23 @@ dg_status run_stage(dg_ctx *c, int s, double t, double dt, const double vw[2], i
             e = dg::launch_stage_tc(c->prm.p, false, false, c->shape, sp, make_phys<float>(c->prm, vw), c->stream);
         }
         else if (c->shape.variant == 2) {
-            sp.bar = c->bar.ptr;
-            sp.bar_err = c->bar_err.ptr;
-            sp.bar_limit = c->bar_limit;
-            c->copy_used = true;
-            e = dg::launch_stage_mixed2(c->prm.p, false, false, c->shape, sp, stage2_args(c, s),
-                                        make_phys<float>(c->prm, vw), c->stream);
+            if (c->shape.handoff) {
+                sp.bar = c->bar.ptr;
+                sp.bar_err = c->bar_err.ptr;
+                sp.bar_limit = c->bar_limit;
+                c->copy_used = true;
+            }
+            const dg::Phys<float> ph = make_phys<float>(c->prm, vw);
+            e = dg::launch_stage_mixed2(c->prm.p, false, false, c->shape, sp, stage2_args(c, s), ph, c->stream);
+            if (e == cudaErrorCooperativeLaunchTooLarge) {
+                // a first stage (or a residual): the others are ordinary launches
+                cudaGetLastError();
+                c->no_coop = true;
+                e = dg::stage_shape_mixed2(c->prm.p, c->K, false, false, false, c->shape2);
+                c->shape = c->shape2;
+                if (e == cudaSuccess)
+                    e = dg::launch_stage_mixed2(c->prm.p, false, false, c->shape, sp, stage2_args(c, s), ph, c->stream);
+            }
         }
         else
             e = dg::launch_stage_mixed(c->prm.p, c->shape, sp, make_phys<float>(c->prm, vw), c->stream);
@@ -585,9 +613,10 @@ dg_status dg_set_stage_variant(dg_ctx *c, int variant)
     if (variant == 3 && !dg::stage_tc_supported(c->prm.p))
         return fail(c, DG_EUNSUPPORTED, "the tensor-core kernel covers p <= 6");
     if (variant == 2 && c->K > 0) {
-        const cudaError_t e = two_node_arrays(c);
-        if (e != cudaSuccess) return cuda_fail(c, e, "arrays of the two-node kernel");
+        dg_status st = two_node_shape(c);
+        if (st != DG_OK) return st;
     }
+    if (variant == 1 || variant == 3) c->drop_handoff();
     c->variant_req = variant;
     c->tuned = (variant != 0);
     if (c->K > 0 && c->prm.precision == DG_PRECISION_MIXED)
@@ -614,6 +643,7 @@ dg_status dg_set_mesh(dg_ctx *c, int64_t Nv, const double *vx, const double *vy,
     std::vector<double> &wxy = ma.wxy;
     // --- device buffers
     c->drop_phases();
+    c->drop_handoff();
     c->K = K;
     const size_t nd = static_cast<size_t>(K) * 4 * Np;
     DG_CUDA(c, c->K0a.alloc(nd));
@@ -641,12 +671,6 @@ dg_status dg_set_mesh(dg_ctx *c, int64_t Nv, const double *vx, const double *vy,
         DG_CUDA(c, cudaMemsetAsync(c->S0b.ptr, 0, np * sizeof(float4), c->stream));
         DG_CUDA(c, cudaMemsetAsync(c->P0a.ptr, 0, npp * sizeof(float), c->stream));
         DG_CUDA(c, cudaMemsetAsync(c->P0b.ptr, 0, npp * sizeof(float), c->stream));
-        c->fd32.release();
-        c->rv32.release();
-        if (c->prm.theta == 0.0) {
-            const cudaError_t e = two_node_arrays(c);
-            if (e != cudaSuccess && c->variant_req == 2) return cuda_fail(c, e, "arrays of the two-node kernel");
-        }
     }
     c->nwall = static_cast<int>(walls.size());
     if (c->nwall > 0) {
@@ -676,10 +700,11 @@ dg_status dg_set_mesh(dg_ctx *c, int64_t Nv, const double *vx, const double *vy,
     c->fshape_variant = 0;           // the cooperative grid is sized per mesh
     c->has_tc = false;
     if (c->prm.precision == DG_PRECISION_MIXED) {
-        if (!th) {
-            e = dg::stage_shape_mixed2(c->prm.p, K, false, false, c->shape2);
-            if (e != cudaSuccess) return cuda_fail(c, e, "stage kernel configuration");
-            if (c->variant_req == 2) c->shape = c->shape2;
+        c->shape2 = dg::LaunchShape();
+        if (!th && c->variant_req == 2) {
+            dg_status st = two_node_shape(c);
+            if (st != DG_OK) return st;
+            c->shape = c->shape2;
         }
         if (dg::stage_tc_supported(c->prm.p)) {
             e = dg::stage_shape_tc(c->prm.p, K, false, false, c->shape3, th);
@@ -807,6 +832,11 @@ static dg_status tune_stage(dg_ctx *c, const double vw[2])
         c->tuned = true;
         return DG_OK;
     }
+    const bool iip = c->prm.theta == 0.0;
+    if (iip) {
+        dg_status st = two_node_shape(c);
+        if (st != DG_OK) return st;
+    }
     // timed on 2^21 nodes at most, four times the L2 cache
     struct Part {
         dg_ctx *c;
@@ -814,7 +844,7 @@ static dg_status tune_stage(dg_ctx *c, const double vw[2])
         ~Part() { c->K = K; }
     } part{c, c->K};
     c->K = std::min<int64_t>(c->K, (1 << 21) / c->ops.Np);
-    const dg::LaunchShape *const cand[3] = {&c->shape1, c->rv32.ptr ? &c->shape2 : nullptr, c->has_tc ? &c->shape3 : nullptr};
+    const dg::LaunchShape *const cand[3] = {&c->shape1, iip ? &c->shape2 : nullptr, c->has_tc ? &c->shape3 : nullptr};
     for (int v = 0; v < 3; ++v) {
         if (!cand[v]) continue;
         c->shape = *cand[v];
@@ -826,6 +856,10 @@ static dg_status tune_stage(dg_ctx *c, const double vw[2])
         DG_CUDA(c, cudaEventRecord(c->tune_ev[3 * v + 2], c->stream));
     }
     DG_CUDA(c, cudaStreamSynchronize(c->stream));
+    c->K = part.K;
+    // a grid that was refused meanwhile was replaced by one for the part
+    if (iip && !c->shape2.handoff)
+        DG_CUDA(c, dg::stage_shape_mixed2(c->prm.p, c->K, false, false, false, c->shape2));
     float best = 0.f;
     dg::LaunchShape pick = c->shape1;
     for (int v = 0; v < 3; ++v) {
@@ -840,6 +874,7 @@ static dg_status tune_stage(dg_ctx *c, const double vw[2])
         }
     }
     c->shape = pick;
+    if (pick.variant != 2) c->drop_handoff();
     c->tuned = true;
     return DG_OK;
 }
@@ -878,7 +913,7 @@ static dg_status run_fused_step(dg_ctx *c, double dt, const double vw[2])
 {
     if (c->fshape_variant != c->shape.variant) {
         cudaError_t e = (c->shape.variant == 3)   ? dg::stage_shape_tc(c->prm.p, c->K, false, true, c->fshape)
-                        : (c->shape.variant == 2) ? dg::stage_shape_mixed2(c->prm.p, c->K, false, true, c->fshape)
+                        : (c->shape.variant == 2) ? dg::stage_shape_mixed2(c->prm.p, c->K, false, true, c->shape.handoff, c->fshape)
                                                   : dg::stage_shape_mixed_fused(c->prm.p, false, c->K, c->fshape);
         if (e != cudaSuccess) return cuda_fail(c, e, "fused stage kernel configuration");
         c->fshape_variant = c->shape.variant;

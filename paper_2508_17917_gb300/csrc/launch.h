@@ -81,11 +81,14 @@ cudaError_t launch_stage_mixed_batch(int p, const LaunchShape &ls, const StagePa
 // Lambda_K of every degree group of a batch in one launch (one block per tile)
 cudaError_t launch_dt_lambda_mixed_multi(const DtGroups &dgs, const BatchCase *cases, const Phys<float> &ph,
                                          float sig_fac, cudaStream_t st);
-// the mixed IIP kernel with two nodes per thread for K elements: one stage, or
-// the five of a step (fused).  Its tables are those of build_sym32_tables; it
-// hands a record per face node (pressure, viscous normal flux) [K][3 Nfp] and
-// the divergence [K][Np] from stage to stage.  A launch with `first` (and a
-// fused one) is cooperative.
+// The mixed IIP kernel with two nodes per thread for K elements: one stage, or
+// the five of a step (fused).  The hand-off kernel (LaunchShape::handoff) has
+// the tables of build_sym32_tables and hands a record per face node (pressure,
+// viscous normal flux) [K][3 Nfp] and the divergence [K][Np] from stage to
+// stage; a launch with `first` (and a fused one) is cooperative.  A single
+// mesh without memory for those, or on a stream that cannot hold its grid,
+// takes the kernel whose stages stand alone (handoff = false), and so do
+// small meshes at some degrees.
 struct Stage2Args {
     const float *ops;
     const int *nodes;
@@ -103,7 +106,7 @@ inline Stage2Args stage2_args(const float *ops, const int *nodes, float4 *fd, fl
     const bool second = s <= 0 || (s & 1);
     return {ops, nodes, second ? fd + n : fd, second ? fd : fd + n, rv, elem_case, s <= 0 ? 1 : 0, s >= 0 && s < 4 ? 1 : 0};
 }
-cudaError_t stage_shape_mixed2(int p, long long K, bool batch, bool fused, LaunchShape &out);
+cudaError_t stage_shape_mixed2(int p, long long K, bool batch, bool fused, bool handoff, LaunchShape &out);
 cudaError_t launch_stage_mixed2(int p, bool batch, bool fused, const LaunchShape &ls, const StageParams &sp,
                                 const Stage2Args &a, const Phys<float> &ph, cudaStream_t st);
 // FP32 rows (each twice) from the FP64 tables, and per thread its two nodes

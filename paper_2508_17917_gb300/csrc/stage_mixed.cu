@@ -154,7 +154,7 @@ cudaError_t launch2_p(const LaunchShape &ls, const StageParams &sp, const Stage2
     return handoff_launch_p<P, BATCH, FUSE, 4>(ls, sp, x, ph, st);
 }
 
-// ... and the kernel whose stages stand alone (single mesh, p = 3 and 5)
+// ... and the kernel whose stages stand alone (single mesh)
 template <int P, bool FUSE>
 cudaError_t alone_shape_p(long long K, LaunchShape &ls)
 {
@@ -317,17 +317,17 @@ cudaError_t launch_dt_screen(const AuxMesh &m, const Phys<float> &ph, double gm1
 #undef C_
 }
 
-cudaError_t stage_shape_mixed2(int p, long long K, bool batch, bool fused, LaunchShape &out)
+cudaError_t stage_shape_mixed2(int p, long long K, bool batch, bool fused, bool handoff, LaunchShape &out)
 {
     // Measured, us for two steps of a single mesh, fastest of the shapes of each
     // side: p = 3, 76^2 quads 138 (stages alone) and 147 (hand-off), 110^2 231
     // and 245, 119^2 295 and 247; p = 5, 50^2 140 and 172, 70^2 235 and 274, 86^2
     // 329 and 341, 90^2 393 and 346.  Other degrees: hand-off ahead or neither
     // the fastest shape.
-    if (!batch && p == 3 && K < 25000) return fused ? alone_shape_p<3, true>(K, out) : alone_shape_p<3, false>(K, out);
-    if (!batch && p == 5 && K < 15000) return fused ? alone_shape_p<5, true>(K, out) : alone_shape_p<5, false>(K, out);
-#define C_(P) (batch ? (fused ? handoff_shape_p<P, true, true>(K, out) : handoff_shape_p<P, true, false>(K, out)) \
-                     : (fused ? handoff_shape_p<P, false, true>(K, out) : handoff_shape_p<P, false, false>(K, out)))
+    const bool alone = !handoff || (p == 3 && K < 25000) || (p == 5 && K < 15000);
+#define C_(P) (batch   ? (fused ? handoff_shape_p<P, true, true>(K, out) : handoff_shape_p<P, true, false>(K, out)) \
+               : alone ? (fused ? alone_shape_p<P, true>(K, out) : alone_shape_p<P, false>(K, out))                 \
+                       : (fused ? handoff_shape_p<P, false, true>(K, out) : handoff_shape_p<P, false, false>(K, out)))
     DG_SWITCH_P(p, C_)
 #undef C_
 }
@@ -336,9 +336,9 @@ cudaError_t launch_stage_mixed2(int p, bool batch, bool fused, const LaunchShape
                                 const Stage2Args &a, const Phys<float> &ph, cudaStream_t st)
 {
     if (!ls.handoff) {
-        if (p == 3) return alone_launch_p<3>(fused, ls, sp, ph, st);
-        if (p == 5) return alone_launch_p<5>(fused, ls, sp, ph, st);
-        return cudaErrorInvalidValue;
+#define C_(P) alone_launch_p<P>(fused, ls, sp, ph, st)
+        DG_SWITCH_P(p, C_)
+#undef C_
     }
     const Stage2 x{reinterpret_cast<const float4 *>(a.ops), a.nodes, a.fin, a.fout, a.rv, a.elem_case, a.first, a.next};
 #define C_(P) (batch ? (fused ? launch2_p<P, true, true>(ls, sp, x, ph, st) : launch2_p<P, true, false>(ls, sp, x, ph, st)) \

@@ -10,9 +10,10 @@ import numpy as np
 import pytest
 
 import dg_inputs
+import oracle
 from dg_inputs.states import to_kcn
 
-from _parity import RHS_TOL_ALL_FP64, STATE_TOL, all_err
+from _parity import INC_TOL, RHS_TOL_ALL_FP64, STATE_TOL, all_err, check_rhs, inc_err
 
 pytestmark = pytest.mark.gpu
 MB = 1 << 20
@@ -105,33 +106,130 @@ def test_over_integration_keeps_no_phase_arrays(dg):
     assert free0 > phases
 
 
-@pytest.mark.parametrize("p,theta", [(4, 0.0), (2, 1.0)])
-def test_fp64_without_memory_between_the_phases(dg, p, theta):
-    """All but what the state needs, and half of what the phases need besides,
-    is taken."""
+def take_all_but(n):
     import torch
+    torch.cuda.empty_cache()
+    return torch.empty(free_bytes() - n, dtype=torch.uint8, device="cuda")
+
+
+@pytest.mark.parametrize("p,theta", [(4, 0.0), (2, 1.0)])
+def test_fp64_without_memory_between_the_phases(dg, part_of_the_device, p, theta):
+    """All but what the state needs, and half of what the phases need besides,
+    is taken.  Same kernel, and so the same bits, as on a part of the device."""
     mesh = dg_inputs.periodic_square(400)               # 320,000 elements
     kw = dict(mu=1e-3, theta=theta, C1=0.05)
-    torch.cuda.empty_cache()
+    alone = dg.Solver(mesh, p, "fp64", stream=part_of_the_device, **kw)
+    U = vortex(alone)
+    alone.set_state(U)
+    want = alone.rhs()
+    dt = alone.dt(0.3)
+    alone.steps(0.0, dt, 1)
+    after = alone.get_state()
+    del alone
     free0 = free_bytes()
-    ref = dg.Solver(mesh, p, "fp64", stream=stream(), **kw)
-    U = vortex(ref)
-    ref.set_state(U)
-    want = ref.rhs()
-    dt = ref.dt(0.3)
+    s = dg.Solver(mesh, p, "fp64", stream=stream(), **kw)
+    s.set_state(U)
+    s.rhs()
     used = free0 - free_bytes()
+    del s
     Np, nfn = (p + 1) * (p + 2) // 2, 3 * (p + 1)
     phases = mesh.K * (64 * Np + 32 * nfn + (64 * nfn if theta else 0))
     assert used > phases
-    del ref
-    hold = torch.empty(free_bytes() - (used - phases // 2), dtype=torch.uint8, device="cuda")
-    try:
-        s = dg.Solver(mesh, p, "fp64", stream=stream(), **kw)
-        s.set_state(U)
-        assert all_err(s.rhs(), want) <= RHS_TOL_ALL_FP64
-        assert s.dt(0.3) == dt
-        s.steps(0.0, dt, 1)
-        assert np.all(np.isfinite(s.get_state()))
-    finally:
+    hold = take_all_but(used - phases // 2)
+    s = dg.Solver(mesh, p, "fp64", stream=stream(), **kw)
+    s.set_state(U)
+    assert np.array_equal(s.rhs(), want)
+    assert s.dt(0.3) == dt
+    s.steps(0.0, dt, 1)
+    assert np.array_equal(s.get_state(), after)
+    del hold
+
+
+@pytest.mark.parametrize("p,variant", [(1, 2), (2, 2), (4, 2), (6, 2), (4, 0), (6, 0)])
+def test_mixed_on_a_part_of_the_device(dg, part_of_the_device, p, variant):
+    mesh = dg_inputs.periodic_square(64)
+    P = oracle.Problem(mesh, p, mu=1e-3)
+    s = dg.Solver(mesh, p, "mixed", stream=part_of_the_device, mu=1e-3)
+    s.set_variant(variant)
+    U = dg_inputs.perturb(to_kcn(dg_inputs.isentropic_vortex(P.x, P.y)), seed=3, amp=1e-3)
+    s.set_state(U)
+    check_rhs(P, U, s.rhs(), "mixed")
+    dt = P.dt(U, 0.3)[0]
+    s.steps(0.0, dt, 2)
+    got = s.get_state()
+    assert np.all(inc_err(P, got, P.run(U, 0.0, dt, 2), U) <= INC_TOL["mixed"])
+    s.set_state(U)
+    s.steps(0.0, dt, 2)
+    assert np.array_equal(s.get_state(), got)
+
+
+@pytest.mark.parametrize("p", [2, 4])
+def test_two_nodes_without_memory_between_the_stages(dg, part_of_the_device, p):
+    """As for the FP64 phases; five launches a step and one."""
+    mesh = dg_inputs.periodic_square(400)
+    alone = dg.Solver(mesh, p, "mixed", stream=part_of_the_device, mu=1e-3)
+    U = vortex(alone)
+    alone.set_variant(2)
+    alone.set_state(U)
+    want = alone.rhs()
+    alone.steps(0.0, 1e-5, 2)
+    after = alone.get_state()
+    del alone
+    free0 = free_bytes()
+    s = dg.Solver(mesh, p, "mixed", stream=stream(), mu=1e-3)
+    s.set_variant(2)
+    s.set_state(U)
+    s.rhs()
+    used = free0 - free_bytes()
+    del s
+    stages = mesh.K * 16 * ((p + 1) * (p + 2) // 2 + 6 * (p + 1))
+    assert used > stages
+    hold = take_all_but(used - stages // 2)
+    s = dg.Solver(mesh, p, "mixed", stream=stream(), mu=1e-3)
+    s.set_variant(2)
+    s.set_state(U)
+    assert np.array_equal(s.rhs(), want)
+    s.steps(0.0, 1e-5, 2)
+    assert np.array_equal(s.get_state(), after)
+    s.set_fused(True)
+    s.set_state(U)
+    s.steps(0.0, 1e-5, 2)
+    assert np.abs(s.get_state() - after).max() <= 1e-9 * np.abs(after).max()
+    del hold
+
+
+def test_the_two_node_arrays_go_when_another_shape_is_taken(dg):
+    mesh = dg_inputs.periodic_square(200)               # 80,000 elements: 58 MB between the stages at p = 4
+    s = dg.Solver(mesh, 4, "mixed", stream=stream(), mu=1e-3)
+    s.set_state(vortex(s))
+    for v in (1, 2, 3):                                 # every kernel is loaded
+        s.set_variant(v)
+        s.steps(0.0, 1e-6, 1)
+    without = free_bytes()
+    s.set_variant(2)
+    assert without - free_bytes() >= 50 * MB
+    s.set_variant(1)
+    assert abs(without - free_bytes()) <= 4 * MB
+    s.set_variant(0)
+    s.steps(0.0, 1e-6, 1)
+    if s.variant != 2:
+        assert abs(without - free_bytes()) <= 4 * MB
+
+
+def test_batch_without_memory_between_the_stages(dg):
+    """A group takes the one-node shape instead of the two-node shape."""
+    kw = dict(rho_inf=1.0, u_inf=1.0, v_inf=0.0, p_inf=17.857142857142858)
+    case = dict(mesh=dg_inputs.ogrid_cylinder(400, 100, 0.5, 20.0, seed=1), p=4, mu=0.01, y0=0.0, ydot0=0.0, M_r=1.0,
+                C_r=0.1, K_r=2.0, mass=8.0)             # 80,000 elements: 58 MB between the stages
+    got = []
+    for variant in (1, 2):
+        b = dg.BatchSolver([case], **kw)
+        b.set_variant(variant)
+        x, y = b.node_coords(0)
+        b.set_state(0, to_kcn(dg_inputs.free_stream(x.shape, rho=1.0, u=1.0, v=0.0, p=kw["p_inf"])))
+        hold = take_all_but(24 * MB) if variant == 2 else None
+        b.run(0.3, 2, use_graph=False)
+        assert b.variant(0) == 1
+        got.append(b.get_state(0))
         del hold
-        torch.cuda.empty_cache()
+    assert np.array_equal(got[0], got[1])
