@@ -139,17 +139,39 @@ bool sym64_tables_p(const RefOps &o, std::vector<double> &tab, std::vector<int> 
             worst = std::fmax(worst, std::fabs(o.LIFT[i * NF + m] - o.LIFT[mirror[i] * NF + NF - 1 - m]));
     }
     if (!(worst < 1e-9)) return false;
+    // The rows of a pair serve both of its nodes, so they are the mean of the
+    // two; and the derivative of a constant is zero.  The tables then carry
+    // less of the operators' own rounding than the operators do (RMS error of
+    // a gradient against exact operators, vortex, p = 4, energy: 0.55e-14 with
+    // them, 1.0e-14 with the plain rows, 1.6e-14 with the rows of one node).
+    std::vector<double> Dr(o.Dr), Ds(o.Ds), LIFT(o.LIFT), Wr(o.Wr), Ws(o.Ws);
+    for (int i = 0; i < Np; ++i) {
+        double sum = 0.0;
+        for (int j = 0; j < Np; ++j) {
+            Dr[i * Np + j] = 0.5 * (o.Dr[i * Np + j] + o.Ds[mirror[i] * Np + mirror[j]]);
+            Wr[i * Np + j] = 0.5 * (o.Wr[i * Np + j] + o.Ws[mirror[i] * Np + mirror[j]]);
+            sum += Dr[i * Np + j];
+        }
+        Dr[i * Np + i] -= sum;
+        for (int m = 0; m < NF; ++m)
+            LIFT[i * NF + m] = 0.5 * (o.LIFT[i * NF + m] + o.LIFT[mirror[i] * NF + NF - 1 - m]);
+    }
+    for (int i = 0; i < Np; ++i)
+        for (int j = 0; j < Np; ++j) {
+            Ds[mirror[i] * Np + mirror[j]] = Dr[i * Np + j];
+            Ws[mirror[i] * Np + mirror[j]] = Wr[i * Np + j];
+        }
     // Q = W LIFT for the theta terms
     std::vector<double> Pm(Np * Np), Mm(Np * Np), Qp(Np * NF, 0.0), Qm(Np * NF, 0.0);
     for (int i = 0; i < Np * Np; ++i) {
-        Pm[i] = 0.5 * (o.Dr[i] + o.Ds[i]);
-        Mm[i] = 0.5 * (o.Dr[i] - o.Ds[i]);
+        Pm[i] = 0.5 * (Dr[i] + Ds[i]);
+        Mm[i] = 0.5 * (Dr[i] - Ds[i]);
     }
     for (int i = 0; i < Np; ++i)
         for (int m = 0; m < NF; ++m)
             for (int j = 0; j < Np; ++j) {
-                Qp[i * NF + m] += 0.5 * (o.Wr[i * Np + j] + o.Ws[i * Np + j]) * o.LIFT[j * NF + m];
-                Qm[i * NF + m] += 0.5 * (o.Wr[i * Np + j] - o.Ws[i * Np + j]) * o.LIFT[j * NF + m];
+                Qp[i * NF + m] += 0.5 * (Wr[i * Np + j] + Ws[i * Np + j]) * LIFT[j * NF + m];
+                Qm[i * NF + m] += 0.5 * (Wr[i * Np + j] - Ws[i * Np + j]) * LIFT[j * NF + m];
             }
     // even (sign +1) and odd (-1) rows of a matrix over nodes, and over face slots
     auto node_row = [&](const std::vector<double> &A, int i, int l, double sign) {
@@ -178,8 +200,8 @@ bool sym64_tables_p(const RefOps &o, std::vector<double> &tab, std::vector<int> 
             put(S::oB + l * TPE, pr ? node_row(Pm, a, l, -1) : (b < 0 ? 0.0 : node_row(Mm, b, l, -1)),
                 node_row(Mm, a, l, -1));
         for (int m = 0; m < NEF; ++m) {
-            put(S::oL + m * TPE, -face_row(o.LIFT, a, m, 1),
-                pr ? -face_row(o.LIFT, a, m, -1) : (b < 0 ? 0.0 : -face_row(o.LIFT, b, m, 1)));
+            put(S::oL + m * TPE, -face_row(LIFT, a, m, 1),
+                pr ? -face_row(LIFT, a, m, -1) : (b < 0 ? 0.0 : -face_row(LIFT, b, m, 1)));
             put(S::oQA + m * TPE, -face_row(Qp, a, m, 1),
                 pr ? -face_row(Qm, a, m, 1) : (b < 0 ? 0.0 : -face_row(Qp, b, m, 1)));
             put(S::oQB + m * TPE, pr ? -face_row(Qp, a, m, -1) : (b < 0 ? 0.0 : -face_row(Qm, b, m, -1)),
