@@ -167,19 +167,24 @@ dt_confirm_kernel(AuxMesh m, Phys<double> ph, double sig_fac, const float *lamS,
 // Force and moment of one wall face: traction p n - tau n at its face nodes
 // (interior trace, n the element's outward normal), integrated with the LGL
 // weights scaled by sJ; moment about (xc, yc).  xy: the face nodes'
-// coordinates (x, y interleaved).  One warp per face: lane 4 i + c forms the
-// broken gradient of field c at face node i, the four lanes of a node
-// exchange fields by shuffles, and lane 0 ends up with the sums over the
-// nodes in node order.  Few faces and long FP64 chains: latency bounds this,
+// coordinates (x, y interleaved).  4 Nfp lanes per face, from lane `base` of
+// the warp: lane base + 4 i + c forms the broken gradient of field c at face
+// node i, the four lanes of a node exchange fields by shuffles, and the sums
+// over the nodes, in node order, end up in all of them.  Few faces and long FP64 chains: latency bounds this,
 // so the Np-term sums of a face run side by side instead of one after the
 // other in one thread (120 faces at p = 4: 39 us and a separate 4 us sum
-// before, 13 us in all now).
+// before, 13 us in all now).  Thousands of faces fill the FP64 pipe, to which
+// an idle lane costs as much as a busy one: a warp takes as many faces as fit
+// (4,000 faces, us a call: p = 1, 54 and 44; p = 2, 56 and 53 -- one face per
+// warp, now).
+__host__ __device__ __forceinline__ int faces_per_warp(int Nfp) { return Nfp < 8 ? 8 / Nfp : 1; }
+
 __device__ void wall_face_force(const AuxMesh &m, Phys<double> ph, long long k, int f, const double *xy,
-                                const double *wface, double xc, double yc, double out[3])
+                                const double *wface, double xc, double yc, int base, double out[3])
 {
     const int p = m.p, Np = (p + 1) * (p + 2) / 2, Nfp = p + 1;
     if (m.elem_case) ph.mu = m.cases[m.elem_case[k]].mu;
-    const int lane = threadIdx.x & 31, i = lane >> 2, c = lane & 3;
+    const int lane = threadIdx.x & 31, i = (lane - base) >> 2, c = lane & 3;
     const int ii = i < Nfp ? i : 0;              // idle lanes repeat node 0 and are not summed
     const double *g = m.geo + k * 16;
     const double rx = g[G_RX], ry = g[G_RY], sx = g[G_SX], sy = g[G_SY];
@@ -211,9 +216,9 @@ __device__ void wall_face_force(const AuxMesh &m, Phys<double> ph, long long k, 
     const double tm = (xy[2 * ii] - xc) * ty - (xy[2 * ii + 1] - yc) * tx;
     out[0] = out[1] = out[2] = 0.0;
     for (int l = 0; l < Nfp; ++l) {
-        out[0] += __shfl_sync(0xffffffffu, tx, 4 * l);
-        out[1] += __shfl_sync(0xffffffffu, ty, 4 * l);
-        out[2] += __shfl_sync(0xffffffffu, tm, 4 * l);
+        out[0] += __shfl_sync(0xffffffffu, tx, base + 4 * l);
+        out[1] += __shfl_sync(0xffffffffu, ty, base + 4 * l);
+        out[2] += __shfl_sync(0xffffffffu, tm, base + 4 * l);
     }
 }
 
@@ -225,6 +230,7 @@ __device__ void block_sum3(const double *partial, int n, double (*s)[256])
 {
     for (int t = threadIdx.x; t < 256; t += blockDim.x) {
         double a[3] = {0, 0, 0};
+#pragma unroll 4      // the reads of four faces in flight, the sums in order
         for (int i = t; i < n; i += 256)
             for (int c = 0; c < 3; ++c) a[c] += __ldcg(partial + static_cast<long long>(i) * 3 + c);
         for (int c = 0; c < 3; ++c) s[c][t] = a[c];
@@ -237,7 +243,7 @@ __device__ void block_sum3(const double *partial, int n, double (*s)[256])
     }
 }
 
-// Wall faces of one mesh, a warp per face: partial[w] = (Fx, Fy, Mz) of face
+// Wall faces of one mesh, faces_per_warp to a warp: partial[w] = (Fx, Fy, Mz) of face
 // w; the last block to finish (ticket, zero between launches) sums them into
 // out, so that no second launch waits for the first.
 __global__ void wall_force_kernel(AuxMesh m, Phys<double> ph, const int2 *faces, const double *face_xy,
@@ -246,12 +252,15 @@ __global__ void wall_force_kernel(AuxMesh m, Phys<double> ph, const int2 *faces,
 {
     __shared__ double s[3][256];
     __shared__ bool last;
-    const int w = blockIdx.x * kWallWarps + (threadIdx.x >> 5);
-    const int Nfp = m.p + 1;
-    if (w < nwall) {
+    const int Nfp = m.p + 1, per = faces_per_warp(Nfp), lane = threadIdx.x & 31;
+    const int sub = min(lane / (4 * Nfp), per - 1), base = 4 * Nfp * sub;      // lanes past the last face go with it
+    const int w0 = (blockIdx.x * kWallWarps + (threadIdx.x >> 5)) * per, w = w0 + sub;
+    if (w0 < nwall) {
+        const int v = min(w, nwall - 1);
         double o[3];
-        wall_face_force(m, ph, faces[w].x, faces[w].y, face_xy + static_cast<long long>(w) * Nfp * 2, wface, xc, yc, o);
-        if ((threadIdx.x & 31) == 0) {
+        wall_face_force(m, ph, faces[v].x, faces[v].y, face_xy + static_cast<long long>(v) * Nfp * 2, wface, xc, yc,
+                        base, o);
+        if (lane == base && w < nwall) {
             for (int c = 0; c < 3; ++c) partial[static_cast<long long>(w) * 3 + c] = o[c];
             __threadfence();
         }
@@ -281,7 +290,7 @@ __global__ void batch_wall_force_kernel(WallGroups wg, Phys<double> ph, double *
     const int i = w - G.base, Nfp = G.m.p + 1;
     double o[3];
     wall_face_force(G.m, ph, G.faces[i].x, G.faces[i].y, G.face_xy + static_cast<long long>(i) * Nfp * 2, G.wface, 0.0,
-                    0.0, o);
+                    0.0, 0, o);
     if ((threadIdx.x & 31) == 0)
         for (int c = 0; c < 3; ++c) partial[static_cast<long long>(w) * 3 + c] = o[c];
 }
@@ -504,7 +513,8 @@ cudaError_t launch_wall_forces(const AuxMesh &m, const Phys<double> &ph, const i
                                const double *wface, int nwall, double xc, double yc, double *partial,
                                unsigned *ticket, double *out, cudaStream_t st)
 {
-    const int blocks = (nwall + kWallWarps - 1) / kWallWarps;
+    const int at_once = kWallWarps * faces_per_warp(m.p + 1);
+    const int blocks = (nwall + at_once - 1) / at_once;
     wall_force_kernel<<<blocks, 32 * kWallWarps, 0, st>>>(m, ph, faces, face_xy, wface, nwall, xc, yc, partial, ticket,
                                                           out);
     return cudaGetLastError();
