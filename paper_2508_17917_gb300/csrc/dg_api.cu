@@ -80,6 +80,7 @@ struct dg_ctx {
     int source_kind = DG_SOURCE_NONE;
     dg::DevBuf<float> gimg;           // split [Dr; Ds] image of the tcgen05 gradient
     bool gimg_ready = false;          // gimg holds the image
+    int ggrid = 0;                    // blocks of the FP64 gradient on this mesh (0: not asked for yet)
     dg::DevBuf<double> gtmp;          // host-output staging of dg_broken_gradient
     dg::VortexSource vortex{};         // DG_SOURCE_VORTEX parameters
     dg::DevBuf<double> src_xy;        // node coordinates for the vortex source
@@ -645,6 +646,7 @@ dg_status dg_set_mesh(dg_ctx *c, int64_t Nv, const double *vx, const double *vy,
     c->drop_phases();
     c->drop_handoff();
     c->K = K;
+    c->ggrid = 0;
     const size_t nd = static_cast<size_t>(K) * 4 * Np;
     DG_CUDA(c, c->K0a.alloc(nd));
     DG_CUDA(c, c->K0b.alloc(nd));
@@ -1068,8 +1070,10 @@ dg_status dg_broken_gradient(dg_ctx *c, double *gx, double *gy, int on_device, i
         oy = c->gtmp.ptr + n;
     }
     if (impl == 0) {
-        DG_CUDA(c, dg::launch_grad64(c->prm.p, c->cur(), c->geo64.ptr, c->sym64.ptr, c->symn.ptr, c->K, ox, oy,
-                                     c->stream));
+        if (!c->ggrid) DG_CUDA(c, dg::grad64_grid(c->prm.p, c->K, c->ggrid));
+        const dg::Grad64Args a{c->ggrid, c->cur(), c->geo64.ptr, c->sym64.ptr, c->symn.ptr, c->Dr64.ptr, c->Ds64.ptr,
+                               c->K, ox, oy};
+        DG_CUDA(c, dg::launch_grad64(c->prm.p, a, c->stream));
     } else {
         dg::GradTc05Args a{};
         a.U = c->cur();

@@ -593,4 +593,29 @@ grad64_kernel(const double *U, const double *geo, const double2 *ops, const int 
     }
 }
 
+// The same with a thread per (element, node) and the plain rows.
+template <int P>
+__global__ void __launch_bounds__(128)
+grad64_rows_kernel(const double *U, const double *Dr, const double *Ds, const double *geo, long long K, double *gx, double *gy)
+{
+    constexpr int Np = Sym64<P>::Np;
+    const long long n = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x;
+    if (n >= K * Np) return;
+    const long long k = n / Np;
+    const int i = static_cast<int>(n - k * Np);
+    const double *g = geo + k * 16;
+    const double rx = g[G_RX], ry = g[G_RY], sx = g[G_SX], sy = g[G_SY];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        const double *u = U + (k * 4 + c) * Np;
+        double ur = 0.0, us = 0.0;
+        for (int j = 0; j < Np; ++j) {
+            ur += Dr[i * Np + j] * u[j];
+            us += Ds[i * Np + j] * u[j];
+        }
+        gx[(k * 4 + c) * Np + i] = rx * ur + sx * us;
+        gy[(k * 4 + c) * Np + i] = ry * ur + sy * us;
+    }
+}
+
 }  // namespace dg

@@ -69,9 +69,19 @@ cudaError_t launch_stage_fp64(int p, const LaunchShape &ls, const StageParams &s
 // false if the operators are not symmetric under r <-> s
 struct RefOps;
 bool build_sym64_tables(const RefOps &o, std::vector<double> &tab, std::vector<int> &nodes);
-// broken gradient [K][4][Np] x 2 in FP64 from those tables
-cudaError_t launch_grad64(int p, const double *U, const double *geo, const double *ops, const int *nodes, long long K,
-                          double *gx, double *gy, cudaStream_t st);
+// broken gradient [K][4][Np] x 2 in FP64, from those tables or the plain rows
+// (both on the device), on `grid` blocks (asked for once per mesh: the query
+// costs as much as the launch)
+struct Grad64Args {
+    int grid;
+    const double *U, *geo, *ops;
+    const int *nodes;
+    const double *Dr, *Ds;
+    long long K;
+    double *gx, *gy;
+};
+cudaError_t grad64_grid(int p, long long K, int &grid);
+cudaError_t launch_grad64(int p, const Grad64Args &a, cudaStream_t st);
 cudaError_t launch_stage_mixed(int p, const LaunchShape &ls, const StageParams &sp,
                                const Phys<float> &ph, cudaStream_t st);
 // batch variant of the mixed kernel (IIP): grid for `ntiles` tiles of a tile table

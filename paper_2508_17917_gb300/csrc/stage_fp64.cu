@@ -93,10 +93,28 @@ cudaError_t launch64_p(const LaunchShape &ls, const StageParams &sp, const Stage
     return cudaLaunchKernelEx(&cfg, stage64_kernel<P, false>, sp, x, ph);
 }
 
+// Whether the symmetric contraction is taken.  It costs fewer FP64
+// instructions from p = 2 on (about, per node, with the plain rows and by symmetry:
+// p = 1 40 and 56, p = 2 64 and 54, p = 3 96 and 70, p = 4 136 and 96); at p = 2
+// its sums and differences round more than they save (RMS error 1.03 times that
+// of the plain rows), and below some thousand elements its two passes through
+// shared memory cost more than the pipe.  us, plain and symmetric: p = 1, 256^2
+// quads 42 and 60; p = 2 101 and 95; p = 3, 16^2 18.0 and 19.0, 32^2 20.2 and
+// 18.8, 256^2 226 and 186.
 template <int P>
-cudaError_t grad64_p(const double *U, const double *geo, const double *ops, const int *nodes, long long K, double *gx,
-                     double *gy, cudaStream_t st)
+constexpr bool grad_by_symmetry(long long K)
 {
+    return P > 3 || (P == 3 && K >= 1500);
+}
+
+// blocks of the FP64 gradient: those resident at once, capped by the tiles
+template <int P>
+cudaError_t grad64_grid_p(long long K, int &grid)
+{
+    if (!grad_by_symmetry<P>(K)) {
+        grid = static_cast<int>((K * Sym64<P>::Np + 127) / 128);
+        return cudaSuccess;
+    }
     using S = Sym64<P>;
     int per_sm = 0, dev = 0, sms = 0;
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, grad64_kernel<P>, S::NT, 0);
@@ -104,8 +122,18 @@ cudaError_t grad64_p(const double *U, const double *geo, const double *ops, cons
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const long long tiles = (K + S::EB - 1) / S::EB, most = static_cast<long long>(sms) * (per_sm < 1 ? 1 : per_sm);
-    grad64_kernel<P><<<static_cast<unsigned>(tiles < most ? tiles : most), S::NT, 0, st>>>(
-        U, geo, reinterpret_cast<const double2 *>(ops), nodes, K, gx, gy);
+    grid = static_cast<int>(tiles < most ? tiles : most);
+    return cudaSuccess;
+}
+
+template <int P>
+cudaError_t grad64_p(const Grad64Args &a, cudaStream_t st)
+{
+    if (grad_by_symmetry<P>(a.K))
+        grad64_kernel<P><<<a.grid, Sym64<P>::NT, 0, st>>>(a.U, a.geo, reinterpret_cast<const double2 *>(a.ops), a.nodes,
+                                                         a.K, a.gx, a.gy);
+    else
+        grad64_rows_kernel<P><<<a.grid, 128, 0, st>>>(a.U, a.Dr, a.Ds, a.geo, a.K, a.gx, a.gy);
     return cudaGetLastError();
 }
 
@@ -242,10 +270,16 @@ cudaError_t launch_stage_fp64(int p, const LaunchShape &ls, const StageParams &s
 #undef C_
 }
 
-cudaError_t launch_grad64(int p, const double *U, const double *geo, const double *ops, const int *nodes, long long K,
-                          double *gx, double *gy, cudaStream_t st)
+cudaError_t grad64_grid(int p, long long K, int &grid)
 {
-#define C_(P) grad64_p<P>(U, geo, ops, nodes, K, gx, gy, st)
+#define C_(P) grad64_grid_p<P>(K, grid)
+    DG_SWITCH_P(p, C_)
+#undef C_
+}
+
+cudaError_t launch_grad64(int p, const Grad64Args &a, cudaStream_t st)
+{
+#define C_(P) grad64_p<P>(a, st)
     DG_SWITCH_P(p, C_)
 #undef C_
 }
