@@ -43,16 +43,22 @@ struct dg_ctx {
     std::vector<double> geo64h;
     // device
     // FP64 and two-node kernels: symmetric operator tables, every face once, arrays between phases
-    dg::DevBuf<double> sym64, flux64, dh64, th64;
+    dg::DevBuf<double> sym64, flux64;                 // sym64: table, then the threads' nodes; flux64: all three arrays
+    size_t nsym64 = 0;
     bool no_coop = false;     // the stream refused a grid of theirs as a cooperative launch
-    dg::DevBuf<float> sym32;
+    dg::DevBuf<float> sym32;                          // likewise
+    size_t nsym32 = 0;
     dg::DevBuf<float4> fd32, rv32;
-    dg::DevBuf<int> symn, symn32;
     dg::DevBuf<int4> faces;
     int nfaces = 0;
     dg::DevBuf<double> K0a, K0b, K1, rtmp, geo64, ops64, Dr64, Ds64, src, scal, fpart, fxy, wface;
     dg::DevBuf<float> lam;                        // time-step bound: screened Lambda_K
-    dg::DevBuf<unsigned> dtw;                     // ... and its words (zero between calls)
+    // zero between calls: [0, 8) time-step bound, [8, 10) grid barriers, [10] finished
+    // blocks of the wall-force kernel, [11] a bounded wait gave up
+    dg::DevBuf<unsigned> words;
+    unsigned *bar() { return words.ptr + 8; }
+    unsigned *ticket() { return words.ptr + 10; }
+    int *bar_err() { return reinterpret_cast<int *>(words.ptr + 11); }
     dg::DevBuf<float> geo32, ops32, P0a, P0b;     // mixed path: pressures of the two K0 buffers
     dg::DevBuf<float4> S0a, S0b;                  // mixed path: FP32 copies of the two K0 buffers
     dg::DevBuf<int4> conn;
@@ -72,8 +78,6 @@ struct dg_ctx {
     bool fused = false;
     dg::LaunchShape fshape;
     int fshape_variant = 0;
-    dg::DevBuf<unsigned> bar;
-    dg::DevBuf<int> bar_err;
     unsigned bar_limit = 1u << 24;
     bool bar_used = false;
     bool copy_used = false;           // a stage kernel with bounded copy waits ran (reported where the API synchronises anyway)
@@ -91,14 +95,10 @@ struct dg_ctx {
     float4 *sother() { return cur_is_a ? S0b.ptr : S0a.ptr; }
     float *pcur() { return cur_is_a ? P0a.ptr : P0b.ptr; }
     float *pother() { return cur_is_a ? P0b.ptr : P0a.ptr; }
-    // finished blocks of the wall-force kernel: the last word of scal
-    unsigned *ticket() { return reinterpret_cast<unsigned *>(scal.ptr + 3); }
     cudaEvent_t tune_ev[9] = {};     // mixed: marks of the stage-shape timing
     void drop_phases()
     {
         flux64.release();
-        dh64.release();
-        th64.release();
         faces.release();
     }
     void drop_handoff()
@@ -149,20 +149,10 @@ dg_status cuda_fail(dg_ctx *c, cudaError_t e, const char *where)
         if (e_ != cudaSuccess) return cuda_fail(ctx, e_, #expr);  \
     } while (0)
 
-// the words of the grid barriers, zero before their first launch
-dg_status need_barrier(dg_ctx *c)
-{
-    if (c->bar.ptr) return DG_OK;
-    DG_CUDA(c, c->bar.alloc(2));
-    DG_CUDA(c, cudaMemset(c->bar.ptr, 0, 2 * sizeof(unsigned)));
-    return DG_OK;
-}
-
 // clear the error flag and the barrier words a launch that gave up left behind
 dg_status wait_gave_up(dg_ctx *c)
 {
-    DG_CUDA(c, cudaMemset(c->bar_err.ptr, 0, sizeof(int)));
-    if (c->bar.ptr) DG_CUDA(c, cudaMemset(c->bar.ptr, 0, 2 * sizeof(unsigned)));
+    DG_CUDA(c, cudaMemset(c->words.ptr + 8, 0, 4 * sizeof(unsigned)));
     return fail(c, DG_ETIMEOUT, kWaitGaveUp);
 }
 
@@ -207,6 +197,40 @@ void manufactured_source(double x, double y, double kappa, double C2, const dg_p
 // C1 (1+theta)^2 (d+1) of Eq. penalty_final, d = 2
 double sigma_factor(const dg_params &p) { return p.C1 * (1.0 + p.theta) * (1.0 + p.theta) * 3.0; }
 
+// Symmetric operator tables with the threads' nodes behind them, one upload
+// each at first use: the FP64 stage and gradient, and the hand-off kernel.
+dg_status sym_tables64(dg_ctx *c)
+{
+    if (c->sym64.ptr) return DG_OK;
+    std::vector<double> tab;
+    std::vector<int> nodes;
+    if (!dg::build_sym64_tables(c->ops, tab, nodes)) return fail(c, DG_EINVAL, "operators without the mirror symmetry");
+    c->nsym64 = tab.size();
+    tab.resize(c->nsym64 + (nodes.size() + 1) / 2);
+    std::memcpy(tab.data() + c->nsym64, nodes.data(), nodes.size() * sizeof(int));
+    DG_CUDA(c, c->sym64.alloc(tab.size()));
+    DG_CUDA(c, cudaMemcpy(c->sym64.ptr, tab.data(), tab.size() * sizeof(double), cudaMemcpyHostToDevice));
+    return DG_OK;
+}
+
+const int *sym_nodes64(const dg_ctx *c) { return reinterpret_cast<const int *>(c->sym64.ptr + c->nsym64); }
+
+dg_status sym_tables32(dg_ctx *c)
+{
+    if (c->sym32.ptr) return DG_OK;
+    std::vector<double> tab;
+    std::vector<int> nodes, slots;
+    std::vector<float> tab32;
+    if (!dg::build_sym64_tables(c->ops, tab, nodes)) return fail(c, DG_EINVAL, "operators without the mirror symmetry");
+    dg::build_sym32_tables(c->ops, tab, nodes, tab32, slots);
+    c->nsym32 = tab32.size();
+    tab32.resize(c->nsym32 + slots.size());
+    std::memcpy(tab32.data() + c->nsym32, slots.data(), slots.size() * sizeof(int));
+    DG_CUDA(c, c->sym32.alloc(tab32.size()));
+    DG_CUDA(c, cudaMemcpy(c->sym32.ptr, tab32.data(), tab32.size() * sizeof(float), cudaMemcpyHostToDevice));
+    return DG_OK;
+}
+
 // What the three-phase FP64 kernel keeps between its phases, for a mesh with
 // connectivity `conn` (host; null: read back).  Over-integration does not run
 // it; without memory for it, or where the stream refused its grid, the mesh
@@ -218,6 +242,8 @@ dg_status phase_arrays(dg_ctx *c, const int4 *conn)
         return DG_OK;
     }
     if (c->flux64.ptr) return DG_OK;
+    dg_status st = sym_tables64(c);
+    if (st != DG_OK) return st;
     std::vector<int4> back, fl;
     if (!conn) {
         back.resize(c->K);
@@ -228,9 +254,7 @@ dg_status phase_arrays(dg_ctx *c, const int4 *conn)
     c->nfaces = static_cast<int>(fl.size());
     const size_t nd = static_cast<size_t>(c->K) * 4 * c->ops.Np, nfn = static_cast<size_t>(c->K) * 3 * c->ops.Nfp;
     cudaError_t e = c->faces.alloc(fl.size());
-    if (e == cudaSuccess) e = c->dh64.alloc(4 * nfn);
-    if (e == cudaSuccess && c->prm.theta != 0.0) e = c->th64.alloc(8 * nfn);
-    if (e == cudaSuccess) e = c->flux64.alloc(2 * nd);
+    if (e == cudaSuccess) e = c->flux64.alloc(2 * nd + (c->prm.theta != 0.0 ? 12 : 4) * nfn);
     if (e == cudaErrorMemoryAllocation) {
         cudaGetLastError();
         c->drop_phases();
@@ -275,6 +299,8 @@ dg_status two_node_shape(dg_ctx *c)
     DG_CUDA(c, dg::stage_shape_mixed2(c->prm.p, c->K, false, false, !c->no_coop, c->shape2));
     c->fshape_variant = 0;
     if (!c->shape2.handoff) return DG_OK;
+    dg_status st = sym_tables32(c);
+    if (st != DG_OK) return st;
     cudaError_t e = c->fd32.alloc(2 * static_cast<size_t>(c->K) * 3 * c->ops.Nfp);
     if (e == cudaSuccess) e = c->rv32.alloc(static_cast<size_t>(c->K) * c->ops.Np);
     if (e != cudaErrorMemoryAllocation) {
@@ -290,7 +316,7 @@ dg_status two_node_shape(dg_ctx *c)
 // s: stage of a step, -1 for a residual
 dg::Stage2Args stage2_args(const dg_ctx *c, int s)
 {
-    return dg::stage2_args(c->sym32.ptr, c->symn32.ptr, c->fd32.ptr, c->rv32.ptr, nullptr, c->fd32.n / 2, s);
+    return dg::stage2_args(c->sym32.ptr, reinterpret_cast<const int *>(c->sym32.ptr + c->nsym32), c->fd32.ptr, c->rv32.ptr, nullptr, c->fd32.n / 2, s);
 }
 
 dg_status run_stage(dg_ctx *c, int s, double t, double dt, const double vw[2], int mode,
@@ -344,13 +370,14 @@ dg_status run_stage(dg_ctx *c, int s, double t, double dt, const double vw[2], i
         sp.ops = c->ops64.ptr;
         if (c->shape.phases) {
             // grid barriers between its phases, reported through the barrier flag
-            sp.bar = c->bar.ptr;
-            sp.bar_err = c->bar_err.ptr;
+            sp.bar = c->bar();
+            sp.bar_err = c->bar_err();
             sp.bar_limit = c->bar_limit;
             c->copy_used = true;
         }
-        const dg::Stage64Args a64{c->sym64.ptr, c->symn.ptr, c->faces.ptr, c->nfaces, c->flux64.ptr, c->dh64.ptr,
-                                  c->th64.ptr};
+        double *const dh = c->flux64.ptr + 2 * ndof(c);
+        const dg::Stage64Args a64{c->sym64.ptr, sym_nodes64(c), c->faces.ptr, c->nfaces, c->flux64.ptr, dh,
+                                  dh + static_cast<size_t>(c->K) * 12 * c->ops.Nfp};
         const dg::Phys<double> ph = make_phys<double>(c->prm, vw);
         e = dg::launch_stage_fp64(c->prm.p, c->shape, sp, a64, ph, c->stream);
         if (e == cudaErrorCooperativeLaunchTooLarge) {
@@ -365,15 +392,15 @@ dg_status run_stage(dg_ctx *c, int s, double t, double dt, const double vw[2], i
         sp.ops = (c->shape.variant == 3) ? static_cast<const void *>(c->tcfrag.ptr) : c->ops32.ptr;
         if (c->shape.variant == 3) {
             // its bounded copy waits report through the barrier flag
-            sp.bar_err = c->bar_err.ptr;
+            sp.bar_err = c->bar_err();
             sp.bar_limit = c->bar_limit;
             c->copy_used = true;
             e = dg::launch_stage_tc(c->prm.p, false, false, c->shape, sp, make_phys<float>(c->prm, vw), c->stream);
         }
         else if (c->shape.variant == 2) {
             if (c->shape.handoff) {
-                sp.bar = c->bar.ptr;
-                sp.bar_err = c->bar_err.ptr;
+                sp.bar = c->bar();
+                sp.bar_err = c->bar_err();
                 sp.bar_limit = c->bar_limit;
                 c->copy_used = true;
             }
@@ -454,13 +481,6 @@ dg_status dg_create(const dg_params *params, void *cuda_stream, dg_ctx **out)
         delete c;
         return DG_ECUDA;
     }
-    if (p.precision == DG_PRECISION_MIXED)
-        for (auto &e : c->tune_ev)
-            if (cudaEventCreate(&e) != cudaSuccess) {
-                cudaGetLastError();
-                delete c;
-                return DG_ECUDA;
-            }
     const int Np = c->ops.Np, NF = 3 * c->ops.Nfp;
     std::vector<double> o64;
     o64.insert(o64.end(), c->ops.Dr.begin(), c->ops.Dr.end());
@@ -480,42 +500,15 @@ dg_status dg_create(const dg_params *params, void *cuda_stream, dg_ctx **out)
     std::vector<float> o32(o64.begin(), o64.end());
     if (c->ops64.alloc(o64.size()) != cudaSuccess || c->ops32.alloc(o32.size()) != cudaSuccess ||
         c->Dr64.alloc(Np * Np) != cudaSuccess || c->Ds64.alloc(Np * Np) != cudaSuccess ||
-        c->fmask.alloc(NF) != cudaSuccess || c->flag.alloc(1) != cudaSuccess || c->bar_err.alloc(1) != cudaSuccess ||
-        c->scal.alloc(4) != cudaSuccess || c->dtw.alloc(8) != cudaSuccess || c->wface.alloc(c->ops.Nfp) != cudaSuccess) {
+        c->fmask.alloc(NF) != cudaSuccess || c->flag.alloc(1) != cudaSuccess || c->words.alloc(12) != cudaSuccess ||
+        c->scal.alloc(4) != cudaSuccess || c->wface.alloc(c->ops.Nfp) != cudaSuccess) {
         cudaGetLastError();
         delete c;
         return DG_ECUDA;
     }
-    cudaMemset(c->bar_err.ptr, 0, sizeof(int));
-    cudaMemset(c->scal.ptr, 0, 4 * sizeof(double));
-    cudaMemset(c->dtw.ptr, 0, 8 * sizeof(unsigned));
+    cudaMemset(c->words.ptr, 0, 12 * sizeof(unsigned));
     cudaMemcpy(c->ops64.ptr, o64.data(), o64.size() * sizeof(double), cudaMemcpyHostToDevice);
     cudaMemcpy(c->ops32.ptr, o32.data(), o32.size() * sizeof(float), cudaMemcpyHostToDevice);
-    {
-        std::vector<double> tab;
-        std::vector<int> nodes;
-        if (!dg::build_sym64_tables(c->ops, tab, nodes)) {
-            delete c;
-            return DG_EINVAL;
-        }
-        if (c->sym64.alloc(tab.size()) != cudaSuccess || c->symn.alloc(nodes.size()) != cudaSuccess) {
-            cudaGetLastError();
-            delete c;
-            return DG_ECUDA;
-        }
-        cudaMemcpy(c->sym64.ptr, tab.data(), tab.size() * sizeof(double), cudaMemcpyHostToDevice);
-        cudaMemcpy(c->symn.ptr, nodes.data(), nodes.size() * sizeof(int), cudaMemcpyHostToDevice);
-        std::vector<float> tab32;
-        std::vector<int> slots;
-        dg::build_sym32_tables(c->ops, tab, nodes, tab32, slots);
-        if (c->sym32.alloc(tab32.size()) != cudaSuccess || c->symn32.alloc(slots.size()) != cudaSuccess) {
-            cudaGetLastError();
-            delete c;
-            return DG_ECUDA;
-        }
-        cudaMemcpy(c->sym32.ptr, tab32.data(), tab32.size() * sizeof(float), cudaMemcpyHostToDevice);
-        cudaMemcpy(c->symn32.ptr, slots.data(), slots.size() * sizeof(int), cudaMemcpyHostToDevice);
-    }
     if (dg::stage_tc_supported(p.p)) {
         std::vector<float> frag;
         dg::build_tc_fragments(Np, NF, c->ops.Dr.data(), c->ops.Ds.data(), c->ops.LIFT.data(), c->ops.Wr.data(),
@@ -573,10 +566,6 @@ dg_status dg_set_fused_steps(dg_ctx *c, int on)
     c->err.clear();
     if (on && (c->prm.precision != DG_PRECISION_MIXED || c->prm.theta != 0.0))
         return fail(c, DG_EUNSUPPORTED, "fused steps use the mixed-precision IIP kernels");
-    if (on) {
-        dg_status st = need_barrier(c);
-        if (st != DG_OK) return st;
-    }
     c->fused = on != 0;
     return DG_OK;
 }
@@ -594,7 +583,7 @@ dg_status dg_barrier_status(dg_ctx *c)
     c->err.clear();
     if (!c->bar_used && !c->copy_used) return DG_OK;
     int e = 0;
-    DG_CUDA(c, cudaMemcpyAsync(&e, c->bar_err.ptr, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+    DG_CUDA(c, cudaMemcpyAsync(&e, c->bar_err(), sizeof(int), cudaMemcpyDeviceToHost, c->stream));
     DG_CUDA(c, cudaStreamSynchronize(c->stream));
     c->bar_used = false;
     c->copy_used = false;
@@ -656,10 +645,6 @@ dg_status dg_set_mesh(dg_ctx *c, int64_t Nv, const double *vx, const double *vy,
     DG_CUDA(c, c->lam.alloc(K));
     DG_CUDA(c, cudaMemcpy(c->geo64.ptr, geo.data(), geo.size() * sizeof(double), cudaMemcpyHostToDevice));
     DG_CUDA(c, cudaMemcpy(c->conn.ptr, conn.data(), K * sizeof(int4), cudaMemcpyHostToDevice));
-    {
-        dg_status bs = need_barrier(c);
-        if (bs != DG_OK) return bs;
-    }
     if (c->prm.precision == DG_PRECISION_MIXED) {
         std::vector<float> g32(geo.begin(), geo.end());
         DG_CUDA(c, c->geo32.alloc(g32.size()));
@@ -766,7 +751,7 @@ dg_status dg_get_state(dg_ctx *c, double *U, int on_device)
     // asynchronous after plain stage launches)
     const bool check = !on_device && (c->bar_used || c->copy_used);
     int e = 0;
-    if (check) DG_CUDA(c, cudaMemcpyAsync(&e, c->bar_err.ptr, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+    if (check) DG_CUDA(c, cudaMemcpyAsync(&e, c->bar_err(), sizeof(int), cudaMemcpyDeviceToHost, c->stream));
     DG_CUDA(c, cudaMemcpyAsync(U, c->cur(), ndof(c) * sizeof(double),
                                on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, c->stream));
     if (!on_device) DG_CUDA(c, cudaStreamSynchronize(c->stream));
@@ -839,6 +824,8 @@ static dg_status tune_stage(dg_ctx *c, const double vw[2])
         dg_status st = two_node_shape(c);
         if (st != DG_OK) return st;
     }
+    for (auto &e : c->tune_ev)
+        if (!e) DG_CUDA(c, cudaEventCreate(&e));
     // timed on 2^21 nodes at most, four times the L2 cache
     struct Part {
         dg_ctx *c;
@@ -897,7 +884,7 @@ dg_status dg_rhs(dg_ctx *c, double t, const double vw[2], double *dUdt, int on_d
         // the error flag of the bounded device waits comes back with the residual
         const bool check = c->bar_used || c->copy_used;
         int e = 0;
-        if (check) DG_CUDA(c, cudaMemcpyAsync(&e, c->bar_err.ptr, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+        if (check) DG_CUDA(c, cudaMemcpyAsync(&e, c->bar_err(), sizeof(int), cudaMemcpyDeviceToHost, c->stream));
         DG_CUDA(c, cudaMemcpyAsync(dUdt, out, ndof(c) * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
         DG_CUDA(c, cudaStreamSynchronize(c->stream));
         if (check) {
@@ -945,10 +932,10 @@ static dg_status run_fused_step(dg_ctx *c, double dt, const double vw[2])
     sp.first_stage = 1;
     sp.geo = c->geo32.ptr;
     sp.ops = (c->fshape.variant == 3) ? static_cast<const void *>(c->tcfrag.ptr) : c->ops32.ptr;
-    sp.bar = c->bar.ptr;
-    sp.bar_err = c->bar_err.ptr;
+    sp.bar = c->bar();
+    sp.bar_err = c->bar_err();
     sp.bar_limit = c->bar_limit;
-    DG_CUDA(c, cudaMemsetAsync(c->bar.ptr, 0, 2 * sizeof(unsigned), c->stream));
+    DG_CUDA(c, cudaMemsetAsync(c->bar(), 0, 2 * sizeof(unsigned), c->stream));
     if (c->fshape.variant == 3)
         DG_CUDA(c, dg::launch_stage_tc(c->prm.p, false, true, c->fshape, sp, make_phys<float>(c->prm, vw), c->stream));
     else if (c->fshape.variant == 2)
@@ -1007,8 +994,8 @@ dg_status dg_compute_dt(dg_ctx *c, double cfl, const double vw[2], double *dt)
     dg::Phys<double> ph = make_phys<double>(c->prm, vw);
     const double sf = sigma_factor(c->prm);
     DG_CUDA(c, dg::launch_dt_screen(aux_mesh(c), make_phys<float>(c->prm, vw), c->prm.gamma - 1.0,
-                                    static_cast<float>(sf), c->lam.ptr, c->dtw.ptr, c->stream));
-    DG_CUDA(c, dg::launch_dt_confirm(aux_mesh(c), ph, sf, c->lam.ptr, c->dtw.ptr, c->scal.ptr, c->stream));
+                                    static_cast<float>(sf), c->lam.ptr, c->words.ptr, c->stream));
+    DG_CUDA(c, dg::launch_dt_confirm(aux_mesh(c), ph, sf, c->lam.ptr, c->words.ptr, c->scal.ptr, c->stream));
     c->launches += 2;
     double lam = 0.0;
     DG_CUDA(c, cudaMemcpyAsync(&lam, c->scal.ptr, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
@@ -1070,8 +1057,10 @@ dg_status dg_broken_gradient(dg_ctx *c, double *gx, double *gy, int on_device, i
         oy = c->gtmp.ptr + n;
     }
     if (impl == 0) {
+        dg_status gs = sym_tables64(c);
+        if (gs != DG_OK) return gs;
         if (!c->ggrid) DG_CUDA(c, dg::grad64_grid(c->prm.p, c->K, c->ggrid));
-        const dg::Grad64Args a{c->ggrid, c->cur(), c->geo64.ptr, c->sym64.ptr, c->symn.ptr, c->Dr64.ptr, c->Ds64.ptr,
+        const dg::Grad64Args a{c->ggrid, c->cur(), c->geo64.ptr, c->sym64.ptr, sym_nodes64(c), c->Dr64.ptr, c->Ds64.ptr,
                                c->K, ox, oy};
         DG_CUDA(c, dg::launch_grad64(c->prm.p, a, c->stream));
     } else {
@@ -1091,7 +1080,7 @@ dg_status dg_broken_gradient(dg_ctx *c, double *gx, double *gy, int on_device, i
         }
         a.bimg = c->gimg.ptr;
         a.upload_ops = !c->gimg_ready;   // the operators are fixed by p: one upload per context
-        a.err = c->bar_err.ptr;        // reported by dg_barrier_status, as for fused steps
+        a.err = c->bar_err();        // reported by dg_barrier_status, as for fused steps
         c->bar_used = true;
         DG_CUDA(c, dg::launch_grad_tc05(c->prm.p, a, c->stream));
         c->gimg_ready = true;
