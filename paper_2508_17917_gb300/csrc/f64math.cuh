@@ -7,8 +7,10 @@
 // FP32 approximation of the mantissa (special-function unit, no FP64
 // instruction; the exponent is integer work) and take one third-order
 // Householder step, y (1 + e + e^2) and y (1 + e/2 + 3 e^2/8) with e the
-// residual of the seed y, |e| < 1e-6: the truncation is below 1e-18, so the
-// results are within one unit in the last place.  The largest eigenvalue of
+// residual of the seed y, |e| < 1e-6: the truncation is below 1e-18 and the
+// last multiply-add rounds once, so these are within one unit in the last
+// place (0.51); a square root, x times the rounded inverse root, rounds a second
+// time and is within two (1.6).  The largest eigenvalue of
 // the penalty matrix starts from the FP32 polynomial of pair2.cuh and takes
 // two Newton steps on 4 w^3 - 3 w = r.
 // Arguments outside the plain range (zero, subnormal, infinite, NaN, very
