@@ -13,7 +13,9 @@
 // Of a single mesh's two-node kernels this is the one for p = 3 below 25,000
 // elements and p = 5 below 15,000, where the hand-off kernel's extra volume
 // phase and barrier in a step's first stage are not earned back or its tiles
-// leave a wave nearly empty (stage_shape_mixed2).
+// leave a wave nearly empty (stage_shape_mixed2), and at every degree for a
+// mesh without memory for what that kernel hands on, or a stream that cannot
+// hold its first stage's grid at once (two_node_shape).
 #pragma once
 #include "dg_stage_mixed.cuh"
 

@@ -106,14 +106,41 @@ def test_over_integration_keeps_no_phase_arrays(dg):
     assert free0 > phases
 
 
-def take_all_but(n):
+@pytest.fixture
+def take_all_but(dg):
+    """take_all_but(n) leaves about n bytes of the device's memory."""
     import torch
-    torch.cuda.empty_cache()
-    return torch.empty(free_bytes() - n, dtype=torch.uint8, device="cuda")
+    cu = C.CDLL("libcuda.so.1")
+    held = []
+
+    def alloc(size, most):
+        got = 0
+        p = C.c_uint64()
+        while got + size <= most and cu.cuMemAlloc_v2(C.byref(p), C.c_size_t(size)) == 0:
+            held.append((p.value, size))
+            got += size
+        return got
+
+    def take(n):
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        for size in (1024 * MB, 64 * MB, 2 * MB):
+            alloc(size, 1 << 40)
+        freed = 0
+        while freed < n:
+            p, size = held.pop()
+            assert cu.cuMemFree_v2(C.c_uint64(p)) == 0
+            freed += size
+        alloc(2 * MB, freed - n)
+
+    yield take
+    torch.cuda.synchronize()
+    for p, _ in held:
+        cu.cuMemFree_v2(C.c_uint64(p))
 
 
 @pytest.mark.parametrize("p,theta", [(4, 0.0), (2, 1.0)])
-def test_fp64_without_memory_between_the_phases(dg, part_of_the_device, p, theta):
+def test_fp64_without_memory_between_the_phases(dg, part_of_the_device, take_all_but, p, theta):
     """All but what the state needs, and half of what the phases need besides,
     is taken.  Same kernel, and so the same bits, as on a part of the device."""
     mesh = dg_inputs.periodic_square(400)               # 320,000 elements
@@ -126,23 +153,16 @@ def test_fp64_without_memory_between_the_phases(dg, part_of_the_device, p, theta
     alone.steps(0.0, dt, 1)
     after = alone.get_state()
     del alone
-    free0 = free_bytes()
-    s = dg.Solver(mesh, p, "fp64", stream=stream(), **kw)
-    s.set_state(U)
-    s.rhs()
-    used = free0 - free_bytes()
-    del s
     Np, nfn = (p + 1) * (p + 2) // 2, 3 * (p + 1)
+    state = mesh.K * (4 * 32 * Np + 128 + 16 + 4)       # two states, register, residual; element records
     phases = mesh.K * (64 * Np + 32 * nfn + (64 * nfn if theta else 0))
-    assert used > phases
-    hold = take_all_but(used - phases // 2)
+    take_all_but(state + phases // 2)
     s = dg.Solver(mesh, p, "fp64", stream=stream(), **kw)
     s.set_state(U)
     assert np.array_equal(s.rhs(), want)
     assert s.dt(0.3) == dt
     s.steps(0.0, dt, 1)
     assert np.array_equal(s.get_state(), after)
-    del hold
 
 
 @pytest.mark.parametrize("p,variant", [(1, 2), (2, 2), (4, 2), (6, 2), (4, 0), (6, 0)])
@@ -164,7 +184,7 @@ def test_mixed_on_a_part_of_the_device(dg, part_of_the_device, p, variant):
 
 
 @pytest.mark.parametrize("p", [2, 4])
-def test_two_nodes_without_memory_between_the_stages(dg, part_of_the_device, p):
+def test_two_nodes_without_memory_between_the_stages(dg, part_of_the_device, take_all_but, p):
     """As for the FP64 phases; five launches a step and one."""
     mesh = dg_inputs.periodic_square(400)
     alone = dg.Solver(mesh, p, "mixed", stream=part_of_the_device, mu=1e-3)
@@ -175,16 +195,10 @@ def test_two_nodes_without_memory_between_the_stages(dg, part_of_the_device, p):
     alone.steps(0.0, 1e-5, 2)
     after = alone.get_state()
     del alone
-    free0 = free_bytes()
-    s = dg.Solver(mesh, p, "mixed", stream=stream(), mu=1e-3)
-    s.set_variant(2)
-    s.set_state(U)
-    s.rhs()
-    used = free0 - free_bytes()
-    del s
-    stages = mesh.K * 16 * ((p + 1) * (p + 2) // 2 + 6 * (p + 1))
-    assert used > stages
-    hold = take_all_but(used - stages // 2)
+    Np = (p + 1) * (p + 2) // 2
+    state = mesh.K * (4 * 32 * Np + 2 * 16 * Np + 2 * 4 * ((Np + 3) & ~3) + 192 + 16 + 4)
+    stages = mesh.K * 16 * (Np + 6 * (p + 1))
+    take_all_but(state + stages // 2)
     s = dg.Solver(mesh, p, "mixed", stream=stream(), mu=1e-3)
     s.set_variant(2)
     s.set_state(U)
@@ -195,7 +209,6 @@ def test_two_nodes_without_memory_between_the_stages(dg, part_of_the_device, p):
     s.set_state(U)
     s.steps(0.0, 1e-5, 2)
     assert np.abs(s.get_state() - after).max() <= 1e-9 * np.abs(after).max()
-    del hold
 
 
 def test_the_two_node_arrays_go_when_another_shape_is_taken(dg):
@@ -216,7 +229,7 @@ def test_the_two_node_arrays_go_when_another_shape_is_taken(dg):
         assert abs(without - free_bytes()) <= 4 * MB
 
 
-def test_batch_without_memory_between_the_stages(dg):
+def test_batch_without_memory_between_the_stages(dg, take_all_but):
     """A group takes the one-node shape instead of the two-node shape."""
     kw = dict(rho_inf=1.0, u_inf=1.0, v_inf=0.0, p_inf=17.857142857142858)
     case = dict(mesh=dg_inputs.ogrid_cylinder(400, 100, 0.5, 20.0, seed=1), p=4, mu=0.01, y0=0.0, ydot0=0.0, M_r=1.0,
@@ -227,9 +240,9 @@ def test_batch_without_memory_between_the_stages(dg):
         b.set_variant(variant)
         x, y = b.node_coords(0)
         b.set_state(0, to_kcn(dg_inputs.free_stream(x.shape, rho=1.0, u=1.0, v=0.0, p=kw["p_inf"])))
-        hold = take_all_but(24 * MB) if variant == 2 else None
+        if variant == 2:
+            take_all_but(24 * MB)
         b.run(0.3, 2, use_graph=False)
         assert b.variant(0) == 1
         got.append(b.get_state(0))
-        del hold
     assert np.array_equal(got[0], got[1])
