@@ -48,7 +48,7 @@ struct dg_ctx {
     bool no_coop = false;     // the stream refused a grid of theirs as a cooperative launch
     dg::DevBuf<float> sym32;                          // likewise
     size_t nsym32 = 0;
-    dg::DevBuf<float4> fd32, rv32;
+    dg::DevBuf<float4> hand32;                        // face records [2][K][3 Nfp], divergence [K][Np]
     dg::DevBuf<int4> faces;
     int nfaces = 0;
     dg::DevBuf<double> K0a, K0b, K1, rtmp, geo64, ops64, Dr64, Ds64, src, scal, fpart, fxy, wface;
@@ -103,8 +103,7 @@ struct dg_ctx {
     }
     void drop_handoff()
     {
-        fd32.release();
-        rv32.release();
+        hand32.release();
     }
     ~dg_ctx()
     {
@@ -276,7 +275,7 @@ template <typename T>
 cudaError_t alloc_needed(dg_ctx *c, dg::DevBuf<T> &b, size_t n)
 {
     cudaError_t e = b.alloc(n);
-    if (e != cudaErrorMemoryAllocation || !(c->flux64.ptr || c->fd32.ptr)) return e;
+    if (e != cudaErrorMemoryAllocation || !(c->flux64.ptr || c->hand32.ptr)) return e;
     cudaGetLastError();
     if (c->flux64.ptr) {
         c->drop_phases();                  // cudaFree waits for the kernels that use them
@@ -295,14 +294,13 @@ cudaError_t alloc_needed(dg_ctx *c, dg::DevBuf<T> &b, size_t n)
 // kernel whose stages stand alone.
 dg_status two_node_shape(dg_ctx *c)
 {
-    if (c->shape2.handoff && c->rv32.ptr) return DG_OK;
+    if (c->shape2.handoff && c->hand32.ptr) return DG_OK;
     DG_CUDA(c, dg::stage_shape_mixed2(c->prm.p, c->K, false, false, !c->no_coop, c->shape2));
     c->fshape_variant = 0;
     if (!c->shape2.handoff) return DG_OK;
     dg_status st = sym_tables32(c);
     if (st != DG_OK) return st;
-    cudaError_t e = c->fd32.alloc(2 * static_cast<size_t>(c->K) * 3 * c->ops.Nfp);
-    if (e == cudaSuccess) e = c->rv32.alloc(static_cast<size_t>(c->K) * c->ops.Np);
+    const cudaError_t e = c->hand32.alloc(static_cast<size_t>(c->K) * (6 * c->ops.Nfp + c->ops.Np));
     if (e != cudaErrorMemoryAllocation) {
         DG_CUDA(c, e);
         return DG_OK;
@@ -313,10 +311,13 @@ dg_status two_node_shape(dg_ctx *c)
     return DG_OK;
 }
 
-// s: stage of a step, -1 for a residual
+// s: stage of a step, -1 for a residual.  By the elements of the whole mesh:
+// the tuner runs a part of it.
 dg::Stage2Args stage2_args(const dg_ctx *c, int s)
 {
-    return dg::stage2_args(c->sym32.ptr, reinterpret_cast<const int *>(c->sym32.ptr + c->nsym32), c->fd32.ptr, c->rv32.ptr, nullptr, c->fd32.n / 2, s);
+    const size_t K = c->hand32.n / (6 * c->ops.Nfp + c->ops.Np), n = K * 3 * c->ops.Nfp;
+    return dg::stage2_args(c->sym32.ptr, reinterpret_cast<const int *>(c->sym32.ptr + c->nsym32), c->hand32.ptr,
+                           c->hand32.ptr + 2 * n, nullptr, n, s);
 }
 
 dg_status run_stage(dg_ctx *c, int s, double t, double dt, const double vw[2], int mode,
@@ -863,7 +864,9 @@ static dg_status tune_stage(dg_ctx *c, const double vw[2])
         }
     }
     c->shape = pick;
-    if (pick.variant != 2) c->drop_handoff();
+    // given back if another shape was picked; a few megabytes stay, a free costs
+    // as much as the step
+    if (pick.variant != 2 && c->hand32.n * sizeof(float4) > (32u << 20)) c->drop_handoff();
     c->tuned = true;
     return DG_OK;
 }

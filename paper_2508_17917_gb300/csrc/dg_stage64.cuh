@@ -7,7 +7,8 @@
 // instructions (one kernel that staged a tile, formed the neighbours'
 // gradients and evaluated every face from both sides took about 20,700 per
 // element at p = 4 and kept the FP64 pipe full: 1121 us per stage on 32,768
-// elements).  This one takes about 7,000, in three phases of one cooperative
+// elements; it is dg_stage.cuh, kept for contexts that this one does not
+// suit).  This one takes about 7,000, in three phases of one cooperative
 // launch with a grid barrier between them:
 //   V  per element: broken gradient, total flux, contravariant components,
 //      kept in memory for every node;
