@@ -496,14 +496,18 @@ cudaError_t launch_batch_forces_record(const double *partial, const int *wseg, B
 cudaError_t launch_dt_confirm(const AuxMesh &m, const Phys<double> &ph, double sig_fac, const float *lam,
                               unsigned *words, double *out, cudaStream_t st)
 {
-    // one tile a block where the device holds that many (8 blocks an SM): a
-    // block takes its tiles one after the other, and on a uniform state every
-    // element is a candidate (8,192 elements, p = 1, uniform: 252 us a call
-    // with a block per 128 elements, 84 us now)
+    // A block takes its tiles one after the other, and on a uniform state every
+    // element is a candidate: few elements go one tile to a block, up to two
+    // blocks an SM, many 128 to a block, up to eight.  (More blocks cost the
+    // usual call, with a handful of candidates, a microsecond per hundred.)  us
+    // a call, uniform state, p = 1, with a block per 128 elements and now: 512
+    // elements 252 and 61, 8,192 258 and 100.
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const long long tiles = (m.K + kDtTile - 1) / kDtTile, most = 8ll * (sms > 0 ? sms : 1);
+    sms = sms > 0 ? sms : 1;
+    const long long tiles = (m.K + kDtTile - 1) / kDtTile, scans = (m.K + 127) / 128;
+    const long long most = scans < 2 * sms ? 2 * sms : (scans < 8 * sms ? scans : 8 * sms);
     const int blocks = static_cast<int>(tiles < most ? tiles : most);
     dt_confirm_kernel<<<blocks, 128, 0, st>>>(m, ph, sig_fac, lam, words, out);
     return cudaGetLastError();
