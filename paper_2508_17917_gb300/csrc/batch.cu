@@ -646,7 +646,7 @@ dg_status dg_batch_create(const dg_params *common, int ncases, const dg_case *ca
         std::vector<double> tab;
         std::vector<int> nodes, slots;
         std::vector<float> tab32;
-        if (!dg::build_sym64_tables(g.ops, tab, nodes)) return bail(DG_EINVAL);
+        if (!dg::build_sym64_tables(g.ops, false, tab, nodes)) return bail(DG_EINVAL);
         dg::build_sym32_tables(g.ops, tab, nodes, tab32, slots);
         chk(g.sym32.alloc(tab32.size()));
         chk(g.symn32.alloc(slots.size()));

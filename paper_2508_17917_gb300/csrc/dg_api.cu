@@ -43,11 +43,12 @@ struct dg_ctx {
     std::vector<double> geo64h;
     // device
     // FP64 and two-node kernels: symmetric operator tables, every face once, arrays between phases
-    dg::DevBuf<double> sym64, flux64;                 // sym64: table, then the threads' nodes; flux64: all three arrays
-    size_t nsym64 = 0;
+    dg::DevBuf<double> flux64;                        // all three arrays
+    // behind the operators in ops64 and ops32: a table, then the threads' nodes
+    const double *sym64 = nullptr;
+    const float *sym32 = nullptr;
+    const int *symn64 = nullptr, *symn32 = nullptr;
     bool no_coop = false;     // the stream refused a grid of theirs as a cooperative launch
-    dg::DevBuf<float> sym32;                          // likewise
-    size_t nsym32 = 0;
     dg::DevBuf<float4> hand32;                        // face records [2][K][3 Nfp], divergence [K][Np]
     dg::DevBuf<int4> faces;
     int nfaces = 0;
@@ -196,40 +197,6 @@ void manufactured_source(double x, double y, double kappa, double C2, const dg_p
 // C1 (1+theta)^2 (d+1) of Eq. penalty_final, d = 2
 double sigma_factor(const dg_params &p) { return p.C1 * (1.0 + p.theta) * (1.0 + p.theta) * 3.0; }
 
-// Symmetric operator tables with the threads' nodes behind them, one upload
-// each at first use: the FP64 stage and gradient, and the hand-off kernel.
-dg_status sym_tables64(dg_ctx *c)
-{
-    if (c->sym64.ptr) return DG_OK;
-    std::vector<double> tab;
-    std::vector<int> nodes;
-    if (!dg::build_sym64_tables(c->ops, tab, nodes)) return fail(c, DG_EINVAL, "operators without the mirror symmetry");
-    c->nsym64 = tab.size();
-    tab.resize(c->nsym64 + (nodes.size() + 1) / 2);
-    std::memcpy(tab.data() + c->nsym64, nodes.data(), nodes.size() * sizeof(int));
-    DG_CUDA(c, c->sym64.alloc(tab.size()));
-    DG_CUDA(c, cudaMemcpy(c->sym64.ptr, tab.data(), tab.size() * sizeof(double), cudaMemcpyHostToDevice));
-    return DG_OK;
-}
-
-const int *sym_nodes64(const dg_ctx *c) { return reinterpret_cast<const int *>(c->sym64.ptr + c->nsym64); }
-
-dg_status sym_tables32(dg_ctx *c)
-{
-    if (c->sym32.ptr) return DG_OK;
-    std::vector<double> tab;
-    std::vector<int> nodes, slots;
-    std::vector<float> tab32;
-    if (!dg::build_sym64_tables(c->ops, tab, nodes)) return fail(c, DG_EINVAL, "operators without the mirror symmetry");
-    dg::build_sym32_tables(c->ops, tab, nodes, tab32, slots);
-    c->nsym32 = tab32.size();
-    tab32.resize(c->nsym32 + slots.size());
-    std::memcpy(tab32.data() + c->nsym32, slots.data(), slots.size() * sizeof(int));
-    DG_CUDA(c, c->sym32.alloc(tab32.size()));
-    DG_CUDA(c, cudaMemcpy(c->sym32.ptr, tab32.data(), tab32.size() * sizeof(float), cudaMemcpyHostToDevice));
-    return DG_OK;
-}
-
 // What the three-phase FP64 kernel keeps between its phases, for a mesh with
 // connectivity `conn` (host; null: read back).  Over-integration does not run
 // it; without memory for it, or where the stream refused its grid, the mesh
@@ -241,8 +208,6 @@ dg_status phase_arrays(dg_ctx *c, const int4 *conn)
         return DG_OK;
     }
     if (c->flux64.ptr) return DG_OK;
-    dg_status st = sym_tables64(c);
-    if (st != DG_OK) return st;
     std::vector<int4> back, fl;
     if (!conn) {
         back.resize(c->K);
@@ -298,8 +263,6 @@ dg_status two_node_shape(dg_ctx *c)
     DG_CUDA(c, dg::stage_shape_mixed2(c->prm.p, c->K, false, false, !c->no_coop, c->shape2));
     c->fshape_variant = 0;
     if (!c->shape2.handoff) return DG_OK;
-    dg_status st = sym_tables32(c);
-    if (st != DG_OK) return st;
     const cudaError_t e = c->hand32.alloc(static_cast<size_t>(c->K) * (6 * c->ops.Nfp + c->ops.Np));
     if (e != cudaErrorMemoryAllocation) {
         DG_CUDA(c, e);
@@ -316,7 +279,7 @@ dg_status two_node_shape(dg_ctx *c)
 dg::Stage2Args stage2_args(const dg_ctx *c, int s)
 {
     const size_t K = c->hand32.n / (6 * c->ops.Nfp + c->ops.Np), n = K * 3 * c->ops.Nfp;
-    return dg::stage2_args(c->sym32.ptr, reinterpret_cast<const int *>(c->sym32.ptr + c->nsym32), c->hand32.ptr,
+    return dg::stage2_args(c->sym32, c->symn32, c->hand32.ptr,
                            c->hand32.ptr + 2 * n, nullptr, n, s);
 }
 
@@ -377,7 +340,7 @@ dg_status run_stage(dg_ctx *c, int s, double t, double dt, const double vw[2], i
             c->copy_used = true;
         }
         double *const dh = c->flux64.ptr + 2 * ndof(c);
-        const dg::Stage64Args a64{c->sym64.ptr, sym_nodes64(c), c->faces.ptr, c->nfaces, c->flux64.ptr, dh,
+        const dg::Stage64Args a64{c->sym64, c->symn64, c->faces.ptr, c->nfaces, c->flux64.ptr, dh,
                                   dh + static_cast<size_t>(c->K) * 12 * c->ops.Nfp};
         const dg::Phys<double> ph = make_phys<double>(c->prm, vw);
         e = dg::launch_stage_fp64(c->prm.p, c->shape, sp, a64, ph, c->stream);
@@ -499,6 +462,29 @@ dg_status dg_create(const dg_params *params, void *cuda_stream, dg_ctx **out)
         for (const auto *v : {&oi.Vq, &oi.Vqr, &oi.Vqs, &oi.Sr, &oi.Ss}) o64.insert(o64.end(), v->begin(), v->end());
     }
     std::vector<float> o32(o64.begin(), o64.end());
+    // the symmetric tables behind them, 16-byte aligned (FP32: of the hand-off kernel)
+    std::vector<double> tab;
+    std::vector<int> nodes, slots;
+    std::vector<float> tab32;
+    if (!dg::build_sym64_tables(c->ops, p.theta != 0.0, tab, nodes)) {
+        delete c;
+        return DG_EINVAL;
+    }
+    auto behind = [](auto &ops, const auto &table, const std::vector<int> &n) {
+        ops.resize((ops.size() + 3) & ~size_t(3));
+        const size_t at = ops.size();
+        ops.insert(ops.end(), table.begin(), table.end());
+        const size_t an = ops.size();
+        ops.resize(an + (n.size() * sizeof(int) + sizeof(ops[0]) - 1) / sizeof(ops[0]));
+        std::memcpy(ops.data() + an, n.data(), n.size() * sizeof(int));
+        return std::make_pair(at, an);
+    };
+    const auto at64 = behind(o64, tab, nodes);
+    std::pair<size_t, size_t> at32;
+    if (p.precision == DG_PRECISION_MIXED && p.theta == 0.0) {
+        dg::build_sym32_tables(c->ops, tab, nodes, tab32, slots);
+        at32 = behind(o32, tab32, slots);
+    }
     if (c->ops64.alloc(o64.size()) != cudaSuccess || c->ops32.alloc(o32.size()) != cudaSuccess ||
         c->Dr64.alloc(Np * Np) != cudaSuccess || c->Ds64.alloc(Np * Np) != cudaSuccess ||
         c->fmask.alloc(NF) != cudaSuccess || c->flag.alloc(1) != cudaSuccess || c->words.alloc(12) != cudaSuccess ||
@@ -508,6 +494,10 @@ dg_status dg_create(const dg_params *params, void *cuda_stream, dg_ctx **out)
         return DG_ECUDA;
     }
     cudaMemset(c->words.ptr, 0, 12 * sizeof(unsigned));
+    c->sym64 = c->ops64.ptr + at64.first;
+    c->symn64 = reinterpret_cast<const int *>(c->ops64.ptr + at64.second);
+    c->sym32 = c->ops32.ptr + at32.first;
+    c->symn32 = reinterpret_cast<const int *>(c->ops32.ptr + at32.second);
     cudaMemcpy(c->ops64.ptr, o64.data(), o64.size() * sizeof(double), cudaMemcpyHostToDevice);
     cudaMemcpy(c->ops32.ptr, o32.data(), o32.size() * sizeof(float), cudaMemcpyHostToDevice);
     if (dg::stage_tc_supported(p.p)) {
@@ -1060,10 +1050,8 @@ dg_status dg_broken_gradient(dg_ctx *c, double *gx, double *gy, int on_device, i
         oy = c->gtmp.ptr + n;
     }
     if (impl == 0) {
-        dg_status gs = sym_tables64(c);
-        if (gs != DG_OK) return gs;
         if (!c->ggrid) DG_CUDA(c, dg::grad64_grid(c->prm.p, c->K, c->ggrid));
-        const dg::Grad64Args a{c->ggrid, c->cur(), c->geo64.ptr, c->sym64.ptr, sym_nodes64(c), c->Dr64.ptr, c->Ds64.ptr,
+        const dg::Grad64Args a{c->ggrid, c->cur(), c->geo64.ptr, c->sym64, c->symn64, c->Dr64.ptr, c->Ds64.ptr,
                                c->K, ox, oy};
         DG_CUDA(c, dg::launch_grad64(c->prm.p, a, c->stream));
     } else {

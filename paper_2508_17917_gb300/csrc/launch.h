@@ -66,9 +66,10 @@ struct Stage64Args {
 };
 cudaError_t launch_stage_fp64(int p, const LaunchShape &ls, const StageParams &sp, const Stage64Args &a,
                               const Phys<double> &ph, cudaStream_t st);
-// false if the operators are not symmetric under r <-> s
+// false if the operators are not symmetric under r <-> s; theta: with the rows
+// of the theta terms (zero otherwise)
 struct RefOps;
-bool build_sym64_tables(const RefOps &o, std::vector<double> &tab, std::vector<int> &nodes);
+bool build_sym64_tables(const RefOps &o, bool theta, std::vector<double> &tab, std::vector<int> &nodes);
 // broken gradient [K][4][Np] x 2 in FP64, from those tables or the plain rows
 // (both on the device), on `grid` blocks (asked for once per mesh: the query
 // costs as much as the launch)

@@ -138,7 +138,7 @@ cudaError_t grad64_p(const Grad64Args &a, cudaStream_t st)
 }
 
 template <int P>
-bool sym64_tables_p(const RefOps &o, std::vector<double> &tab, std::vector<int> &nodes)
+bool sym64_tables_p(const RefOps &o, bool theta, std::vector<double> &tab, std::vector<int> &nodes)
 {
     using S = Sym64<P>;
     constexpr int Np = S::Np, NF = S::NF, NO = S::NO, NE = S::NE, TPE = S::TPE, NEF = S::NEF;
@@ -195,7 +195,7 @@ bool sym64_tables_p(const RefOps &o, std::vector<double> &tab, std::vector<int> 
         Pm[i] = 0.5 * (Dr[i] + Ds[i]);
         Mm[i] = 0.5 * (Dr[i] - Ds[i]);
     }
-    for (int i = 0; i < Np; ++i)
+    for (int i = 0; theta && i < Np; ++i)
         for (int m = 0; m < NF; ++m)
             for (int j = 0; j < Np; ++j) {
                 Qp[i * NF + m] += 0.5 * (Wr[i * Np + j] + Ws[i * Np + j]) * LIFT[j * NF + m];
@@ -284,15 +284,15 @@ cudaError_t launch_grad64(int p, const Grad64Args &a, cudaStream_t st)
 #undef C_
 }
 
-bool build_sym64_tables(const RefOps &o, std::vector<double> &tab, std::vector<int> &nodes)
+bool build_sym64_tables(const RefOps &o, bool theta, std::vector<double> &tab, std::vector<int> &nodes)
 {
     switch (o.p) {
-    case 1: return sym64_tables_p<1>(o, tab, nodes);
-    case 2: return sym64_tables_p<2>(o, tab, nodes);
-    case 3: return sym64_tables_p<3>(o, tab, nodes);
-    case 4: return sym64_tables_p<4>(o, tab, nodes);
-    case 5: return sym64_tables_p<5>(o, tab, nodes);
-    case 6: return sym64_tables_p<6>(o, tab, nodes);
+    case 1: return sym64_tables_p<1>(o, theta, tab, nodes);
+    case 2: return sym64_tables_p<2>(o, theta, tab, nodes);
+    case 3: return sym64_tables_p<3>(o, theta, tab, nodes);
+    case 4: return sym64_tables_p<4>(o, theta, tab, nodes);
+    case 5: return sym64_tables_p<5>(o, theta, tab, nodes);
+    case 6: return sym64_tables_p<6>(o, theta, tab, nodes);
     default: return false;
     }
 }
