@@ -43,7 +43,7 @@ constexpr float kDtSpread = 100.0f;
 // the size of the terms of one trace's norm, Q / rho
 __device__ __forceinline__ float norm_terms(float ir, float vsq, float e, float gPr)
 {
-    return ir * fmaf(gPr, e + vsq, (4.0f / 3.0f) * vsq);
+    return ir * fmaf(gPr, fabsf(e) + vsq, (4.0f / 3.0f) * vsq);
 }
 
 // words: [0] largest screened Lambda (FP32 bits), [1] finished blocks,
@@ -79,39 +79,37 @@ dt_screen_kernel(const double *U, const double *geo, const int4 *conn, const int
             Ed = U[(k * 4 + c) * Np + vm];
             u[c] = cvt_d2f(Ed);
         }
-        float rmin = u[0], rmax = u[0];
+        float rmin = u[0];
         if (bt == BCT_INTERIOR) {
             const long long nb = (ff == 0) ? cn.x : (ff == 1 ? cn.y : cn.z);
             const int vp = fmask[f2 * Nfp + (Nfp - 1 - fi)];
 #pragma unroll
             for (int c = 0; c < 4; ++c) w[c] = cvt_d2f(U[(nb * 4 + c) * Np + vp]);
-            rmin = fminf(rmin, w[0]);
-            rmax = fmaxf(rmax, w[0]);
-        } else if (bt == BCT_FARFIELD) {
-            rmin = fminf(rmin, ph.Uinf[0]);
+        } else {
+#pragma unroll
+            for (int c = 0; c < 4; ++c) w[c] = ph.Uinf[c];
         }
+        if (bt != BCT_WALL) rmin = fminf(rmin, w[0]);
         const float pw = (bt == BCT_WALL) ? pressure<float>(u, Ed, gm1d) : 0.f;
         const float ir = 1.0f / u[0];
         const float nrm = trace_norms_max(u, ir, pw, bt, w, n1, n2, ph);
+        // the guards; what is not finite reaches `own` or `other`, and the
+        // comparisons are written so that a NaN fails them
         const float msq = u[1] * u[1] + u[2] * u[2];
-        float terms = norm_terms(ir, msq * ir * ir, u[3] * ir, ph.gPr);
-        bool wall_ok = true;
+        const float own = norm_terms(ir, msq * ir * ir, u[3] * ir, ph.gPr);
+        float other;
+        bool ok = rmin > 1e-12f && fmaxf(u[0], w[0]) < 1e12f && nrm < 1e15f && (nrm > 1e-15f || ph.mu == 0.f);
         if (bt == BCT_WALL) {
             const float wsq = ph.vw1 * ph.vw1 + ph.vw2 * ph.vw2;
-            const float tw = norm_terms(ir, wsq, fmaf(0.5f, wsq, pw / ph.gm1 * ir), ph.gPr);
-            wall_ok = pw > 1e-2f * (msq * ir) && ph.mu * tw <= 4.0f * nrm;
+            other = norm_terms(ir, wsq, fmaf(0.5f, wsq, pw / ph.gm1 * ir), ph.gPr);
+            ok = ok && pw > 1e-2f * (msq * ir) && ph.mu * other <= 4.0f * nrm;
         } else {
-            const float r = (bt == BCT_INTERIOR) ? w[0] : ph.Uinf[0], m1 = (bt == BCT_INTERIOR) ? w[1] : ph.Uinf[1];
-            const float m2 = (bt == BCT_INTERIOR) ? w[2] : ph.Uinf[2], E = (bt == BCT_INTERIOR) ? w[3] : ph.Uinf[3];
-            const float iw = 1.0f / r;
-            terms = fmaxf(terms, norm_terms(iw, (m1 * m1 + m2 * m2) * iw * iw, E * iw, ph.gPr));
+            const float iw = 1.0f / w[0];
+            other = norm_terms(iw, (w[1] * w[1] + w[2] * w[2]) * iw * iw, w[3] * iw, ph.gPr);
         }
+        ok = ok && ph.mu * (own + other) <= kDtSpread * nrm;
         sNorm[fm + fe * NF] = nrm;
         sRmin[fm + fe * NF] = rmin;
-        // comparisons written so that a NaN fails them
-        const float all = (u[0] + u[1]) + (u[2] + u[3]) + ((bt == BCT_INTERIOR) ? (w[0] + w[1]) + (w[2] + w[3]) : 0.f);
-        const bool ok = rmin > 1e-12f && rmax < 1e12f && nrm < 1e15f && (nrm > 1e-15f || ph.mu == 0.f) &&
-                        all - all == 0.f && ph.mu * terms <= kDtSpread * nrm && wall_ok;
         if (!ok) sMark[fe] = 1;
     }
     const int ve = tid / Np, vi = tid - (tid / Np) * Np;
