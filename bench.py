@@ -877,7 +877,7 @@ def run_profile(args):
         return
     prec, n, theta, var, p = {"mixed512": ("mixed", 512, 0.0, 0, P), "mixed128": ("mixed", 128, 0.0, 0, P),
                               "fp64_128": ("fp64", 128, 0.0, 0, P), "sip128": ("mixed", 128, 1.0, 0, P),
-                              "tc512": ("mixed", 512, 0.0, 3, P), "tcsip512": ("mixed", 512, 1.0, 3, P),
+                              "handoff256": ("mixed", 256, 0.0, 2, P), "tc512": ("mixed", 512, 0.0, 3, P), "tcsip512": ("mixed", 512, 1.0, 3, P),
                               "tc6_375": ("mixed", 375, 0.0, 3, 6)}[args.profile]
     torch.cuda.set_device(0)
     mesh = vortex_problem(n)
@@ -916,7 +916,7 @@ def main():
                     help="ncu raw-page CSV of one stage launch: write its DRAM bytes per DOF-stage")
     ap.add_argument("--record-k", type=int, default=2 * 512 * 512,
                     help="elements of the captured launch (--record-traffic)")
-    ap.add_argument("--profile", choices=["mixed512", "mixed128", "fp64_128", "sip128", "tc512", "tcsip512", "tc6_375", "mlp4096",
+    ap.add_argument("--profile", choices=["mixed512", "mixed128", "fp64_128", "sip128", "handoff256", "tc512", "tcsip512", "tc6_375", "mlp4096",
                              "batch64", "grad512"], default=None)
     args = ap.parse_args()
     if args.record_traffic:

@@ -15,7 +15,7 @@
 //   F  per face, once for both sides: Roe flux, penalty and viscous flux from
 //      the two traces and the stored fluxes; Fscale (F.n - H) for each side;
 //   U  per element: divergence, lift, stage update.
-// The phases' arrays (96 bytes per node and 32 per face node) cost memory
+// The phases' arrays (64 bytes per node and 32 per face node) cost memory
 // traffic, of which this path has none to spare: 0.1 of the time.
 //
 // Contractions by symmetry: the nodes are symmetric under r <-> s, which
