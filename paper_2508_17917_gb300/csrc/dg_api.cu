@@ -49,6 +49,7 @@ struct dg_ctx {
     const float *sym32 = nullptr;
     const int *symn64 = nullptr, *symn32 = nullptr;
     bool no_coop = false;     // the stream refused a grid of theirs as a cooperative launch
+    bool captured = false;    // a launch with their arrays is in a caller's graph: they stay until the next mesh
     dg::DevBuf<float4> hand32;                        // face records [2][K][3 Nfp], divergence [K][Np]
     dg::DevBuf<int4> faces;
     int nfaces = 0;
@@ -99,12 +100,21 @@ struct dg_ctx {
     cudaEvent_t tune_ev[9] = {};     // mixed: marks of the stage-shape timing
     void drop_phases()
     {
+        if (captured) return;
         flux64.release();
         faces.release();
     }
     void drop_handoff()
     {
-        hand32.release();
+        if (!captured) hand32.release();
+    }
+    // before a launch that uses them
+    void note_capture()
+    {
+        cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+        if (captured) return;
+        if (cudaStreamIsCapturing(stream, &st) != cudaSuccess) cudaGetLastError();      // the legacy stream, while another captures
+        captured = st != cudaStreamCaptureStatusNone;
     }
     ~dg_ctx()
     {
@@ -231,7 +241,7 @@ dg_status phase_arrays(dg_ctx *c, const int4 *conn)
 
 cudaError_t shape_fp64(dg_ctx *c)
 {
-    return dg::stage_shape_fp64(c->prm.p, c->K, c->prm.theta != 0.0, c->shape, c->overint, c->flux64.ptr != nullptr);
+    return dg::stage_shape_fp64(c->prm.p, c->K, c->prm.theta != 0.0, c->shape, c->overint, c->flux64.ptr && !c->no_coop);
 }
 
 // An array that a call needs.  Where there is no memory for it, the arrays that
@@ -240,7 +250,7 @@ template <typename T>
 cudaError_t alloc_needed(dg_ctx *c, dg::DevBuf<T> &b, size_t n)
 {
     cudaError_t e = b.alloc(n);
-    if (e != cudaErrorMemoryAllocation || !(c->flux64.ptr || c->hand32.ptr)) return e;
+    if (e != cudaErrorMemoryAllocation || !(c->flux64.ptr || c->hand32.ptr) || c->captured) return e;
     cudaGetLastError();
     if (c->flux64.ptr) {
         c->drop_phases();                  // cudaFree waits for the kernels that use them
@@ -333,6 +343,7 @@ dg_status run_stage(dg_ctx *c, int s, double t, double dt, const double vw[2], i
         sp.geo = c->geo64.ptr;
         sp.ops = c->ops64.ptr;
         if (c->shape.phases) {
+            c->note_capture();
             // grid barriers between its phases, reported through the barrier flag
             sp.bar = c->bar();
             sp.bar_err = c->bar_err();
@@ -363,6 +374,7 @@ dg_status run_stage(dg_ctx *c, int s, double t, double dt, const double vw[2], i
         }
         else if (c->shape.variant == 2) {
             if (c->shape.handoff) {
+                c->note_capture();
                 sp.bar = c->bar();
                 sp.bar_err = c->bar_err();
                 sp.bar_limit = c->bar_limit;
@@ -623,6 +635,7 @@ dg_status dg_set_mesh(dg_ctx *c, int64_t Nv, const double *vx, const double *vy,
     std::vector<int2> &walls = ma.walls;
     std::vector<double> &wxy = ma.wxy;
     // --- device buffers
+    c->captured = false;             // graphs of the old mesh go with it
     c->drop_phases();
     c->drop_handoff();
     c->K = K;
@@ -931,10 +944,11 @@ static dg_status run_fused_step(dg_ctx *c, double dt, const double vw[2])
     DG_CUDA(c, cudaMemsetAsync(c->bar(), 0, 2 * sizeof(unsigned), c->stream));
     if (c->fshape.variant == 3)
         DG_CUDA(c, dg::launch_stage_tc(c->prm.p, false, true, c->fshape, sp, make_phys<float>(c->prm, vw), c->stream));
-    else if (c->fshape.variant == 2)
+    else if (c->fshape.variant == 2) {
+        if (c->fshape.handoff) c->note_capture();
         DG_CUDA(c, dg::launch_stage_mixed2(c->prm.p, false, true, c->fshape, sp, stage2_args(c, 0),
                                            make_phys<float>(c->prm, vw), c->stream));
-    else
+    } else
         DG_CUDA(c, dg::launch_stage_mixed_fused(c->prm.p, false, c->fshape, sp, make_phys<float>(c->prm, vw), c->stream));
     c->launches += 1;
     c->cur_is_a = !c->cur_is_a;   // five swaps

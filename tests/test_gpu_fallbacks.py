@@ -246,3 +246,40 @@ def test_batch_without_memory_between_the_stages(dg, take_all_but):
         assert b.variant(0) == 1
         got.append(b.get_state(0))
     assert np.array_equal(got[0], got[1])
+
+
+@pytest.mark.parametrize("precision,fused", [("fp64", False), ("mixed", False), ("mixed", True)])
+def test_arrays_in_a_callers_graph_stay(dg, precision, fused):
+    """Steps captured into a graph of the caller's hold the addresses of the
+    arrays between phases or stages: another shape, over-integration or the
+    tuner does not give them back, and the graph replays the same steps."""
+    import torch
+    st = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(st):
+        s = dg.Solver(dg_inputs.periodic_square(200), 4, precision, stream=st.cuda_stream, mu=1e-3)
+        if precision == "mixed":
+            s.set_variant(2)
+            s.set_fused(fused)
+        U = vortex(s)
+        s.set_state(U)
+        s.steps(0.0, 1e-5, 2)
+        want = s.get_state()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=st):
+            s.steps(0.0, 1e-5, 2)
+        held = free_bytes()
+        if precision == "fp64":
+            s.set_overint(True)
+        else:
+            s.set_fused(False)
+            s.set_variant(3)
+            s.set_variant(0)
+            s.set_state(U)
+            s.steps(0.0, 1e-5, 2)
+        assert held - free_bytes() >= -MB
+        s.set_state(U)
+        g.replay()
+        st.synchronize()
+        assert np.array_equal(s.get_state(), want)
+        del g
